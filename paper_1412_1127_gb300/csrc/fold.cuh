@@ -193,12 +193,38 @@ __device__ __forceinline__ void for_each_elem(const uint4 *v, F &&f) {
     }
 }
 
-// Neumaier step: (s, c) += x.
+// Larger / smaller of two or three floats by the hardware's max/min, whose
+// order puts -0 below +0 (the order of the keys above).
+__device__ __forceinline__ float fmax2(float a, float b) {
+    float r;
+    asm("max.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float fmin2(float a, float b) {
+    float r;
+    asm("min.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float fmax3(float a, float b, float c) {
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+__device__ __forceinline__ float fmin3(float a, float b, float c) {
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+// Compensated step: (s, c) += x.  The rounding error of s + x comes from
+// Knuth's TwoSum: the same exact error as Neumaier's ordered form, in six
+// additions for the FMA pipe instead of three plus a compare and two selects
+// for the half-rate ALU pipe, which is what bounded compensated sums.
 __device__ __forceinline__ void neumaier(float &s, float &c, float x) {
-    float t = __fadd_rn(s, x);
-    float big = fabsf(s) >= fabsf(x) ? s : x;
-    float small = fabsf(s) >= fabsf(x) ? x : s;
-    c = __fadd_rn(c, __fadd_rn(__fsub_rn(big, t), small));
+    const float t = __fadd_rn(s, x);
+    const float xp = __fsub_rn(t, s);
+    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, xp)), __fsub_rn(x, xp));
+    c = __fadd_rn(c, e);
     s = t;
 }
 
@@ -264,6 +290,66 @@ __device__ __forceinline__ double chunk_sum_f64(const uint4 *v) {
         // S counts units of 2^(emax - 1075 - 6); that power of two is normal here
         const double scale = u2d((uint64_t)(emax - 1081 + 1023) << 52);
         return __dmul_rn(__ll2double_rn((long long)S), scale);
+    }
+}
+
+// a += the sum of the 4*NV floats of a chunk, in double.  Converting and adding
+// each float costs two operations of the FP64 pipe (about two a clock per SM,
+// which bounded a float array summed into a double at 0.72 TB/s), so the chunk
+// is summed by extraction (Rump, Ogita and Oishi's error-free split against a
+// power-of-two anchor): with 2^E <= max |x| < 2^(E+1), adding and subtracting
+// 1.5 * 2^(E+2) splits x exactly into a multiple of 2^(E-21) and a remainder,
+// whose own split against 2^-23 of that anchor leaves a multiple of 2^(E-44)
+// and a second remainder.  The multiples are added as integers (the anchored
+// values' bits, modulo 2^32), the second remainders as floats (an error below
+// 2^(E-63)), and the total, in units of 2^(E-54), meets the double accumulator
+// in one fused multiply-add: two FP64-pipe operations a chunk, and at most
+// 2^(E-54) lost before the accumulator's own rounding.  A chunk whose largest
+// magnitude is not finite, or outside 2^-70 .. 2^120 (zero included), is added
+// as doubles.
+template <int NV>
+__device__ __forceinline__ double add_chunk_wide(double a, const uint4 *v) {
+    constexpr int E = 4 * NV;
+    if constexpr (NV < 2) {
+#pragma unroll
+        for (int j = 0; j < E; ++j) a = __dadd_rn(a, (double)__uint_as_float(word32(v[j >> 2], j & 3)));
+        return a;
+    } else {
+        uint32_t mb = 0;  // largest magnitude, as bits: a NaN's exceed infinity's
+#pragma unroll
+        for (int j = 0; j < E; ++j) mb = max(mb, word32(v[j >> 2], j & 3) & 0x7fffffffu);
+        const int e = (int)(mb >> 23) - 127;
+        if (e < -70 || e > 120) {
+#pragma unroll
+            for (int j = 0; j < E; ++j) {
+                double d;  // volatile: the conversions (FP64 pipe) stay inside this branch
+                asm volatile("cvt.f64.f32 %0, %1;" : "=d"(d) : "f"(__uint_as_float(word32(v[j >> 2], j & 3))));
+                a = __dadd_rn(a, d);
+            }
+            return a;
+        }
+        const uint32_t b1 = ((uint32_t)(e + 2 + 127) << 23) | 0x400000u;   // 1.5 * 2^(e + 2)
+        const uint32_t b2 = ((uint32_t)(e - 21 + 127) << 23) | 0x400000u;  // 1.5 * 2^(e - 21)
+        const float s1 = __uint_as_float(b1), s2 = __uint_as_float(b2);
+        uint32_t i1 = 0, i2 = 0;
+        float r0 = 0.f, r1 = 0.f;
+#pragma unroll
+        for (int j = 0; j < E; ++j) {
+            const float x = __uint_as_float(word32(v[j >> 2], j & 3));
+            const float t = __fadd_rn(x, s1);
+            i1 += __float_as_uint(t);
+            const float r = __fsub_rn(x, __fsub_rn(t, s1));
+            const float u = __fadd_rn(r, s2);
+            i2 += __float_as_uint(u);
+            const float q = __fsub_rn(r, __fsub_rn(u, s2));
+            if (j & 1) r1 = __fadd_rn(r1, q);
+            else r0 = __fadd_rn(r0, q);
+        }
+        const int32_t n1 = (int32_t)(i1 - (uint32_t)E * b1), n2 = (int32_t)(i2 - (uint32_t)E * b2);
+        // units of 2^(e - 54): |n1| < 2^28 of 2^33 each, |n2| < 2^28 of 2^10 each
+        const float rs = __fmul_rn(__fadd_rn(r0, r1), __uint_as_float((uint32_t)(54 - e + 127) << 23));
+        const long long S = ((long long)n1 << 33) + ((long long)n2 << 10) + (long long)__float2int_rn(rs);
+        return __fma_rn(__ll2double_rn(S), u2d((uint64_t)(uint32_t)(e - 54 + 1023) << 52), a);
     }
 }
 
@@ -360,9 +446,7 @@ __device__ __forceinline__ void fold_vec(int w, Acc &A, const uint4 *v) {
             }
         } break;
         case W_ADDF_WIDE: {
-            double a = u2d(A.a);
-            for_each_elem<T, NV>(v, [&](T x) { a = __dadd_rn(a, (double)x); });
-            A.a = d2u(a);
+            if constexpr (F32) A.a = d2u(add_chunk_wide<NV>(u2d(A.a), v));
         } break;
         case W_MULF: {
             T a = F32 ? (T)u2f((uint32_t)A.a) : (T)u2d(A.a);
@@ -375,16 +459,14 @@ __device__ __forceinline__ void fold_vec(int w, Acc &A, const uint4 *v) {
             A.a = d2u(a);
         } break;
         case W_MAXF: {
-            if constexpr (F32) {  // four independent key chains, as for the sum
-                int32_t a0 = (int32_t)(uint32_t)A.a, a1 = a0, a2 = a0, a3 = a0;
+            if constexpr (F32) {  // two independent chains on the hardware's max, two elements a step
+                float a0 = u2f((uint32_t)fkey32((uint32_t)A.a)), a1 = a0;
 #pragma unroll
                 for (int i = 0; i < NV; ++i) {
-                    a0 = max(a0, fkey32(v[i].x));
-                    a1 = max(a1, fkey32(v[i].y));
-                    a2 = max(a2, fkey32(v[i].z));
-                    a3 = max(a3, fkey32(v[i].w));
+                    a0 = fmax3(a0, __uint_as_float(v[i].x), __uint_as_float(v[i].y));
+                    a1 = fmax3(a1, __uint_as_float(v[i].z), __uint_as_float(v[i].w));
                 }
-                A.a = (uint32_t)max(max(a0, a1), max(a2, a3));
+                A.a = (uint32_t)fkey32(f2u(fmax2(a0, a1)));
             } else {
                 int64_t a = (int64_t)A.a;
                 for_each_elem<T, NV>(v, [&](T x) {
@@ -395,16 +477,14 @@ __device__ __forceinline__ void fold_vec(int w, Acc &A, const uint4 *v) {
             }
         } break;
         case W_MINF: {
-            if constexpr (F32) {
-                int32_t a0 = (int32_t)(uint32_t)A.a, a1 = a0, a2 = a0, a3 = a0;
+            if constexpr (F32) {  // two independent chains on the hardware's min, two elements a step
+                float a0 = u2f((uint32_t)fkey32((uint32_t)A.a)), a1 = a0;
 #pragma unroll
                 for (int i = 0; i < NV; ++i) {
-                    a0 = min(a0, fkey32(v[i].x));
-                    a1 = min(a1, fkey32(v[i].y));
-                    a2 = min(a2, fkey32(v[i].z));
-                    a3 = min(a3, fkey32(v[i].w));
+                    a0 = fmin3(a0, __uint_as_float(v[i].x), __uint_as_float(v[i].y));
+                    a1 = fmin3(a1, __uint_as_float(v[i].z), __uint_as_float(v[i].w));
                 }
-                A.a = (uint32_t)min(min(a0, a1), min(a2, a3));
+                A.a = (uint32_t)fkey32(f2u(fmin2(a0, a1)));
             } else {
                 int64_t a = (int64_t)A.a;
                 for_each_elem<T, NV>(v, [&](T x) {
@@ -417,6 +497,26 @@ __device__ __forceinline__ void fold_vec(int w, Acc &A, const uint4 *v) {
         default: break;
         }
     }
+}
+
+// Fold the first `cnt` of NV vectors (a stretch's last, partial round).  A
+// float sum in double takes them as one chunk, the missing ones as -0: vector
+// by vector it would pay the FP64 pipe per element.
+template <typename T, int NV>
+__device__ __forceinline__ void fold_prefix(int w, Acc &A, const uint4 *v, int cnt) {
+    if constexpr (std::is_same<T, float>::value && NV > 1) {
+        if (w == W_ADDF_WIDE) {
+            uint4 f[NV];
+#pragma unroll
+            for (int u = 0; u < NV; ++u)
+                f[u] = u < cnt ? v[u] : make_uint4(0x80000000u, 0x80000000u, 0x80000000u, 0x80000000u);
+            if (cnt > 0) fold_vec<T, NV>(w, A, f);
+            return;
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < NV; ++u)
+        if (u < cnt) fold_vec<T, 1>(w, A, v + u);
 }
 
 // Fold one scalar element (unaligned heads and ragged tails).
@@ -531,18 +631,34 @@ __host__ __device__ __forceinline__ void merge(int w, bool elem64, Acc &A, const
     }
 }
 
-__device__ __forceinline__ Acc shfl_xor_acc(const Acc &A, int m) {
+// The other half of a butterfly step.  With the working code fixed at compile
+// time (FIXED) a 32-bit working value moves in one shuffle, a 64-bit one in two,
+// and only compensated sums carry their second term; a code read at run time
+// moves all three words (choosing would cost a branch a step).
+template <bool FIXED>
+__device__ __forceinline__ Acc shfl_xor_acc(int w, bool elem64, const Acc &A, int m) {
     Acc B;
-    B.a = __shfl_xor_sync(0xffffffffu, (unsigned long long)A.a, m);
-    B.c = __shfl_xor_sync(0xffffffffu, A.c, m);
+    if (FIXED) {
+        const bool wide = elem64 || w == W_ADD64 || w == W_MUL64 || w == W_ADDF_WIDE || w == W_MULF_WIDE;
+        const uint32_t lo = __shfl_xor_sync(0xffffffffu, (uint32_t)A.a, m);
+        const uint32_t hi = wide ? __shfl_xor_sync(0xffffffffu, (uint32_t)(A.a >> 32), m) : 0u;
+        B.a = ((uint64_t)hi << 32) | lo;
+        B.c = w == W_ADDF_COMP ? __shfl_xor_sync(0xffffffffu, A.c, m) : 0.f;
+    } else {
+        B.a = __shfl_xor_sync(0xffffffffu, (unsigned long long)A.a, m);
+        B.c = __shfl_xor_sync(0xffffffffu, A.c, m);
+    }
     return B;
 }
 
-// Butterfly merge across the 32 lanes of a warp (every lane ends with the total).
-__device__ __forceinline__ void warp_merge(int w, bool elem64, Acc &A) {
+// Butterfly merge across groups of `lanes` (a power of two) neighbouring lanes
+// of a warp: every lane ends with its group's total.
+template <bool FIXED>
+__device__ __forceinline__ void group_merge(int w, bool elem64, Acc &A, int lanes) {
 #pragma unroll
     for (int m = 16; m >= 1; m >>= 1) {
-        Acc B = shfl_xor_acc(A, m);
+        if (m >= lanes) continue;
+        Acc B = shfl_xor_acc<FIXED>(w, elem64, A, m);
         // combine in a lane-independent order so all lanes hold identical bits
         Acc lo = (threadIdx.x & m) ? B : A;
         Acc hi = (threadIdx.x & m) ? A : B;
@@ -551,15 +667,21 @@ __device__ __forceinline__ void warp_merge(int w, bool elem64, Acc &A) {
     }
 }
 
+template <bool FIXED = false>
+__device__ __forceinline__ void warp_merge(int w, bool elem64, Acc &A) {
+    group_merge<FIXED>(w, elem64, A, 32);
+}
+
 // Merge one accumulator per clause across a CTA of NT threads (all threads
 // call it); thread 0 ends with the totals.  `sh` is NC x NT/32 shared slots.
-template <int NC, int NT>
+// FIXED: the codes are compile-time constants of the kernel.
+template <int NC, int NT, bool FIXED = false>
 __device__ __forceinline__ void cta_merge(const int (&w)[NC], const uint64_t (&ident)[NC], bool e64,
                                           Acc (&A)[NC], Acc (*sh)[NT / 32]) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-        warp_merge(w[c], e64, A[c]);
+        warp_merge<FIXED>(w[c], e64, A[c]);
         if (lane == 0) sh[c][warp] = A[c];
     }
     __syncthreads();
@@ -569,7 +691,7 @@ __device__ __forceinline__ void cta_merge(const int (&w)[NC], const uint64_t (&i
             Acc B;
             if (lane < NT / 32) B = sh[c][lane];
             else { B.a = ident[c]; B.c = 0.f; }
-            warp_merge(w[c], e64, B);
+            warp_merge<FIXED>(w[c], e64, B);
             A[c] = B;
         }
     }
