@@ -1,0 +1,161 @@
+// group.cuh -- a short stretch of elements (at most GROUP_BYTES) folded by a group
+// of 1 to 32 neighbouring lanes: short rows and short segments.
+#pragma once
+
+#include <math.h>
+
+#include "common.cuh"
+#include "fold.cuh"
+
+namespace accr {
+
+constexpr int GV = 8;                          // vectors per lane at most
+constexpr int64_t GROUP_BYTES = GV * 32 * 16;  // 4 KiB
+
+// A running fold of one clause of a fixed code in registers: whole vectors and
+// single elements in, an accumulator out.  The primary form keeps the
+// accumulator itself; the float sums and extremes keep their own chains between
+// vectors, which saves the accumulator's packing and the chains' merge per vector.
+template <typename T, int W>
+struct GroupFold {
+    Acc A;
+    __device__ __forceinline__ void init(uint64_t ident) { A.a = ident, A.c = 0.f; }
+    __device__ __forceinline__ void vec(const uint4 &v) { fold_vec<T, 1>(W, A, &v); }
+    __device__ __forceinline__ void one(T x) { fold_one<T>(W, A, x); }
+    __device__ __forceinline__ Acc get() const { return A; }
+};
+template <>
+struct GroupFold<float, W_ADDF> {
+    float p0, p1, p2, p3;
+    __device__ __forceinline__ void init(uint64_t) { p0 = p1 = p2 = p3 = -0.f; }
+    __device__ __forceinline__ void vec(const uint4 &v) {
+        p0 = __fadd_rn(p0, __uint_as_float(v.x));
+        p1 = __fadd_rn(p1, __uint_as_float(v.y));
+        p2 = __fadd_rn(p2, __uint_as_float(v.z));
+        p3 = __fadd_rn(p3, __uint_as_float(v.w));
+    }
+    __device__ __forceinline__ void one(float x) { p0 = __fadd_rn(p0, x); }
+    __device__ __forceinline__ Acc get() const {
+        Acc A;
+        A.a = f2u(__fadd_rn(__fadd_rn(p0, p1), __fadd_rn(p2, p3)));
+        A.c = 0.f;
+        return A;
+    }
+};
+template <bool MAX>
+struct GroupExtreme {
+    float m;
+    __device__ __forceinline__ void init(uint64_t) { m = MAX ? -INFINITY : INFINITY; }
+    __device__ __forceinline__ void vec(const uint4 &v) {
+        if (MAX) m = fmax3(fmax3(m, __uint_as_float(v.x), __uint_as_float(v.y)), __uint_as_float(v.z), __uint_as_float(v.w));
+        else m = fmin3(fmin3(m, __uint_as_float(v.x), __uint_as_float(v.y)), __uint_as_float(v.z), __uint_as_float(v.w));
+    }
+    __device__ __forceinline__ void one(float x) { m = MAX ? fmax2(m, x) : fmin2(m, x); }
+    __device__ __forceinline__ Acc get() const {
+        Acc A;
+        A.a = (uint32_t)fkey32(f2u(m));
+        A.c = 0.f;
+        return A;
+    }
+};
+template <>
+struct GroupFold<float, W_MAXF> : GroupExtreme<true> {};
+template <>
+struct GroupFold<float, W_MINF> : GroupExtreme<false> {};
+
+// Folds the loaded vectors of one lane.  A pair kernel folds the vectors the
+// lane holds one by one; a generic one fills the others with the clause's
+// neutral element, so that its operator switch runs once for all of them.
+template <typename T, int NV>
+__device__ __forceinline__ void fold_filled(int w, Acc &A, const uint4 (&b)[GV], const bool (&ok)[GV], uint64_t neutral) {
+    const uint32_t lo = (uint32_t)neutral, hi = sizeof(T) == 8 ? (uint32_t)(neutral >> 32) : lo;
+    uint4 f[NV];
+#pragma unroll
+    for (int u = 0; u < NV; ++u) f[u] = ok[u] ? b[u] : make_uint4(lo, hi, lo, hi);
+    fold_vec<T, NV>(w, A, f);
+}
+
+// One stretch of `len` elements at `in`, folded by a group of L lanes (this lane is
+// number l of it) into A and merged across the group.  `rounds`: no lane of the
+// warp has more than this many vectors (at most GV).  Lanes that are not live
+// take part in the merge only.  Every load is in flight before any is folded.
+template <typename T, int NC, int W0, int W1>
+__device__ __forceinline__ void group_fold(const T *in, int len, bool live, int l, int L, int rounds,
+                                           const ClauseDev *cl, const uint64_t *neutral, const int (&w)[NC],
+                                           Acc (&A)[NC]) {
+    constexpr bool E64 = sizeof(T) == 8, PAIR = W0 >= 0;
+    constexpr int EPV = 16 / (int)sizeof(T);
+    const int mis = (int)(((16 - ((uintptr_t)in & 15)) & 15) / sizeof(T));
+    const int end = live ? len : 0;
+    const int head = mis < end ? mis : end;
+    const uint4 *vr = (const uint4 *)(in + head) + l;
+    const int nvec = (end - head) / EPV;
+    const int tail0 = head + nvec * EPV;
+    uint4 b[GV];
+    bool ok[GV];
+    T h = T(), t = T();  // this lane's first head and tail element
+#pragma unroll
+    for (int u = 0; u < GV; ++u) {
+        ok[u] = u < rounds && u * L + l < nvec;
+        if (ok[u]) b[u] = __ldg(vr + u * L);
+    }
+    if (l < head) h = __ldg(in + l);
+    if (tail0 + l < end) t = __ldg(in + tail0 + l);
+    if constexpr (PAIR) {
+        GroupFold<T, W0> F0;
+        GroupFold<T, W1> F1;
+        F0.init(cl[0].ident);
+        F1.init(cl[1].ident);
+#pragma unroll
+        for (int u = 0; u < GV; ++u) {
+            if (ok[u]) {
+                F0.vec(b[u]);
+                F1.vec(b[u]);
+            }
+        }
+        if (l < head) F0.one(h), F1.one(h);
+        if (tail0 + l < end) F0.one(t), F1.one(t);
+        if (L < EPV) {  // fewer lanes than a head or tail may have elements
+            for (int j = L + l; j < head; j += L) F0.one(__ldg(in + j)), F1.one(__ldg(in + j));
+            for (int j = tail0 + L + l; j < end; j += L) F0.one(__ldg(in + j)), F1.one(__ldg(in + j));
+        }
+        A[0] = F0.get();
+        A[1] = F1.get();
+    } else {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            A[c].a = cl[c].ident;
+            A[c].c = 0.f;
+            if (rounds > GV / 2) fold_filled<T, GV>(w[c], A[c], b, ok, neutral[c]);
+            else if (rounds > 0) fold_filled<T, GV / 2>(w[c], A[c], b, ok, neutral[c]);
+            for (int j = l; j < head; j += L) fold_one<T>(w[c], A[c], j == l ? h : __ldg(in + j));
+            for (int j = tail0 + l; j < end; j += L) fold_one<T>(w[c], A[c], j == tail0 + l ? t : __ldg(in + j));
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) group_merge<PAIR>(w[c], E64, A[c], L);
+}
+
+// The element that leaves a fold under working code w as it is (element bits).
+template <typename T>
+inline uint64_t neutral_element(int w) {
+    constexpr bool e64 = sizeof(T) == 8;
+    switch (w) {
+    case W_MUL32:
+    case W_MUL64:
+    case W_LAND: return 1;
+    case W_MAXI: return e64 ? (uint64_t)INT64_MIN : (uint64_t)(uint32_t)INT32_MIN;
+    case W_MINI: return e64 ? (uint64_t)INT64_MAX : (uint64_t)(uint32_t)INT32_MAX;
+    case W_AND: return ~0ull;
+    case W_ADDF:
+    case W_ADDF_COMP:
+    case W_ADDF_WIDE: return e64 ? d2u(-0.0) : f2u(-0.0f);
+    case W_MULF:
+    case W_MULF_WIDE: return e64 ? d2u(1.0) : f2u(1.0f);
+    case W_MAXF: return e64 ? d2u(-INFINITY) : f2u(-INFINITY);
+    case W_MINF: return e64 ? d2u(INFINITY) : f2u(INFINITY);
+    default: return 0;  // sums, |, ^, ||
+    }
+}
+
+}  // namespace accr

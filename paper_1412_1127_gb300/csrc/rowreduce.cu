@@ -2,15 +2,22 @@
 // one reduction variable per row of a row-major matrix (the two-level loop
 // shape of Listing 1a with an inner reduction; IPMACC Sec. 1.3, Stage 3.4).
 //
-// Mapping: gang -> CTA, worker -> warp, vector -> lane.  A warp folds one
-// stretch of a row at a time: lanes stream it in 16-byte vectors (RU2 in
-// flight per lane) and merge through shuffles.  Stretches whose start is not
-// 16-byte aligned (ld not a multiple of the vector) fold their head and tail
-// element by element.  Two forms, chosen by the row's length alone, so a
-// row's result never depends on how many rows the matrix has:
+// Mapping: gang -> CTA, worker -> warp, vector -> lane.  Lanes stream a stretch
+// of a row in 16-byte vectors and merge through shuffles; a stretch whose start
+// is not 16-byte aligned (ld not a multiple of the vector) folds its head and
+// tail element by element.  Four forms, chosen by the row's length alone, so
+// a row's result never depends on how many rows the matrix has:
 //
-//   * rows shorter than SPLIT_ROW_BYTES: the stretch is the whole row and
-//     lane 0 writes the row's variable; no cross-warp merge at all.
+//   * rows of at most GROUP_BYTES: a group of 1 to 32 neighbouring lanes
+//     per row, about four vectors a lane, so a warp folds up to 32 rows at
+//     once and every load of a row is in flight before any is folded.
+//   * rows of at most WARP_ROW_BYTES: a warp per row, RU2 vectors in flight a
+//     lane; lane 0 writes the row's variable, no cross-warp merge at all.
+//   * rows shorter than SPLIT_ROW_BYTES: SEG_BYTES segments, each folded by a
+//     warp, merged by one butterfly over the segments' partials (lane s holds
+//     segment s).  With enough rows to fill the chip a warp takes its row's
+//     segments in turn; with fewer, a CTA per row takes them at once.  Both
+//     do the same operations in the same order.
 //   * longer rows: the stretch is one of the row's SPLIT_CHUNK_BYTES chunks
 //     (a few long rows then spread over every SM instead of a few warps).
 //     The launch has one 1024-thread CTA per SM (256-thread CTAs, as many as
@@ -35,37 +42,33 @@
 #include "common.cuh"
 #include "debug.cuh"
 #include "fold.cuh"
+#include "group.cuh"
+#include "rows.cuh"
 
 namespace accr {
 
 
-constexpr int WB = 256;  // threads per CTA of the warp-per-row form (8 rows in flight)
-// Threads per CTA of the split form: 1024 (one CTA per SM) where the fold
-// fits 64 registers (4-byte elements, one or two clauses), else 256 (as many
-// CTAs per SM as the registers allow).
-template <typename T, int NC, bool SPLIT>
+enum RowForm { ROW_SEG = 0, ROW_SPLIT = 1, ROW_SEG_CTA = 2 };
+
+constexpr int WB = 256;  // threads per CTA of the group and warp-per-row forms
+// Threads per CTA.  Split form: 1024 (one CTA per SM) where the fold fits 64
+// registers (4-byte elements, one or two clauses), else 256 (as many CTAs per
+// SM as the registers allow).  One-row CTAs of the segment form: at most 1024
+// or 512, one warp per segment (the launch has no more warps than segments).
+template <typename T, int NC, int FORM>
 constexpr int row_threads() {
-    return !SPLIT ? WB : (sizeof(T) == 4 && NC <= 2) ? 1024 : 256;
+    return FORM == ROW_SPLIT     ? ((sizeof(T) == 4 && NC <= 2) ? 1024 : 256)
+           : FORM == ROW_SEG_CTA ? ((sizeof(T) == 4 && NC <= 2) ? 1024 : 512)
+                                 : WB;
 }
-// 16-byte vectors per lane per iteration: picked by the autotuner ("vectors"
-// in tuning.json), passed in by the build.
-#ifndef ACCR_ROW_RU
-#define ACCR_ROW_RU 8
-#endif
-constexpr int RU2 = ACCR_ROW_RU;
+constexpr int64_t WARP_ROW_BYTES = 16 * 1024;
+constexpr int64_t SEG_BYTES = 8 * 1024;
 constexpr int64_t SPLIT_ROW_BYTES = 256 * 1024;
 constexpr int64_t SPLIT_CHUNK_BYTES = 32 * 1024;
-
-struct RowArgs {
-    const void *A;
-    int64_t rows, cols, ld;
-    int nc;
-    ClauseDev cl[ACCR_MAX_CLAUSES];
-    int64_t chunk;        // split form: elements per chunk
-    int64_t cpr;          // split form: chunks per row
-    Partial *partials;    // split form: [rows][nc][cpr]
-    unsigned *counters;   // split form: [rows], zero on entry, zero again on exit (zeroed_words_for)
-};
+static_assert(SPLIT_ROW_BYTES / SEG_BYTES <= 32, "a row's segments fit one warp's lanes");
+// Segment form: below this many rows per SM a CTA takes each row (a warp per
+// row keeps 4 KiB in flight; 24 warps an SM are past what HBM needs).
+constexpr int64_t SEG_WARP_ROWS_PER_SM = 24;
 
 __device__ __forceinline__ Partial ld_row_partial(const Partial *p) {
     uint4 v = __ldcg(reinterpret_cast<const uint4 *>(p));
@@ -76,70 +79,13 @@ __device__ __forceinline__ Partial ld_row_partial(const Partial *p) {
     return q;
 }
 
-__device__ __forceinline__ uint4 ld_row(const uint4 *p) {
-    uint4 v;
-    asm("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4];"
-        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-        : "l"(p));
-    return v;
-}
-
-// One stretch of a row (elements [lo, lo + len) of row r), folded by one
-// warp and merged across its lanes.
-template <typename T, int NC>
-__device__ __forceinline__ void fold_stretch(const RowArgs &p, const int (&w)[NC], int64_t r, int64_t lo, int64_t len,
-                                             int lane, Acc (&A)[NC]) {
-    constexpr bool E64 = sizeof(T) == 8;
-    constexpr int EPV = 16 / (int)sizeof(T);
-    const T *row = (const T *)p.A + r * p.ld + lo;
-    const int64_t mis = (int64_t)(((16 - ((uintptr_t)row & 15)) & 15) / sizeof(T));
-    const int64_t head = mis < len ? mis : len;
-    const uint4 *vr = (const uint4 *)(row + head);
-    const int64_t nvec = (len - head) / EPV;
-    const int64_t tail0 = head + nvec * EPV;
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        A[c].a = p.cl[c].ident;
-        A[c].c = 0.f;
-    }
-    if (lane < head) {
-        T x = row[lane];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) fold_one<T>(w[c], A[c], x);
-    }
-    if (tail0 + lane < len) {
-        T x = row[tail0 + lane];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) fold_one<T>(w[c], A[c], x);
-    }
-    int64_t v = lane;
-    for (; v + (RU2 - 1) * 32 < nvec; v += 32 * RU2) {
-        uint4 b[RU2];
-#pragma unroll
-        for (int u = 0; u < RU2; ++u) b[u] = ld_row(vr + v + u * 32);
-#pragma unroll
-        for (int c = 0; c < NC; ++c) fold_vec<T, RU2>(w[c], A[c], b);
-    }
-#pragma unroll
-    for (int u = 0; u < RU2; ++u) {
-        const int64_t vv = v + u * 32;
-        if (vv < nvec) {
-            uint4 b = ld_row(vr + vv);
-#pragma unroll
-            for (int c = 0; c < NC; ++c) fold_vec<T, 1>(w[c], A[c], &b);
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < NC; ++c) warp_merge(w[c], E64, A[c]);
-}
-
 // W0 / W1 >= 0 fix the working codes of clauses 0 / 1 at compile time (the
 // fold's operator switch then disappears from the row loop); -1 reads them
-// from the arguments.  SPLIT selects the chunked form for long rows.
-template <typename T, int NC, int W0 = -1, int W1 = -1, bool SPLIT = false>
-__global__ void __launch_bounds__(row_threads<T, NC, SPLIT>()) rowreduce_kernel(const __grid_constant__ RowArgs p) {
-    constexpr bool E64 = sizeof(T) == 8;
-    constexpr int NTH = row_threads<T, NC, SPLIT>(), NW = NTH / 32;
+// from the arguments.  FORM: see the top of the file.
+template <typename T, int NC, int W0 = -1, int W1 = -1, int FORM = ROW_SEG>
+__global__ void __launch_bounds__(row_threads<T, NC, FORM>()) rowreduce_kernel(const __grid_constant__ RowArgs p) {
+    constexpr bool E64 = sizeof(T) == 8, FIXED = W0 >= 0;
+    constexpr int NTH = row_threads<T, NC, FORM>(), NW = NTH / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t gw = (int64_t)blockIdx.x * NW + warp;
     const int64_t cols = p.cols;
@@ -148,15 +94,52 @@ __global__ void __launch_bounds__(row_threads<T, NC, SPLIT>()) rowreduce_kernel(
     for (int c = 0; c < NC; ++c) w[c] = (c == 0 && W0 >= 0) ? W0 : (c == 1 && W1 >= 0) ? W1 : p.cl[c].wcode;
     Acc A[NC];
 
-    if (!SPLIT) {
-        const int64_t warps = (int64_t)gridDim.x * NW;
-        for (int64_t r = gw; r < p.rows; r += warps) {
-            fold_stretch<T, NC>(p, w, r, 0, cols, lane, A);
-            if (lane == 0) {
+    if (FORM == ROW_SEG || FORM == ROW_SEG_CTA) {
+        // The partial of segment s goes to lane s (identity past the last), in
+        // the code of the final merge, and one butterfly merges the lanes.
+        const int nseg = (int)p.cpr;
+        __shared__ Acc seg[NC][FORM == ROW_SEG_CTA ? 32 : 1];
+        Acc P[NC];
+        int fw[NC];
 #pragma unroll
-                for (int c = 0; c < NC; ++c)
-                    if (ACCR_DCHECK(r < p.rows, DS_ROW_VAR))
-                        store_var(p.cl[c], r, finish(p.cl[c], E64, cols == 0, to_final(w[c], A[c])));
+        for (int c = 0; c < NC; ++c) fw[c] = final_code(w[c]);
+        const int64_t step = FORM == ROW_SEG ? (int64_t)gridDim.x * NW : (int64_t)gridDim.x;
+        for (int64_t r = FORM == ROW_SEG ? gw : (int64_t)blockIdx.x; r < p.rows; r += step) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                P[c].a = final_ident(p.cl[c]);
+                P[c].c = 0.f;
+            }
+            const int s0 = FORM == ROW_SEG ? 0 : warp, ds = FORM == ROW_SEG ? 1 : (int)(blockDim.x >> 5);
+            for (int s = s0; s < nseg; s += ds) {
+                const int64_t lo = s * p.chunk;
+                const int64_t len = (cols - lo) < p.chunk ? (cols - lo) : p.chunk;
+                if (!ACCR_DCHECK(lo + len <= cols && s < 32, DS_ROW_CHUNK)) continue;
+                fold_stretch<T, NC, FIXED>((const T *)p.A + r * p.ld + lo, (int)len, p.cl, w, lane, A);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    if (FORM == ROW_SEG) {
+                        const Acc F = to_final(w[c], A[c]);
+                        if (lane == s) P[c] = F;
+                    } else if (lane == 0) {
+                        seg[c][s] = to_final(w[c], A[c]);
+                    }
+                }
+            }
+            if (FORM == ROW_SEG_CTA) {
+                __syncthreads();
+                if (warp == 0 && lane < nseg) {
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) P[c] = seg[c][lane];
+                }
+                __syncthreads();  // the next row's partials may follow
+                if (warp != 0) continue;
+            }
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                if (nseg > 1) warp_merge<FIXED>(fw[c], E64, P[c]);
+                if (lane == 0 && ACCR_DCHECK(r < p.rows, DS_ROW_VAR))
+                    store_var(p.cl[c], r, finish(p.cl[c], E64, cols == 0, P[c]));
             }
         }
         return;
@@ -169,7 +152,7 @@ __global__ void __launch_bounds__(row_threads<T, NC, SPLIT>()) rowreduce_kernel(
         const int64_t r = k / p.cpr, j = k - r * p.cpr, lo = j * p.chunk;
         const int64_t len = (cols - lo) < p.chunk ? (cols - lo) : p.chunk;
         if (!ACCR_DCHECK(r < p.rows && lo + len <= cols, DS_ROW_CHUNK)) continue;
-        fold_stretch<T, NC>(p, w, r, lo, len, lane, A);
+        fold_stretch<T, NC, FIXED>((const T *)p.A + r * p.ld + lo, (int)len, p.cl, w, lane, A);
         if (lane == 0) {
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
@@ -240,7 +223,7 @@ __global__ void __launch_bounds__(row_threads<T, NC, SPLIT>()) rowreduce_kernel(
                         }
                     }
             }
-            cta_merge<NC, NTH>(fw, fid, E64, A, sh);
+            cta_merge<NC, NTH, FIXED>(fw, fid, E64, A, sh);
             if (threadIdx.x == 0) {
 #pragma unroll
                 for (int c = 0; c < NC; ++c)
@@ -253,89 +236,47 @@ __global__ void __launch_bounds__(row_threads<T, NC, SPLIT>()) rowreduce_kernel(
     }
 }
 
-template <typename T, int NC, int W0, int W1, bool SPLIT>
-static int max_row_grid() {
+// ---- host side ---------------------------------------------------------------------
+
+template <typename T, int NC, int W0, int W1, int FORM>
+static void row_form(const RowArgs &a, cudaStream_t s) {
     static std::atomic<int> cached[64];
-    const DeviceInfo &d = device_info();
-    std::atomic<int> &slot = cached[d.id & 63];
-    int g = slot.load(std::memory_order_relaxed);
-    if (!g) {
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, rowreduce_kernel<T, NC, W0, W1, SPLIT>,
-                                                      row_threads<T, NC, SPLIT>(), 0);
-        if (per_sm < 1) per_sm = 1;
-        g = per_sm * d.sms;
-        slot.store(g, std::memory_order_relaxed);
+    constexpr int NTH = row_threads<T, NC, FORM>();
+    if (FORM == ROW_SEG_CTA) {  // a CTA per row, a warp per segment
+        const int nt = a.cpr * 32 < NTH ? (int)a.cpr * 32 : NTH;
+        rowreduce_kernel<T, NC, W0, W1, FORM><<<(unsigned)a.rows, nt, 0, s>>>(a);
+        return;
     }
-    return g;
+    const int maxg = resident_ctas(rowreduce_kernel<T, NC, W0, W1, FORM>, NTH, cached);
+    // chunks of long rows: at most one CTA per chunk, each taking a contiguous
+    // run; else a warp per row, rows past the resident grid in later rounds
+    const int64_t want = FORM == ROW_SPLIT ? a.rows * a.cpr : (a.rows + NTH / 32 - 1) / (NTH / 32);
+    rowreduce_kernel<T, NC, W0, W1, FORM><<<clamp_grid(want, maxg), NTH, 0, s>>>(a);
 }
 
-// CTAs for `segs` stretches: rows (one warp per row, at most the resident
-// grid, the rest in later rounds), or chunks of long rows (the resident grid,
-// at most one CTA per chunk, each CTA taking a contiguous run).
-template <typename T, int NC, int W0, int W1, bool SPLIT>
-static int row_grid(int64_t segs) {
-    const int64_t maxg = max_row_grid<T, NC, W0, W1, SPLIT>();
-    const int64_t g = SPLIT ? segs : (segs + WB / 32 - 1) / (WB / 32);
-    return (int)(g < 1 ? 1 : g < maxg ? g : maxg);
-}
-
-template <typename T, int NC, int W0 = -1, int W1 = -1>
-static int row_launch_t(RowArgs &a, cudaStream_t s) {
+template <typename T, int NC, int W0, int W1>
+static int row_launch_t(RowArgs &a, int form, cudaStream_t s) {
     int rc = launch_guard("rowreduce_kernel");
     if (rc != ACCR_OK) return rc;
-    if (a.cpr > 0) {
-        rowreduce_kernel<T, NC, W0, W1, true>
-            <<<row_grid<T, NC, W0, W1, true>(a.rows * a.cpr), row_threads<T, NC, true>(), 0, s>>>(a);
+    if (form == ROW_SPLIT) {
+        row_form<T, NC, W0, W1, ROW_SPLIT>(a, s);
+    } else if (form == ROW_SEG) {
+        row_form<T, NC, W0, W1, ROW_SEG>(a, s);
     } else {
-        rowreduce_kernel<T, NC, W0, W1, false><<<row_grid<T, NC, W0, W1, false>(a.rows), WB, 0, s>>>(a);
+        row_form<T, NC, W0, W1, ROW_SEG_CTA>(a, s);
     }
     return launched("rowreduce_kernel");
 }
 
-// A sum together with a max or a min (the two-clause form of a region that
-// reports a total and an extreme) gets a kernel with both codes fixed: the
-// generic two-clause fold needs 64 registers a thread, the fixed one 32-40,
-// which leaves room for more rows in flight per SM.
-template <typename T, int W0, int W1>
-static bool pair_launch(RowArgs &a, cudaStream_t s, int &rc) {
-    if (a.cl[0].wcode != W0 || a.cl[1].wcode != W1) return false;
-    rc = row_launch_t<T, 2, W0, W1>(a, s);
-    return true;
-}
+struct RowLaunch {
+    int form;
+    template <typename T, int NC, int W0, int W1>
+    int run(RowArgs &a, cudaStream_t s) const {
+        return row_launch_t<T, NC, W0, W1>(a, form, s);
+    }
+};
 
-template <typename T>
-static bool row_launch_pair(RowArgs &a, cudaStream_t s, int &rc) {
-    auto is_sum = [](int w) { return w == W_ADD32 || w == W_ADD64 || w == W_ADDF || w == W_ADDF_COMP; };
-    if (!is_sum(a.cl[0].wcode) && is_sum(a.cl[1].wcode)) {  // each clause carries its own output
-        const ClauseDev t = a.cl[0];
-        a.cl[0] = a.cl[1];
-        a.cl[1] = t;
-    }
-    if constexpr (std::is_same<T, float>::value) {
-        return pair_launch<T, W_ADDF, W_MAXF>(a, s, rc) || pair_launch<T, W_ADDF, W_MINF>(a, s, rc) ||
-               pair_launch<T, W_ADDF_COMP, W_MAXF>(a, s, rc) || pair_launch<T, W_ADDF_COMP, W_MINF>(a, s, rc);
-    } else if constexpr (std::is_same<T, double>::value) {
-        return pair_launch<T, W_ADDF, W_MAXF>(a, s, rc) || pair_launch<T, W_ADDF, W_MINF>(a, s, rc);
-    } else if constexpr (std::is_same<T, int32_t>::value) {
-        return pair_launch<T, W_ADD32, W_MAXI>(a, s, rc) || pair_launch<T, W_ADD32, W_MINI>(a, s, rc) ||
-               pair_launch<T, W_ADD64, W_MAXI>(a, s, rc) || pair_launch<T, W_ADD64, W_MINI>(a, s, rc);
-    } else {
-        return pair_launch<T, W_ADD64, W_MAXI>(a, s, rc) || pair_launch<T, W_ADD64, W_MINI>(a, s, rc);
-    }
-}
-
-template <typename T>
-static int row_launch(RowArgs &a, cudaStream_t s) {
-    int rc = ACCR_OK;
-    if (a.nc == 2 && row_launch_pair<T>(a, s, rc)) return rc;
-    switch (a.nc) {
-    case 1: return row_launch_t<T, 1>(a, s);
-    case 2: return row_launch_t<T, 2>(a, s);
-    case 3: return row_launch_t<T, 3>(a, s);
-    default: return row_launch_t<T, 4>(a, s);
-    }
-}
+int rowgroup_launch(RowArgs &a, int in_type, cudaStream_t s);  // rowgroup.cu
 
 }  // namespace accr
 
@@ -361,10 +302,15 @@ extern "C" ACCR_API int accr_rowreduce(const void *A, int64_t rows, int64_t cols
     RowArgs a;
     memset(&a, 0, sizeof a);
     const int64_t eb = type_bytes(in_type), row_bytes = cols * eb;
-    log_msg(2, "accr_rowreduce: %lld x %lld (ld %lld) type=%d clauses=%d form=%s", (long long)rows, (long long)cols,
-            (long long)ld, in_type, nclauses, row_bytes >= SPLIT_ROW_BYTES ? "split rows" : "warp per row");
-    if (row_bytes >= SPLIT_ROW_BYTES) {
+    int form = ROW_SEG;
+    if (row_bytes <= GROUP_BYTES) {
+        // about four vectors a lane: fewer leave lanes idle and pay more
+        // shuffles a row, more lengthen each lane's chain
+        a.lanes = 1;
+        while (a.lanes < 32 && a.lanes * 4 * 16 < row_bytes) a.lanes *= 2;
+    } else if (row_bytes >= SPLIT_ROW_BYTES) {
         // chunked form: partials [rows][nclauses][cpr] and one counter per row
+        form = ROW_SPLIT;
         a.chunk = SPLIT_CHUNK_BYTES / eb;
         a.cpr = (cols + a.chunk - 1) / a.chunk;
         const size_t pbytes = (size_t)rows * (size_t)nclauses * (size_t)a.cpr * sizeof(Partial);
@@ -373,19 +319,24 @@ extern "C" ACCR_API int accr_rowreduce(const void *A, int64_t rows, int64_t cols
         a.partials = (Partial *)scr->buf;
         a.counters = zeroed_words_for(stream, (size_t)rows);  // every row completes, so each returns to zero
         if (!a.counters) return ACCR_ENOMEM;
+    } else if (row_bytes > WARP_ROW_BYTES) {
+        form = rows < SEG_WARP_ROWS_PER_SM * device_info().sms ? ROW_SEG_CTA : ROW_SEG;
+        a.chunk = SEG_BYTES / eb;
+        a.cpr = (cols + a.chunk - 1) / a.chunk;
+    } else {
+        a.chunk = cols;  // one stretch, no merge of segments
+        a.cpr = 1;
     }
+    static const char *const names[] = {"warp per row", "split rows", "CTA per row"};
+    log_msg(2, "accr_rowreduce: %lld x %lld (ld %lld) type=%d clauses=%d form=%s", (long long)rows, (long long)cols,
+            (long long)ld, in_type, nclauses, a.lanes > 0 ? "lane group per row" : names[form]);
     a.A = A;
     a.rows = rows;
     a.cols = cols;
     a.ld = ld;
     a.nc = nclauses;
     for (int c = 0; c < nclauses; ++c) a.cl[c] = cl[c];
-    switch (in_type) {
-    case ACCR_I32: rc = row_launch<int32_t>(a, s); break;
-    case ACCR_I64: rc = row_launch<int64_t>(a, s); break;
-    case ACCR_F32: rc = row_launch<float>(a, s); break;
-    default: rc = row_launch<double>(a, s); break;
-    }
+    rc = a.lanes > 0 ? rowgroup_launch(a, in_type, s) : row_dispatch(a, in_type, RowLaunch{form}, s);
     if (rc != ACCR_OK) return rc;
     if (flags & ACCR_SYNC) return cuda_check(cudaStreamSynchronize(s), "accr_rowreduce: sync");
     return ACCR_OK;
