@@ -9,8 +9,8 @@
 
 namespace accr {
 
-constexpr int GV = 8;                          // vectors per lane at most
-constexpr int64_t GROUP_BYTES = GV * 32 * 16;  // 4 KiB
+constexpr int GROUP_GV = 8;                          // vectors per lane at most
+constexpr int64_t GROUP_BYTES = GROUP_GV * 32 * 16;  // 4 KiB
 
 // A running fold of one clause of a fixed code in registers: whole vectors and
 // single elements in, an accumulator out.  The primary form keeps the
@@ -66,7 +66,7 @@ struct GroupFold<float, W_MINF> : GroupExtreme<false> {};
 // Folds the loaded vectors of one lane.  A pair kernel folds the vectors the
 // lane holds one by one; a generic one fills the others with the clause's
 // neutral element, so that its operator switch runs once for all of them.
-template <typename T, int NV>
+template <typename T, int NV, int GV>
 __device__ __forceinline__ void fold_filled(int w, Acc &A, const uint4 (&b)[GV], const bool (&ok)[GV], uint64_t neutral) {
     const uint32_t lo = (uint32_t)neutral, hi = sizeof(T) == 8 ? (uint32_t)(neutral >> 32) : lo;
     uint4 f[NV];
@@ -79,7 +79,7 @@ __device__ __forceinline__ void fold_filled(int w, Acc &A, const uint4 (&b)[GV],
 // number l of it) into A and merged across the group.  `rounds`: no lane of the
 // warp has more than this many vectors (at most GV).  Lanes that are not live
 // take part in the merge only.  Every load is in flight before any is folded.
-template <typename T, int NC, int W0, int W1>
+template <typename T, int NC, int W0, int W1, int GV>
 __device__ __forceinline__ void group_fold(const T *in, int len, bool live, int l, int L, int rounds,
                                            const ClauseDev *cl, const uint64_t *neutral, const int (&w)[NC],
                                            Acc (&A)[NC]) {
@@ -126,8 +126,8 @@ __device__ __forceinline__ void group_fold(const T *in, int len, bool live, int 
         for (int c = 0; c < NC; ++c) {
             A[c].a = cl[c].ident;
             A[c].c = 0.f;
-            if (rounds > GV / 2) fold_filled<T, GV>(w[c], A[c], b, ok, neutral[c]);
-            else if (rounds > 0) fold_filled<T, GV / 2>(w[c], A[c], b, ok, neutral[c]);
+            if (rounds > GV / 2) fold_filled<T, GV, GV>(w[c], A[c], b, ok, neutral[c]);
+            else if (rounds > 0) fold_filled<T, GV / 2, GV>(w[c], A[c], b, ok, neutral[c]);
             for (int j = l; j < head; j += L) fold_one<T>(w[c], A[c], j == l ? h : __ldg(in + j));
             for (int j = tail0 + l; j < end; j += L) fold_one<T>(w[c], A[c], j == tail0 + l ? t : __ldg(in + j));
         }
