@@ -322,7 +322,8 @@ ACCR_API int accr_standardize(const float *x, int64_t n, float *y,
 
 #define ACCR_BFS_REDUCE 0     /* levels driven by the host; || reduction of the flag */
 #define ACCR_BFS_GUARDED 1    /* levels driven by the host; flag cleared, threads write only 1 */
-#define ACCR_BFS_PERSISTENT 2 /* all levels in one cooperative launch, grid barriers */
+#define ACCR_BFS_PERSISTENT 2 /* all levels in one cooperative launch; grids of at most
+                                 2^28 cells on bitmaps, several levels between barriers */
 
 /*
  * accr_grid_bfs -- BFS's convergence loop: level-synchronous search on a

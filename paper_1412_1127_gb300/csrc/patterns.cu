@@ -22,7 +22,8 @@
 //    OpenACC version reduces a global boolean with ||; the CUDA version
 //    initialises the flag and lets threads write only `true`.  Both forms run
 //    here with the host driving the levels, and a third keeps every level in
-//    one cooperative launch with a bounded grid barrier between levels.
+//    one cooperative launch: on bitmaps, in tiles whose halo lets a CTA run
+//    several levels between two bounded grid barriers.
 //
 // Every cross-CTA wait spins a bounded number of times; on expiry it records
 // a code in a status word and the host reports ACCR_ETIMEDOUT.
@@ -51,12 +52,12 @@ __device__ __forceinline__ void st_release(unsigned *p, unsigned v) {
 }
 
 // Grid barrier for a cooperative launch that also ORs one CTA-uniform flag:
-// generation counting, bounded spin.  bar[0] counts arrivals (low 20 bits)
-// and raised flags (bits 20 and up); bar[1] holds (generation << 1) | OR of
-// the flags, published by the last CTA to arrive, so the flag comes back
-// with the release instead of through a word of its own.  Returns 0 if the
-// wait ran out, else 1 + the OR of the flags.
-__device__ __forceinline__ int grid_barrier_or(unsigned *bar, unsigned &gen, bool flag) {
+// generation counting, bounded spin.  `ctas` CTAs take part.  bar[0] counts
+// arrivals (low 20 bits) and raised flags (bits 20 and up); bar[1] holds
+// (generation << 1) | OR of the flags, published by the last CTA to arrive, so
+// the flag comes back with the release instead of through a word of its own.
+// Returns 0 if the wait ran out, else 1 + the OR of the flags.
+__device__ __forceinline__ int grid_barrier_or(unsigned *bar, unsigned &gen, bool flag, unsigned ctas) {
     __shared__ int s_res;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -64,7 +65,7 @@ __device__ __forceinline__ int grid_barrier_or(unsigned *bar, unsigned &gen, boo
         __threadfence();
         const unsigned old = atomicAdd(&bar[0], 1u + (flag ? (1u << 20) : 0u));
         int res = 0;
-        if ((old & 0xfffffu) == gridDim.x - 1) {
+        if ((old & 0xfffffu) == ctas - 1) {
             const unsigned any = ((old >> 20) != 0u || flag) ? 1u : 0u;
             bar[0] = 0u;
             st_release(&bar[1], (my << 1) | any);
@@ -73,7 +74,7 @@ __device__ __forceinline__ int grid_barrier_or(unsigned *bar, unsigned &gen, boo
             uint32_t i = 0;
             unsigned v = ld_acquire(&bar[1]);
             while ((v >> 1) != my && ++i <= kSpinLimit) {
-                __nanosleep(64);
+                if (i > 256) __nanosleep(64);
                 v = ld_acquire(&bar[1]);
             }
             if ((v >> 1) == my) res = 1 + (int)(v & 1u);
@@ -903,7 +904,7 @@ __global__ void __launch_bounds__(BFP_THREADS, 1) bfs_persistent_kernel(const ui
     for (; L < max_levels; ++L) {
         const bool changed = bfs_level(open, dist, rows, cols, (int32_t)L);
         const int any = __syncthreads_or(changed ? 1 : 0);
-        const int r = grid_barrier_or(bar, gen, any != 0);
+        const int r = grid_barrier_or(bar, gen, any != 0, gridDim.x);
         if (r == 0) {
             if (threadIdx.x == 0) atomicExch(err, 7);
             return;
@@ -911,6 +912,297 @@ __global__ void __launch_bounds__(BFP_THREADS, 1) bfs_persistent_kernel(const ui
         if (r == 1) break;  // no cell changed at this level
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) *levels_out = L + 1;  // the level that found nothing new
+}
+
+
+// All levels in one cooperative launch, on bitmaps.  A level of the cell-wise
+// form costs a sweep of every cell through L2 and a grid barrier (4.8 us at
+// 1024 x 1024); the levels here run in shared memory and registers, several
+// between barriers.
+//
+//   * A cell is a bit of two bitmaps, 32 cells of a row to a word: still free
+//     (open and unvisited) and frontier (joined at the current level).  A level
+//     is new = (frontier shifted by one cell each way) & free.
+//   * A CTA takes a tile of BT_ROWS rows by 32 words: lane = word, thread = four
+//     rows of it in registers, rows past a warp's own through shared memory, so
+//     a level costs about 60 instructions a warp and one CTA barrier.
+//   * A tile carries a halo of `depth` cells on each side that is not the
+//     grid's own edge.  A cell's state after d levels depends on cells at most
+//     d away, so `depth` levels run on the tile's own copy and leave its
+//     interior exact; then the interior goes back to the bitmaps (two copies,
+//     read and written in turn), one grid barrier carries the `||` of "a
+//     frontier is left", and the tiles load again.
+//
+// With one tile the loop runs to the end without grid barriers.  1024 x 1024
+// cells, 62 % open, about 1,260 levels: 6.2 ms in the cell-wise form, 0.63 ms here
+// (0.33 us a level, and 4 us a step of 28 levels for loading, storing and the
+// barrier; what is left is the chain of a level's instructions and its CTA barrier).
+constexpr int BT_R = 4;                     // rows per thread
+constexpr int BT_THREADS = 512;             // 16 warps: 64 rows a tile
+constexpr int BT_ROWS = BT_R * (BT_THREADS / 32);
+constexpr int BT_MAX_DEPTH = 30;            // at most 31 (five bit planes), and the 32 columns of halo a tile has
+                                            // on each side where a row needs several tiles
+constexpr int64_t BT_MAX_CELLS = (int64_t)1 << 28;  // larger grids: the cell-wise form (bitmaps are kept as scratch)
+
+struct BfsTiles {
+    const uint8_t *open;
+    int32_t *dist;
+    int rows, cols, wpr;        // wpr: words per row
+    int64_t src;                // -1: none
+    uint32_t *free_[2], *front[2];
+    int tiles_r, tiles_c, int_rows, int_words, depth;  // depth 0: one tile, until nothing changes
+    unsigned tile_ctas;         // CTAs with tiles (the others only set up)
+    unsigned *bar;
+    int *best;                  // largest distance so far, and CTAs done; zero on entry and exit
+    unsigned *done;
+    int64_t *result;            // pinned: {levels, status}
+};
+
+__global__ void __launch_bounds__(BT_THREADS, 1) bfs_tile_kernel(const __grid_constant__ BfsTiles p) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int NW = BT_THREADS / 32;
+    __shared__ uint32_t edge[2][NW][2][32];
+    __shared__ uint32_t planes[5][BT_ROWS / 2][32];
+    unsigned gen = (*(volatile unsigned *)&p.bar[1]) >> 1;
+
+    // set-up: the bitmaps and dist = -1, one word (32 cells) per warp step
+    constexpr int SUN = 4;
+    const int nwords = p.rows * p.wpr;  // below 2^26: BT_MAX_CELLS cells and at least one cell a word
+    for (int i0 = (blockIdx.x * NW + warp) * SUN; i0 < nwords; i0 += gridDim.x * NW * SUN) {
+        uint8_t o[SUN];
+        int64_t c[SUN];
+        bool in[SUN];
+#pragma unroll
+        for (int j = 0; j < SUN; ++j) {
+            const int i = i0 + j, r = i / p.wpr, q = (i - r * p.wpr) * 32 + lane;
+            in[j] = i < nwords && q < p.cols;
+            c[j] = (int64_t)r * p.cols + q;
+            o[j] = in[j] ? __ldg(p.open + c[j]) : (uint8_t)0;
+        }
+#pragma unroll
+        for (int j = 0; j < SUN; ++j) {
+            const bool is_src = in[j] && c[j] == p.src && o[j] != 0;
+            const unsigned fr = __ballot_sync(0xffffffffu, is_src);
+            const unsigned av = __ballot_sync(0xffffffffu, o[j] != 0 && !is_src);
+            if (in[j]) p.dist[c[j]] = is_src ? 0 : -1;
+            if (lane == 0 && i0 + j < nwords) {
+                p.free_[0][i0 + j] = av;
+                p.front[0][i0 + j] = fr;
+            }
+        }
+    }
+    const bool started = p.src >= 0 && __ldg(p.open + (p.src >= 0 ? p.src : 0)) != 0;
+    int ok = grid_barrier_or(p.bar, gen, false, gridDim.x);
+    if (ok && blockIdx.x >= p.tile_ctas) return;
+
+    int reached = 0;  // largest distance this thread gave
+    int L = 0;
+    const int ntiles = p.tiles_r * p.tiles_c;
+    for (int k = 0; ok && started; ++k) {
+        const uint32_t *fin = p.free_[k & 1], *rin = p.front[k & 1];
+        uint32_t *fout = p.free_[(k & 1) ^ 1], *rout = p.front[(k & 1) ^ 1];
+        bool left = false;
+        for (int tile = blockIdx.x; tile < ntiles; tile += p.tile_ctas) {
+            const int tr = tile / p.tiles_c, tc = tile - tr * p.tiles_c;
+            const int r0 = tr * p.int_rows, r1 = min(p.rows, r0 + p.int_rows);
+            const int top = p.tiles_r > 1 ? r0 - p.depth : 0;
+            const int word = p.tiles_c > 1 ? tc * p.int_words - 1 + lane : lane;
+            const bool col_in = word >= 0 && word < p.wpr;
+            const bool mine = col_in && (p.tiles_c == 1 || (lane >= 1 && lane <= p.int_words));
+            uint32_t a[BT_R], f[BT_R];
+            bool own[BT_R];
+#pragma unroll
+            for (int j = 0; j < BT_R; ++j) {
+                const int r = top + warp * BT_R + j;
+                const bool in = col_in && r >= 0 && r < p.rows;
+                own[j] = mine && r >= r0 && r < r1;
+                a[j] = in ? __ldcg(fin + (int64_t)r * p.wpr + word) : 0u;
+                f[j] = in ? __ldcg(rin + (int64_t)r * p.wpr + word) : 0u;
+            }
+            bool more = true;
+            int base = L;
+            do {
+                // up to `run` levels; the level each cell joined at (1 .. 30) is kept
+                // in five bit planes and its distance stored at the end: stores
+                // inside the loop held up the whole CTA at every level's barrier
+                uint32_t pl[5][BT_R];
+#pragma unroll
+                for (int i = 0; i < 5; ++i)
+#pragma unroll
+                    for (int j = 0; j < BT_R; ++j) pl[i][j] = 0u;
+                const int run = p.depth == 0 ? 30 : p.depth;  // even: the next run starts on the other edge words
+                for (int d = 1; d <= run; ++d) {
+                    edge[d & 1][warp][0][lane] = f[0];
+                    edge[d & 1][warp][1][lane] = f[BT_R - 1];
+                    uint32_t any = f[0];
+#pragma unroll
+                    for (int j = 1; j < BT_R; ++j) any |= f[j];
+                    if ((d & 3) != 1) {
+                        __syncthreads();
+                    } else if (!__syncthreads_or((int)any)) {  // no frontier in the tile: the same for the whole CTA
+                        more = false;
+                        break;
+                    }
+                    uint32_t above = warp > 0 ? edge[d & 1][warp - 1][1][lane] : 0u;
+                    const uint32_t below = warp + 1 < NW ? edge[d & 1][warp + 1][0][lane] : 0u;
+                    if (!__any_sync(0xffffffffu, (any | above | below) != 0u)) continue;  // nothing near this warp's rows
+#pragma unroll
+                    for (int j = 0; j < BT_R; ++j) {
+                        uint32_t lw = __shfl_up_sync(0xffffffffu, f[j], 1), rw = __shfl_down_sync(0xffffffffu, f[j], 1);
+                        if (lane == 0) lw = 0u;
+                        if (lane == 31) rw = 0u;
+                        const uint32_t next = j + 1 < BT_R ? f[j + 1] : below;
+                        const uint32_t n = (__funnelshift_l(lw, f[j], 1) | __funnelshift_r(f[j], rw, 1) | above | next) & a[j];
+                        above = f[j];
+                        f[j] = n;
+                        a[j] &= ~n;
+                    }
+#pragma unroll
+                    for (int i = 0; i < 5; ++i) {
+                        if ((d >> i) & 1) {
+#pragma unroll
+                            for (int j = 0; j < BT_R; ++j) pl[i][j] |= f[j];
+                        }
+                    }
+                }
+                // the interior's planes to shared memory, half a tile of rows at a
+                // time, and from there by every warp, a word (32 cells, one a lane) a
+                // step: the interior's own warps are few
+                const int irows = r1 - r0;
+                for (int h = 0; h < irows; h += BT_ROWS / 2) {
+#pragma unroll
+                    for (int j = 0; j < BT_R; ++j) {
+                        const int i = top + warp * BT_R + j - r0 - h;
+                        if (i >= 0 && i < BT_ROWS / 2) {
+#pragma unroll
+                            for (int q = 0; q < 5; ++q) planes[q][i][lane] = own[j] ? pl[q][j] : 0u;
+                        }
+                    }
+                    __syncthreads();
+                    const int n = min(BT_ROWS / 2, irows - h) * 32;
+                    for (int e = warp; e < n; e += NW) {
+                        const int i = e >> 5, c = e & 31;  // c: the lane that holds the word
+                        uint32_t q[5], m = 0u;
+#pragma unroll
+                        for (int z = 0; z < 5; ++z) {
+                            q[z] = planes[z][i][c];
+                            m |= q[z];
+                        }
+                        if ((m >> lane) & 1u) {
+                            int d = 0;
+#pragma unroll
+                            for (int z = 0; z < 5; ++z) d |= (int)((q[z] >> lane) & 1u) << z;
+                            const int w = p.tiles_c > 1 ? tc * p.int_words - 1 + c : c;
+                            p.dist[(int64_t)(r0 + h + i) * p.cols + w * 32 + lane] = base + d;
+                            reached = max(reached, base + d);
+                        }
+                    }
+                    __syncthreads();
+                }
+                base += run;
+            } while (p.depth == 0 && more);
+#pragma unroll
+            for (int j = 0; j < BT_R; ++j) {
+                if (own[j]) {
+                    const int64_t i = (int64_t)(top + warp * BT_R + j) * p.wpr + word;
+                    fout[i] = a[j];
+                    rout[i] = f[j];
+                    left |= f[j] != 0u;
+                }
+            }
+            __syncthreads();  // the next tile's first level writes the same edge words
+        }
+        if (p.depth == 0) break;
+        ok = grid_barrier_or(p.bar, gen, __syncthreads_or(left ? 1 : 0) != 0, p.tile_ctas);
+        if (ok == 1) break;  // no frontier is left anywhere
+        L += p.depth;
+    }
+    // largest distance, then the host's words by the last CTA
+#pragma unroll
+    for (int s = 16; s >= 1; s >>= 1) reached = max(reached, __shfl_xor_sync(0xffffffffu, reached, s));
+    __shared__ int far_[NW];
+    if (lane == 0) far_[warp] = reached;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < NW; ++w) reached = max(reached, far_[w]);
+        if (!ok) {
+            p.result[1] = 7;  // a barrier wait ran out; the host resets the words below
+        } else {
+            if (reached) atomicMax(p.best, reached);
+            __threadfence();
+            if (atomicAdd(p.done, 1u) == p.tile_ctas - 1) {
+                __threadfence();
+                p.result[0] = started ? (int64_t)*(volatile int *)p.best + 1 : 0;
+                *p.best = 0;
+                *p.done = 0u;
+            }
+        }
+    }
+}
+
+// ---- host side ---------------------------------------------------------------------
+
+// The tiled form.  Tiles are sized so that there is about one per SM (its
+// interior then small and its halo, and so the levels between two barriers,
+// large); the interior is at most 32 rows and at least 4.
+static int bfs_tiled(const uint8_t *open, int64_t rows, int64_t cols, int64_t src, int32_t *dist, int64_t *levels,
+                     cudaStream_t s) {
+    const DeviceInfo &di = device_info();
+    BfsTiles a;
+    memset(&a, 0, sizeof a);
+    a.open = open;
+    a.dist = dist;
+    a.rows = (int)rows;
+    a.cols = (int)cols;
+    a.wpr = (int)((cols + 31) / 32);
+    a.src = (src >= 0 && src < rows * cols) ? src : -1;
+    a.int_words = a.wpr <= 32 ? 32 : 30;
+    a.tiles_c = a.wpr <= 32 ? 1 : (a.wpr + 29) / 30;
+    if (rows <= BT_ROWS) {
+        a.int_rows = (int)rows;
+        a.depth = a.tiles_c == 1 ? 0 : BT_MAX_DEPTH;
+    } else {
+        const int64_t per_sm = (rows * a.tiles_c + di.sms - 1) / di.sms;
+        a.int_rows = (int)std::min<int64_t>(std::max<int64_t>(per_sm, 4), 32);
+        a.depth = std::min((BT_ROWS - a.int_rows) / 2, BT_MAX_DEPTH);
+    }
+    a.tiles_r = (int)((rows + a.int_rows - 1) / a.int_rows);
+    const int64_t ntiles = (int64_t)a.tiles_r * a.tiles_c, nwords = rows * a.wpr;
+    a.tile_ctas = (unsigned)std::min<int64_t>(ntiles, di.sms);
+    // set-up takes 64 words a CTA and step
+    const int64_t setup = (nwords + 63) / 64;
+    const int grid = (int)std::min<int64_t>(std::max<int64_t>(setup, a.tile_ctas), di.sms);
+    const size_t wbytes = ((size_t)nwords * 4 + 255) & ~(size_t)255;
+    Scratch *scr = scratch_for((accr_stream_t)s, 4 * wbytes);
+    if (!scr) return ACCR_ENOMEM;
+    int64_t *res = (int64_t *)host_staging_for((accr_stream_t)s, 64);
+    if (!res) return ACCR_ENOMEM;
+    for (int i = 0; i < 2; ++i) {
+        a.free_[i] = (uint32_t *)((char *)scr->buf + (size_t)(2 * i) * wbytes);
+        a.front[i] = (uint32_t *)((char *)scr->buf + (size_t)(2 * i + 1) * wbytes);
+    }
+    a.bar = scr->counters + 12;            // arrivals, generation
+    a.best = (int *)(scr->counters + 15);
+    a.done = scr->counters + 16;
+    a.result = res;
+    res[0] = -1;
+    res[1] = 0;
+    int rc = launch_guard("bfs_tile_kernel");
+    if (rc != ACCR_OK) return rc;
+    void *args[] = {(void *)&a};
+    rc = cuda_check(cudaLaunchCooperativeKernel((const void *)bfs_tile_kernel, grid, BT_THREADS, args, 0, s),
+                    "accr_grid_bfs: cooperative launch");
+    if (rc != ACCR_OK) return rc;
+    if ((rc = launched("bfs_tile_kernel")) != ACCR_OK) return rc;
+    rc = cuda_check(cudaStreamSynchronize(s), "accr_grid_bfs: sync");
+    if (rc != ACCR_OK) return rc;
+    if (*(volatile int64_t *)&res[1] != 0 || *(volatile int64_t *)&res[0] < 0) {
+        cudaMemsetAsync(a.bar, 0, sizeof(unsigned), s);
+        cudaMemsetAsync(a.best, 0, 2 * sizeof(unsigned), s);
+        return set_error(ACCR_ETIMEDOUT, "accr_grid_bfs: grid barrier wait ran out");
+    }
+    *levels = res[0];
+    return ACCR_OK;
 }
 
 }  // namespace accr
@@ -1052,6 +1344,8 @@ extern "C" ACCR_API int accr_grid_bfs(const uint8_t *open, int64_t rows, int64_t
     if (total == 0) return ACCR_OK;
     cudaStream_t s = (cudaStream_t)stream;
     const DeviceInfo &di = device_info();
+    if (mode == ACCR_BFS_PERSISTENT && total <= BT_MAX_CELLS && (int64_t)rows * ((cols + 31) / 32) <= BT_MAX_CELLS / 8)
+        return bfs_tiled(open, rows, cols, src, dist, levels, s);
     int rc;
     if ((rc = launch_guard("bfs_init_kernel")) != ACCR_OK) return rc;
     bfs_init_kernel<<<di.sms * 4, 256, 0, s>>>(dist, total, (src >= 0 && src < total) ? src : -1, open);
