@@ -3,12 +3,9 @@
 //
 //  * Nearest Neighbor: distances to a query point and the k smallest -- a
 //    reduction whose operator keeps a sorted list of k (distance, index)
-//    pairs.  Each warp keeps one list in shared memory and tests a whole round
-//    of its points against the list's k-th distance at once; distance bounds
-//    (a warp's first round, then one taken from a sample of the whole array
-//    and published while the scan runs) keep the lists' slow path rare.  The
-//    CTA ranks its warps' entries, and the last CTA to finish ranks the few
-//    CTA entries that can still be among the k smallest.
+//    pairs.  The scan keeps each thread's nearest point; the last CTA to finish
+//    takes a bound from those and looks again at the few threads' points that
+//    can be among the k nearest.
 //
 //  * SRAD: a reduction region whose result feeds a data-parallel region.  The
 //    paper's OpenACC code merges the block partials on the CPU and launches
@@ -89,16 +86,43 @@ __device__ __forceinline__ int grid_barrier_or(unsigned *bar, unsigned &gen, boo
 // ============================================================================
 // Nearest Neighbor: k smallest squared distances
 // ============================================================================
+//
+// One plain launch, no CTA waits for another.  The scan keeps one thing per
+// thread, its nearest point, so it runs at the rate of its loads: lists of k per
+// warp cost it an insertion path, a merge of the lists per CTA and a k-round
+// tournament at the end (10 million points, k = 10: 42 us against the 11.8 us
+// their bytes take).  The k nearest are then found by the last CTA to finish:
+//
+//   * the k-th nearest of its 16 warps' shares of the warps' nearest points is a
+//     bound that at least k points reach;
+//   * a thread that holds one of the k nearest points has a nearest point within
+//     the bound, so only such threads' points are looked at again -- a few dozen
+//     threads of the 150,000, some hundred points each -- and the points within
+//     the bound become candidates;
+//   * the candidates are ranked by (distance, index).  If there are ever more
+//     than the array holds, the k best of them stay and the k-th is the new bound.
+//
+// Distances are never negative, so their bits order as unsigned integers, with
+// a NaN above infinity: NK_NONE, one above infinity, is "no point yet", and a
+// point whose distance is NaN never enters.  Ten million points, k = 10: 42 -> 24.7 us,
+// of which the bytes take 11.8 and the last CTA about 6.
 
-constexpr int NK_THREADS = 256;
+constexpr int NK_THREADS = 512;               // two CTAs per SM
+constexpr int NK_WARPS = NK_THREADS / 32;
+constexpr int NK_U = 8;                       // 16-byte vectors (two points each) a thread and round
+constexpr uint32_t NK_NONE = 0x7f800001u;
+constexpr int NK_BATCH = 64;                  // warps whose threads are looked at together
+constexpr int NK_CAND = 1536;                 // candidates held: one pass adds at most 64 a warp
+constexpr int NK_MAX_WARPS = 5120;            // warps of the scan (the grid is bounded accordingly: 320 CTAs)
 
 struct __align__(16) PairSlot {
     int64_t i;
-    float d;
+    uint32_t d;
     uint32_t pad;
 };
 
-__device__ __forceinline__ bool pless(float da, int64_t ia, float db, int64_t ib) {
+// (distance bits, index) order
+__device__ __forceinline__ bool pless(uint32_t da, int64_t ia, uint32_t db, int64_t ib) {
     return da < db || (da == db && ia < ib);
 }
 
@@ -111,455 +135,290 @@ __device__ __forceinline__ float4 ld_pts(const float4 *p) {
     return v;
 }
 
-__device__ __forceinline__ float sqdist(float x, float y, float qx, float qy) {
+__device__ __forceinline__ uint32_t sqdist(float x, float y, float qx, float qy) {
     const float dx = __fsub_rn(x, qx), dy = __fsub_rn(y, qy);
-    return __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy));  // no fused multiply-add
+    return __float_as_uint(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)));  // no fused multiply-add
 }
 
-// One list per warp in shared memory, kept sorted in the (distance, index)
-// order; its first k entries are the warp's k smallest so far, and every
-// lane keeps the k-th (the threshold) in registers.  Entries past the k-th
-// never rise above it, so they never matter.  A lane's candidate that beats
-// the threshold is found by a ballot; such candidates (rare once the list
-// holds real points, or from the start under a bound) go through the
-// out-of-line slow path one at a time, lane 0 inserting into the shared list.
-struct Thr {
-    float d;
-    int64_t i;
+// The smallest (distance, index) pair of a warp, in every lane.
+__device__ __forceinline__ void warp_min_pair(uint32_t &d, int64_t &i) {
+    const uint32_t m = __reduce_min_sync(0xffffffffu, d);
+    uint64_t j = d == m ? (uint64_t)i : ~0ull >> 1;
+#pragma unroll
+    for (int s = 16; s >= 1; s >>= 1) {
+        const uint64_t o = __shfl_xor_sync(0xffffffffu, (unsigned long long)j, s);
+        j = o < j ? o : j;
+    }
+    d = m;
+    i = (int64_t)j;
+}
+
+struct NearestArgs {
+    const float *pts;
+    int64_t n;
+    float qx, qy;
+    int k;
+    int64_t *idx_out;
+    float *d_out;
+    uint32_t *tmin;     // [threads] each thread's smallest distance
+    PairSlot *wmin;     // [warps] each warp's nearest point
+    unsigned *counter;  // zero on entry and exit
 };
 
-template <int KT>
-__device__ __noinline__ Thr warp_insert_slow(float *LD, int64_t *LI, int k, float d, int64_t i, unsigned mask) {
-    const int lane = threadIdx.x & 31;
-    while (mask) {
-        const int src = __ffs(mask) - 1;
-        mask &= mask - 1;
-        const float cd = __shfl_sync(0xffffffffu, d, src);
-        const int64_t ci = (int64_t)__shfl_sync(0xffffffffu, (unsigned long long)i, src);
-        if (lane == 0 && pless(cd, ci, LD[k - 1], LI[k - 1])) {
-            int j = k - 1;
-            while (j > 0 && pless(cd, ci, LD[j - 1], LI[j - 1])) {
-                LD[j] = LD[j - 1];
-                LI[j] = LI[j - 1];
-                --j;
-            }
-            LD[j] = cd;
-            LI[j] = ci;
+struct NearestShared {
+    uint16_t warps[NK_MAX_WARPS];
+    uint32_t units[NK_BATCH * 32];
+    int64_t ci[NK_CAND];
+    uint32_t cd[NK_CAND];
+    int64_t gi[NK_WARPS];
+    uint32_t gd[NK_WARPS];
+    int nwarps, nunits, ncand;
+    int64_t bi;   // the bound
+    uint32_t bd;
+};
+
+__device__ __forceinline__ void nk_offer(NearestShared &s, bool ok, uint32_t d, int64_t i, uint32_t bd, int64_t bi) {
+    if (ok && d < NK_NONE && !pless(bd, bi, d, i)) {
+        const int at = atomicAdd(&s.ncand, 1);
+        if (ACCR_DCHECK(at < NK_CAND, DS_NEAREST_SLOT)) {
+            s.cd[at] = d;
+            s.ci[at] = i;
         }
-        __syncwarp();
     }
-    Thr t;
-    t.d = LD[k - 1];
-    t.i = LI[k - 1];
-    __syncwarp();
-    return t;
 }
 
-// The hot path is one compare: d <= the warp's k-th distance admits a
-// superset of the winners (ties included); the slow path applies the exact
-// (distance, index) order.
-template <int KT>
-__device__ __forceinline__ void warp_offer(float *LD, int64_t *LI, int k, Thr &thr, float d, int64_t i) {
-    const unsigned mask = __ballot_sync(0xffffffffu, d <= thr.d);
-    if (mask) thr = warp_insert_slow<KT>(LD, LI, k, d, i, mask);
+// Rank of candidate c among the first n (distinct points: no two are equal).
+__device__ __forceinline__ int nk_rank(const NearestShared &s, int c, int n) {
+    const uint32_t d = s.cd[c];
+    const int64_t i = s.ci[c];
+    int r = 0;
+    for (int o = 0; o < n; ++o) r += pless(s.cd[o], s.ci[o], d, i) ? 1 : 0;
+    return r;
 }
 
-// A distance bound B that at least k distinct points reach may stand in for
-// k placeholders (B, no index): every entry of the list at or past (B, no
-// index) becomes one (the prefix below it stays), so the list keeps the k
-// smallest of what it held and the placeholders.  Returns the new threshold.
-template <int KT>
-__device__ __noinline__ Thr warp_apply_bound(float *LD, int64_t *LI, int k, float B) {
-    if ((threadIdx.x & 31) == 0) {
+// The last CTA: the k nearest of all points, from the threads' nearest ones.
+__device__ __noinline__ void nearest_select(const NearestArgs &p, NearestShared &s) {
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int W = (int)gridDim.x * NK_WARPS;
+    const int64_t head = (((uintptr_t)p.pts & 15) != 0 && p.n > 0) ? 1 : 0;
+    const float4 *v4 = (const float4 *)(p.pts + 2 * head);
+    const int64_t npairs = (p.n - head) / 2, last = head + 2 * npairs;
+    const int64_t rstep = (int64_t)gridDim.x * NK_THREADS * NK_U;
+    // the bound: the k-th of the warps' shares (scan warp w belongs to warp w % 16
+    // here); all of a thread's loads in flight, and kept
+    constexpr int NW = NK_MAX_WARPS / NK_THREADS;
+    uint32_t wd[NW];
+    int64_t wi[NW];
+    uint32_t d = NK_NONE;
+    int64_t i = INT64_MAX;
 #pragma unroll
-        for (int j = 0; j < KT; ++j)
-            if (!pless(LD[j], LI[j], B, INT64_MAX)) {
-                LD[j] = B;
-                LI[j] = INT64_MAX;
-            }
+    for (int j = 0; j < NW; ++j) {
+        const int w = warp + NK_WARPS * lane + j * NK_THREADS;
+        const uint4 r = w < W ? __ldcg(reinterpret_cast<const uint4 *>(p.wmin + w)) : make_uint4(~0u, ~0u >> 1, NK_NONE, 0u);
+        wd[j] = r.z;
+        wi[j] = (int64_t)(((uint64_t)r.y << 32) | r.x);
     }
-    __syncwarp();
-    Thr t;
-    t.d = LD[k - 1];
-    t.i = LI[k - 1];
-    __syncwarp();
-    return t;
-}
-
-// The k-th smallest of one value per lane (k <= 32; every lane gets it).
-__device__ __forceinline__ float warp_kth_smallest(float v, int k) {
-    const int lane = threadIdx.x & 31;
-    float t = INFINITY;
-    for (int r = 0; r < k; ++r) {
-        float w = v;
 #pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) w = fminf(w, __shfl_xor_sync(0xffffffffu, w, o));
-        t = w;
-        const unsigned who = __ballot_sync(0xffffffffu, v == w);
-        if (lane == __ffs(who) - 1) v = INFINITY;  // exactly one lane gives up its value
-    }
-    return t;
-}
-
-// The CTA's KT smallest of its warps' lists (shared memory), written to
-// MD/MI: each entry's rank is the number of entries before it in the
-// (distance, index) order, equal entries (placeholders) ordered by position,
-// so the ranks are distinct and entry r of the result is the one of rank r.
-template <int KT, int NT>
-__device__ __forceinline__ void cta_merge_warp_lists(const float (*wld)[KT], const int64_t (*wli)[KT], float *MD,
-                                                     int64_t *MI) {
-    constexpr int NC = (NT / 32) * KT;
+    for (int j = 0; j < NW; ++j)
+        if (pless(wd[j], wi[j], d, i)) d = wd[j], i = wi[j];
+    warp_min_pair(d, i);
+    if (lane == 0) s.gd[warp] = d, s.gi[warp] = i;
+    if (t == 0) s.nwarps = 0, s.ncand = 0, s.bd = NK_NONE, s.bi = INT64_MAX;
     __syncthreads();
-    const float *fd = &wld[0][0];
-    const int64_t *fi = &wli[0][0];
-    for (int c = threadIdx.x; c < NC; c += NT) {
-        const float dc = fd[c];
-        const int64_t ic = fi[c];
-        int rank = 0;
-        for (int o = 0; o < NC; ++o) {
-            const float dd = fd[o];
-            const int64_t io = fi[o];
-            rank += (pless(dd, io, dc, ic) || (dd == dc && io == ic && o < c)) ? 1 : 0;
-        }
-        if (rank < KT) {
-            MD[rank] = dc;
-            MI[rank] = ic;
-        }
+    if (t < NK_WARPS) {  // k <= 16 shares; fewer with a point: no bound
+        const uint32_t gd = s.gd[t];
+        const int64_t gi = s.gi[t];
+        int r = 0;
+#pragma unroll
+        for (int o = 0; o < NK_WARPS; ++o) r += (pless(s.gd[o], s.gi[o], gd, gi)) ? 1 : 0;
+        if (gd < NK_NONE && r == p.k - 1) s.bd = gd, s.bi = gi;
     }
     __syncthreads();
-}
-
-// The sampled bound.  Every CTA of the scan launch takes NK_SAMPLE
-// consecutive points at blockIdx.x * sample_stride (so the sample spreads
-// over the whole array) and records its smallest distance; those minima
-// belong to distinct points, so the k-th smallest of them is a distance that
-// at least k points reach.  The last CTA to record its minimum selects it and
-// publishes it as one word (its bits + 1; zero means not yet).  Nobody waits
-// for it: each warp polls the word once per round and applies the bound when
-// it appears; until then its first round's own k-th smallest lane minimum
-// serves as a bound.
-constexpr int NK_SAMPLE = NK_THREADS;        // points sampled per CTA (one per thread)
-constexpr int64_t NK_BOUND_MIN_N = 1 << 22;  // smaller inputs skip the sampled bound
-
-template <int KT>
-__device__ __forceinline__ void flist_insert(float (&D)[KT], float d) {
-    if (!(d < D[KT - 1])) return;  // NaN never enters
 #pragma unroll
-    for (int j = KT - 1; j > 0; --j) D[j] = d < D[j - 1] ? D[j - 1] : (d < D[j] ? d : D[j]);
-    D[0] = d < D[0] ? d : D[0];
-}
-
-// The k-th smallest of cnt values (one warp; every lane gets it; k <= KT).
-template <int KT>
-__device__ __forceinline__ float kth_of_values(const float *v, int cnt, int k) {
-    const int lane = threadIdx.x & 31;
-    float D[KT];
-#pragma unroll
-    for (int j = 0; j < KT; ++j) D[j] = INFINITY;
-    for (int j0 = lane; j0 < cnt; j0 += 32 * 8) {
-        float mv[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) mv[u] = (j0 + 32 * u < cnt) ? __ldcg(v + j0 + 32 * u) : INFINITY;  // in flight together
-#pragma unroll
-        for (int u = 0; u < 8; ++u) flist_insert<KT>(D, mv[u]);
-    }
-    // k rounds of a warp minimum, each taking the head of exactly one lane
-    float t = INFINITY;
-    for (int r = 0; r < k; ++r) {
-        float w = D[0];
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) w = fminf(w, __shfl_xor_sync(0xffffffffu, w, o));
-        t = w;
-        const unsigned who = __ballot_sync(0xffffffffu, D[0] == w);
-        if (lane == __ffs(who) - 1) {
-#pragma unroll
-            for (int j = 0; j < KT - 1; ++j) D[j] = D[j + 1];
-            D[KT - 1] = INFINITY;
+    for (int j = 0; j < NW; ++j)
+        if (wd[j] < NK_NONE && !pless(s.bd, s.bi, wd[j], wi[j]))
+            s.warps[atomicAdd(&s.nwarps, 1)] = (uint16_t)(warp + NK_WARPS * lane + j * NK_THREADS);
+    __syncthreads();
+    const int nwarps = s.nwarps;
+    const int64_t rounds = npairs > 0 ? (npairs + rstep - 1) / rstep : 1;
+    const int64_t nvec = rounds * NK_U, chunks = (nvec + 31) / 32;  // a thread's vectors, 32 to a pass of a warp
+    for (int b0 = 0; b0 < nwarps; b0 += NK_BATCH) {
+        if (t == 0) s.nunits = 0;
+        __syncthreads();
+        for (int b = b0 + warp; b < nwarps && b < b0 + NK_BATCH; b += NK_WARPS) {
+            const uint32_t u = (uint32_t)s.warps[b] * 32u + lane;
+            const uint32_t du = __ldcg(p.tmin + u);
+            if (du < NK_NONE && du <= s.bd) s.units[atomicAdd(&s.nunits, 1)] = u;
+        }
+        __syncthreads();
+        const int64_t tasks = s.nunits * chunks;
+        for (int64_t t0 = 0; t0 < tasks; t0 += NK_WARPS) {
+            const int n = s.ncand;
+            __syncthreads();                       // every thread has the same count
+            if (n > NK_CAND - NK_WARPS * 68) {     // no room for a pass
+                for (int c = t; c < n; c += NK_THREADS) {
+                    const int r = nk_rank(s, c, n);
+                    if (r < p.k) s.gd[r] = s.cd[c], s.gi[r] = s.ci[c];
+                }
+                __syncthreads();
+                if (t < p.k) s.cd[t] = s.gd[t], s.ci[t] = s.gi[t];
+                if (t == 0) s.ncand = p.k, s.bd = s.gd[p.k - 1], s.bi = s.gi[p.k - 1];
+                __syncthreads();
+            }
+            const uint32_t bd = s.bd;
+            const int64_t bi = s.bi, task = t0 + warp;
+            if (task < tasks) {
+                const uint32_t u = s.units[task / chunks];
+                const int64_t j = (task % chunks) * 32 + lane;  // vector of the thread
+                const int64_t v = (int64_t)(u / NK_THREADS) * (NK_THREADS * NK_U) + (u % NK_THREADS) +
+                                  (j % NK_U) * NK_THREADS + (j / NK_U) * rstep;
+                const bool ok = j < nvec && v < npairs;
+                const float4 q = ok ? ld_pts(v4 + v) : make_float4(0.f, 0.f, 0.f, 0.f);
+                nk_offer(s, ok, sqdist(q.x, q.y, p.qx, p.qy), head + 2 * v, bd, bi);
+                nk_offer(s, ok, sqdist(q.z, q.w, p.qx, p.qy), head + 2 * v + 1, bd, bi);
+                if (j == 0 && u == 0 && head) nk_offer(s, true, sqdist(p.pts[0], p.pts[1], p.qx, p.qy), 0, bd, bi);
+                if (j == 0 && u == 1 && last < p.n)
+                    nk_offer(s, true, sqdist(p.pts[2 * last], p.pts[2 * last + 1], p.qx, p.qy), last, bd, bi);
+            }
+            __syncthreads();
         }
     }
-    return t;
+    const int n = s.ncand;
+    for (int c = t; c < n; c += NK_THREADS) {
+        const int r = nk_rank(s, c, n);
+        if (r < p.k && ACCR_DCHECK(p.k <= 16, DS_NEAREST_OUT)) {
+            p.idx_out[r] = s.ci[c];
+            p.d_out[r] = __uint_as_float(s.cd[c]);
+        }
+    }
+    if (t >= n && t < p.k) {  // fewer points than k
+        p.idx_out[t] = -1;
+        p.d_out[t] = INFINITY;
+    }
 }
 
-__device__ __forceinline__ unsigned ld_relaxed(const unsigned *p) {
-    unsigned v;
-    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// Last CTA: the k smallest of the G <= 2 NT CTA lists (each sorted) by k
-// rounds of a tournament over the lists' heads.  Thread t holds the heads of
-// lists t and t + NT and the entry after each (loaded ahead, so the winner of
-// a round seldom waits for its next entry); a round takes the CTA-wide
-// smallest (distance, index, list) and its list advances.
-constexpr int NK_MAX_GRID = 2 * NK_THREADS;  // CTA lists the tournament takes
-template <int KT, int NT>
-__device__ __noinline__ void final_tournament(const PairSlot *partials, int G, int k, float *MD, int64_t *MI) {
-    __shared__ float wd[2][NT / 32];
-    __shared__ int64_t wi[2][NT / 32];
-    __shared__ int wo[2][NT / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int NONE = 0x7fffffff;  // no list
-    auto slot = [&](int L, int j, float &d, int64_t &i) {
-        if (L < G && j < k) {
-            const uint4 r = __ldcg(reinterpret_cast<const uint4 *>(partials + (int64_t)L * KT + j));
-            d = __uint_as_float(r.z);
-            i = (int64_t)(((uint64_t)r.y << 32) | r.x);
-        } else {
-            d = INFINITY;
-            i = INT64_MAX;
+__global__ void __launch_bounds__(NK_THREADS, 2) nearest_kernel(const __grid_constant__ NearestArgs p) {
+    __shared__ NearestShared s;
+    __shared__ int am_last;
+    const int t = threadIdx.x, lane = t & 31;
+    // points are float2; the vector part starts at a 16-byte boundary
+    const int64_t head = (((uintptr_t)p.pts & 15) != 0 && p.n > 0) ? 1 : 0;
+    const float4 *v4 = (const float4 *)(p.pts + 2 * head);
+    const int64_t npairs = (p.n - head) / 2, last = head + 2 * npairs;
+    uint32_t bd = NK_NONE;
+    int64_t bi = INT64_MAX;
+    if (blockIdx.x == 0 && t == 0 && head) {  // the unaligned first point
+        const uint32_t d = sqdist(p.pts[0], p.pts[1], p.qx, p.qy);
+        if (d < bd) bd = d, bi = 0;
+    }
+    // A round's smallest distance first (one compare with the thread's); only a
+    // round that beats it looks for its first point with that distance.
+    int64_t v = (int64_t)blockIdx.x * (NK_THREADS * NK_U) + t;
+    const int64_t step = (int64_t)gridDim.x * (NK_THREADS * NK_U);
+    constexpr int H = NK_U / 2;
+    auto half = [&](const float4 (&q)[H], int64_t v0) {
+        uint32_t m = NK_NONE;
+#pragma unroll
+        for (int u = 0; u < H; ++u)
+            m = min(m, min(sqdist(q[u].x, q[u].y, p.qx, p.qy), sqdist(q[u].z, q[u].w, p.qx, p.qy)));
+        if (m < bd) {
+            bd = m;
+            int j = 0;
+#pragma unroll
+            for (int u = H - 1; u >= 0; --u) {
+                if (sqdist(q[u].z, q[u].w, p.qx, p.qy) == m) j = 2 * u + 1;
+                if (sqdist(q[u].x, q[u].y, p.qx, p.qy) == m) j = 2 * u;
+            }
+            bi = head + 2 * (v0 + (j >> 1) * NK_THREADS) + (j & 1);
         }
     };
-    const int L0 = threadIdx.x, L1 = threadIdx.x + NT;
-    float h0, n0, h1, n1;
-    int64_t g0, m0, g1, m1;
-    slot(L0, 0, h0, g0);
-    slot(L1, 0, h1, g1);
-    slot(L0, 1, n0, m0);
-    slot(L1, 1, n1, m1);
-    int p0 = 0, p1 = 0;
-    for (int r = 0; r < k; ++r) {
-        const bool second = pless(h1, g1, h0, g0);  // ties: the lower list
-        float d = second ? h1 : h0;
-        int64_t i = second ? g1 : g0;
-        int o = (second ? L1 : L0) < G ? (second ? L1 : L0) : NONE;
+    if (v + (NK_U - 1) * NK_THREADS < npairs) {  // full rounds, in halves: one is folded while the other loads
+        float4 a[H], b[H];
 #pragma unroll
-        for (int s = 16; s >= 1; s >>= 1) {
-            const float od = __shfl_xor_sync(0xffffffffu, d, s);
-            const int64_t oi = (int64_t)__shfl_xor_sync(0xffffffffu, (unsigned long long)i, s);
-            const int oo = __shfl_xor_sync(0xffffffffu, o, s);
-            if (pless(od, oi, d, i) || (od == d && oi == i && oo < o)) d = od, i = oi, o = oo;
-        }
-        if (lane == 0) wd[r & 1][warp] = d, wi[r & 1][warp] = i, wo[r & 1][warp] = o;
-        __syncthreads();
-        d = wd[r & 1][0], i = wi[r & 1][0], o = wo[r & 1][0];
+        for (int u = 0; u < H; ++u) a[u] = ld_pts(v4 + v + u * NK_THREADS);
 #pragma unroll
-        for (int w = 1; w < NT / 32; ++w) {
-            const float od = wd[r & 1][w];
-            const int64_t oi = wi[r & 1][w];
-            const int oo = wo[r & 1][w];
-            if (pless(od, oi, d, i) || (od == d && oi == i && oo < o)) d = od, i = oi, o = oo;
+        for (int u = 0; u < H; ++u) b[u] = ld_pts(v4 + v + (H + u) * NK_THREADS);
+        for (v += step; v + (NK_U - 1) * NK_THREADS < npairs; v += step) {
+            half(a, v - step);
+#pragma unroll
+            for (int u = 0; u < H; ++u) a[u] = ld_pts(v4 + v + u * NK_THREADS);
+            half(b, v - step + H * NK_THREADS);
+#pragma unroll
+            for (int u = 0; u < H; ++u) b[u] = ld_pts(v4 + v + (H + u) * NK_THREADS);
         }
-        if (threadIdx.x == 0) MD[r] = d, MI[r] = i;
-        if (o == L0) {  // the winner's list advances; the entry after the new head is loaded ahead
-            h0 = n0, g0 = m0, ++p0;
-            slot(L0, p0 + 1, n0, m0);
-        } else if (o == L1) {
-            h1 = n1, g1 = m1, ++p1;
-            slot(L1, p1 + 1, n1, m1);
+        half(a, v - step);
+        half(b, v - step + H * NK_THREADS);
+    }
+    if (v < npairs) {  // the last, partial round: loads in flight together
+        float4 q[NK_U];
+#pragma unroll
+        for (int u = 0; u < NK_U; ++u)
+            if (v + u * NK_THREADS < npairs) q[u] = ld_pts(v4 + v + u * NK_THREADS);
+#pragma unroll
+        for (int u = 0; u < NK_U; ++u) {
+            if (v + u * NK_THREADS < npairs) {
+                const uint32_t d0 = sqdist(q[u].x, q[u].y, p.qx, p.qy), d1 = sqdist(q[u].z, q[u].w, p.qx, p.qy);
+                const int64_t i = head + 2 * (v + u * NK_THREADS);
+                if (d0 < bd) bd = d0, bi = i;
+                if (d1 < bd) bd = d1, bi = i + 1;
+            }
         }
+    }
+    if (blockIdx.x == 0 && t == 1 && last < p.n) {  // the odd last point
+        const uint32_t d = sqdist(p.pts[2 * last], p.pts[2 * last + 1], p.qx, p.qy);
+        if (d < bd) bd = d, bi = last;
+    }
+    const int gt = (int)blockIdx.x * NK_THREADS + t;
+    p.tmin[gt] = bd;
+    warp_min_pair(bd, bi);
+    if (lane == 0) {
+        PairSlot w;
+        w.i = bi;
+        w.d = bd;
+        w.pad = 0;
+        p.wmin[gt >> 5] = w;
     }
     __syncthreads();
-}
-
-// With sample_stride > 0 every CTA samples, the last one publishes the
-// sampled bound in bstate[1], and warps pick it up as described above.
-// bstate[0] counts the CTAs that recorded their sample minimum; the last CTA
-// of the launch returns both words to zero.
-template <int KT, int NT>
-__global__ void __launch_bounds__(NT, 2) nearest_kernel(const float *__restrict__ pts, int64_t n, float qx, float qy,
-                                                     int k, int64_t *idx_out, float *d_out, PairSlot *partials,
-                                                     unsigned *counter, int64_t sample_stride, float *minima,
-                                                     unsigned *bstate) {
-    __shared__ float wld[NT / 32][KT];
-    __shared__ int64_t wli[NT / 32][KT];
-    __shared__ float MD[KT];
-    __shared__ int64_t MI[KT];
-    __shared__ float s_min[NT / 32];
-    __shared__ int am_last;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float *LD = wld[warp];
-    int64_t *LI = wli[warp];
-    if (lane < KT) {
-        LD[lane] = INFINITY;
-        LI[lane] = INT64_MAX;
-    }
-    __syncwarp();
-    Thr thr;
-    thr.d = INFINITY;
-    thr.i = INT64_MAX;
-    // points are float2; the vector part starts at a 16-byte boundary
-    const int64_t head = (((uintptr_t)pts & 15) != 0 && n > 0) ? 1 : 0;
-    const float4 *v4 = (const float4 *)(pts + 2 * head);
-    const int64_t npairs = (n - head) / 2;
-    const int64_t nth = (int64_t)gridDim.x * NT;
-    // Full rounds: NU 16-byte loads (2 points each) per lane, every one in
-    // range, so no per-point bounds test; the round's smallest distance is
-    // compared once with the warp's k-th, and only a round in which some lane
-    // beats it tests its points.  The trip count is uniform across each warp
-    // so that the votes see 32 lanes.
-    constexpr int NU = 16;
-    const int64_t vstep = nth * NU;
-    int64_t vb = (int64_t)blockIdx.x * (NT * NU) + warp * 32;
-    float4 q[NU];
-    bool full = vb + (NU - 1) * NT + 31 < npairs;  // uniform across the warp
-    if (full) {  // the first round's loads go out before the sample
-        const float4 *p = v4 + vb + lane;
-#pragma unroll
-        for (int u = 0; u < NU; ++u) q[u] = ld_pts(p + u * NT);
-    }
-    bool poll = false;
-    if (sample_stride > 0) {
-        const float2 sp = __ldg((const float2 *)pts + (int64_t)blockIdx.x * sample_stride + threadIdx.x);
-        float m = sqdist(sp.x, sp.y, qx, qy);
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (lane == 0) s_min[warp] = m;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            float cm = s_min[0];
-#pragma unroll
-            for (int w = 1; w < NT / 32; ++w) cm = fminf(cm, s_min[w]);  // fminf passes over NaN
-            minima[blockIdx.x] = cm;
-            __threadfence();
-            am_last = atomicAdd(&bstate[0], 1u) == gridDim.x - 1u;
-        }
-        __syncthreads();
-        if (am_last && warp == 0) {
-            __threadfence();
-            const float t = kth_of_values<KT>(minima, (int)gridDim.x, k);
-            if (lane == 0) st_release(&bstate[1], __float_as_uint(t) + 1u);  // t in [0, inf]: never wraps to 0
-        }
-        poll = true;
-    }
-    if (blockIdx.x == 0 && warp == 0) {  // the unaligned first point and the odd last point
-        const int64_t last = head + 2 * npairs;
-        float d = INFINITY;
-        int64_t i = INT64_MAX;
-        if (lane == 0 && head) d = sqdist(pts[0], pts[1], qx, qy), i = 0;
-        if (lane == 1 && last < n) d = sqdist(pts[2 * last], pts[2 * last + 1], qx, qy), i = last;
-        warp_offer<KT>(LD, LI, k, thr, d, i);
-    }
-    while (full) {
-        const unsigned pb = (poll && lane == 0) ? ld_relaxed(&bstate[1]) : 0u;  // the bound, if published
-        float dm = INFINITY;
-#pragma unroll
-        for (int u = 0; u < NU; ++u)
-            dm = fminf(dm, fminf(sqdist(q[u].x, q[u].y, qx, qy), sqdist(q[u].z, q[u].w, qx, qy)));
-        if (poll) {
-            const unsigned b = __shfl_sync(0xffffffffu, pb, 0);
-            if (b != 0u) {
-                const float B = __uint_as_float(b - 1u);
-                if (B < thr.d) thr = warp_apply_bound<KT>(LD, LI, k, B);
-                poll = false;
-            }
-        }
-        if (thr.d == INFINITY && k <= 32) {  // no bound yet: the k-th smallest lane minimum of this round
-            const float B = warp_kth_smallest(dm, k);   // k distinct points reach it
-            if (B < thr.d) thr = warp_apply_bound<KT>(LD, LI, k, B);
-        }
-        if (__any_sync(0xffffffffu, dm <= thr.d)) {
-            // the points of this lane that beat the threshold now (it only
-            // falls, so later winners are among them), then one pass over
-            // the positions some lane has, in order
-            unsigned bits = 0u;
-#pragma unroll
-            for (int j = 0; j < 2 * NU; ++j) {
-                const float4 &v = q[j >> 1];
-                const float dj = (j & 1) ? sqdist(v.z, v.w, qx, qy) : sqdist(v.x, v.y, qx, qy);
-                bits |= (dj <= thr.d ? 1u : 0u) << j;
-            }
-            const unsigned any = __reduce_or_sync(0xffffffffu, bits);
-            const int64_t ibase = head + 2 * (vb + lane);  // this lane's first point this round
-#pragma unroll
-            for (int j = 0; j < 2 * NU; ++j) {
-                if (any & (1u << j)) {  // uniform across the warp
-                    const float4 &v = q[j >> 1];
-                    const float dj = (j & 1) ? sqdist(v.z, v.w, qx, qy) : sqdist(v.x, v.y, qx, qy);
-                    const unsigned mask = __ballot_sync(0xffffffffu, ((bits >> j) & 1u) && dj <= thr.d);
-                    if (mask) thr = warp_insert_slow<KT>(LD, LI, k, dj, ibase + 2 * (j >> 1) * NT + (j & 1), mask);
-                }
-            }
-        }
-        vb += vstep;
-        full = vb + (NU - 1) * NT + 31 < npairs;
-        if (full) {
-            const float4 *p = v4 + vb + lane;
-#pragma unroll
-            for (int u = 0; u < NU; ++u) q[u] = ld_pts(p + u * NT);
-        }
-    }
-    if (vb < npairs) {  // the last, partial round: points past the end never compete
-        const int64_t ibase = head + 2 * (vb + lane);
-#pragma unroll
-        for (int u = 0; u < NU; ++u) {
-            const int64_t vv = vb + lane + u * NT;
-            const bool ok = vv < npairs;
-            const float4 v = ok ? ld_pts(v4 + vv) : make_float4(0.f, 0.f, 0.f, 0.f);
-            const float d0 = ok ? sqdist(v.x, v.y, qx, qy) : INFINITY;
-            const float d1 = ok ? sqdist(v.z, v.w, qx, qy) : INFINITY;
-            unsigned mask = __ballot_sync(0xffffffffu, ok && d0 <= thr.d);
-            if (mask) thr = warp_insert_slow<KT>(LD, LI, k, d0, ibase + 2 * u * NT, mask);
-            mask = __ballot_sync(0xffffffffu, ok && d1 <= thr.d);
-            if (mask) thr = warp_insert_slow<KT>(LD, LI, k, d1, ibase + 2 * u * NT + 1, mask);
-        }
-    }
-    cta_merge_warp_lists<KT, NT>(wld, wli, MD, MI);
-    const int G = gridDim.x;
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int j = 0; j < KT; ++j) {
-            PairSlot p;
-            p.i = MI[j];
-            p.d = MD[j];
-            p.pad = 0;
-            // the slots end where the sample's minima begin
-            if (ACCR_DCHECK((int64_t)blockIdx.x * KT + j < (int64_t)((const char *)minima - (const char *)partials) /
-                                                              (int64_t)sizeof(PairSlot),
-                            DS_NEAREST_SLOT))
-                partials[(int64_t)blockIdx.x * KT + j] = p;
-        }
+    if (t == 0) {
         __threadfence();
-        am_last = atomicAdd(counter, 1u) == (unsigned)G - 1u;
+        am_last = atomicAdd(p.counter, 1u) == gridDim.x - 1u;
     }
     __syncthreads();
     if (!am_last) return;
     __threadfence();
-    final_tournament<KT, NT>(partials, G, k, MD, MI);
-    if (threadIdx.x == 0) {
-        const int kk = ACCR_DCHECK(k >= 1 && k <= KT, DS_NEAREST_OUT) ? k : 0;  // the list holds KT entries
-        for (int j = 0; j < kk; ++j) {
-            const bool real = MI[j] != INT64_MAX;
-            idx_out[j] = real ? MI[j] : -1;
-            d_out[j] = real ? MD[j] : INFINITY;
-        }
-        *counter = 0u;
-        if (sample_stride > 0) {  // every CTA has recorded its minimum and stopped polling
-            bstate[0] = 0u;
-            bstate[1] = 0u;
-        }
-    }
+    nearest_select(p, s);
+    if (t == 0) *p.counter = 0u;
 }
 
-template <int KT>
 static int nearest_launch(const float *pts, int64_t n, float qx, float qy, int k, int64_t *idx, float *d,
                           cudaStream_t s) {
-    constexpr int NT = NK_THREADS;
     static int per_sm = 0;
     static std::once_flag once;
     std::call_once(once, [] {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, nearest_kernel<KT, NT>, NT, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, nearest_kernel, NK_THREADS, 0);
         if (per_sm < 1) per_sm = 1;
     });
     const DeviceInfo &di = device_info();
-    const int64_t want = (n / 2 + NT * 16 - 1) / (NT * 16);  // one round of 16 vectors per thread
-    const int64_t resident = std::min<int64_t>((int64_t)per_sm * di.sms, NK_MAX_GRID);
+    const int64_t want = (n / 2 + NK_THREADS * NK_U - 1) / (NK_THREADS * NK_U);  // one round a thread
+    const int64_t resident = std::min<int64_t>((int64_t)per_sm * di.sms, NK_MAX_WARPS / NK_WARPS);
     const int grid = (int)std::min<int64_t>(std::max<int64_t>(want, 1), resident);
-    // a sample of NK_SAMPLE points per CTA, spread over the array
-    const bool use_bound = n >= NK_BOUND_MIN_N && grid >= 32 && n / grid >= NK_SAMPLE;
-    // scratch: [partials: grid * KT slots][the CTAs' sample minima]
-    const size_t part_bytes = sizeof(PairSlot) * (size_t)grid * KT;
-    const size_t minima_off = (part_bytes + 255) & ~(size_t)255;
-    Scratch *scr = scratch_for((accr_stream_t)s, minima_off + sizeof(float) * (size_t)grid);
+    NearestArgs a;
+    a.pts = pts;
+    a.n = n;
+    a.qx = qx;
+    a.qy = qy;
+    a.k = k;
+    a.idx_out = idx;
+    a.d_out = d;
+    const size_t tbytes = sizeof(uint32_t) * (size_t)grid * NK_THREADS;
+    Scratch *scr = scratch_for((accr_stream_t)s, tbytes + sizeof(PairSlot) * (size_t)grid * NK_WARPS);
     if (!scr) return ACCR_ENOMEM;
-    PairSlot *partials = (PairSlot *)scr->buf;
-    unsigned *counter = scr->counters + 1;
-    unsigned *bstate = scr->counters + 5;  // words 5-6
-    float *minima = (float *)((char *)scr->buf + minima_off);
-    const int64_t stride = use_bound ? n / grid : 0;
+    a.tmin = (uint32_t *)scr->buf;
+    a.wmin = (PairSlot *)((char *)scr->buf + tbytes);
+    a.counter = scr->counters + 1;
     int rc = launch_guard("nearest_kernel");
     if (rc != ACCR_OK) return rc;
-    // no CTA waits for another: a plain launch
-    nearest_kernel<KT, NT><<<grid, NT, 0, s>>>(pts, n, qx, qy, k, idx, d, partials, counter, stride, minima, bstate);
+    nearest_kernel<<<grid, NK_THREADS, 0, s>>>(a);
     return launched("nearest_kernel");
 }
 
@@ -1221,8 +1080,7 @@ extern "C" ACCR_API int accr_nearest_k(const float *pts, int64_t n, float qx, fl
     if (((uintptr_t)pts & 7) || ((uintptr_t)idx_out & 7) || ((uintptr_t)d2_out & 3))
         return set_error(ACCR_EINVAL, "accr_nearest_k: misaligned pointer (points need 8 bytes)");
     cudaStream_t s = (cudaStream_t)stream;
-    int rc = k <= 8 ? nearest_launch<8>(pts, n, qx, qy, k, idx_out, d2_out, s)
-                    : nearest_launch<16>(pts, n, qx, qy, k, idx_out, d2_out, s);
+    int rc = nearest_launch(pts, n, qx, qy, k, idx_out, d2_out, s);
     if (rc != ACCR_OK) return rc;
     if (flags & ACCR_SYNC) return cuda_check(cudaStreamSynchronize(s), "accr_nearest_k: sync");
     return ACCR_OK;
