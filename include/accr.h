@@ -307,8 +307,8 @@ ACCR_API int accr_nearest_k(const float *pts, int64_t n, float qx, float qy,
  * sums, merged in double), then y_i = (x_i - (float)mean) * (float)(1/sqrt(var))
  * (y may alias x).  stats receives {mean, var} (DEVICE double[2]).
  *
- * Default: one cooperative launch -- the last CTA of the reduction publishes
- * the statistics and every CTA waits for them (bounded) before the
+ * Default: one cooperative launch -- every CTA passes a bounded grid barrier
+ * after its part of the reduction, merges the parts' results and runs the
  * elementwise pass.  ACCR_UNFUSED: two launches, statistics kept on the
  * device.  ACCR_TWO_LEVEL_HOST: the paper's form (partials merged on the
  * host, then the elementwise launch; synchronous).

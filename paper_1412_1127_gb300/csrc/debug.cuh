@@ -22,8 +22,8 @@ enum DebugSite : unsigned {
     DS_BATCH_TILE = 5,     // batch: tile of a region < the region's tiles
     DS_BATCH_SLOT = 6,     // batch: partial slot < all tiles' slots
     DS_BATCH_REGION = 7,   // batch: region index < descriptors
-    DS_NEAREST_SLOT = 8,   // k-nearest: partial slot < CTAs x list length
-    DS_NEAREST_OUT = 9,    // k-nearest: output index < k
+    DS_NEAREST_SLOT = 8,   // k-nearest: candidate slot < candidates held
+    DS_NEAREST_OUT = 9,    // k-nearest: k within the candidates' lists
     DS_GEMM_STORE = 10,    // BF16x3 epilogue: row < M and columns < N
 };
 

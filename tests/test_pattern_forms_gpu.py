@@ -53,6 +53,28 @@ def test_nearest_k_adversarial(kind, k):
     check_nearest(pts, 50.0, 50.0, k, kind)
 
 
+KEPT = 8 * 4 * 1024  # elements a CTA of the fused form keeps in registers
+
+
+@pytest.mark.parametrize("n", [2, 3, 4, 4095, 4097, KEPT + 1, 152 * KEPT - 5, 152 * KEPT + 4099, 12345677])
+@pytest.mark.parametrize("off", [0, 1])
+@pytest.mark.parametrize("in_place", [False, True])
+def test_standardize_fused_forms(n, off, in_place):
+    x = (inputs.normal(n, np.float32, salt=n % 13) * 3 + 5).astype(np.float32)
+    xt = torch.from_numpy(np.concatenate([np.zeros(off, np.float32), x])).cuda()[off:]
+    gy, gst = guarded((n,), torch.float32, float("nan")), guarded((2,), torch.float64, float("nan"))
+    y = gy.t
+    if in_place:
+        gy.t.copy_(xt)
+        xt = gy.t
+    api.accr_standardize(xt, y, gst.t, flags=api.ACCR_SYNC)
+    wy, (wm, wv) = oracle.standardize(x)
+    mean, var = gst.check("stats").cpu().numpy()
+    assert abs(mean - wm) <= 1e-9 * max(abs(wm), 1.0) and abs(var - wv) <= 1e-9 * wv
+    got = gy.check("y").cpu().numpy()
+    assert np.max(np.abs(got - wy) / np.maximum(np.abs(wy), 1.0)) <= 4e-6
+
+
 @pytest.mark.parametrize("shape,p", [((64, 1024), 0.7), ((65, 40), 0.7), ((64, 1025), 0.8), ((63, 3000), 0.75),
                                      ((129, 1), 1.0), ((4000, 33), 0.8), ((500, 1100), 0.62), ((2000, 2000), 0.7),
                                      ((31, 31), 0.0), ((1, 5000), 1.0), ((6000, 64), 0.9)])
