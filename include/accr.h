@@ -239,8 +239,11 @@ ACCR_API int accr_batch_reduce(const accr_region *regions, int64_t nregions,
  * accr_segmented_reduce -- regions that share one element array, element type
  * and clause list: segment s is values[offsets[s] .. offsets[s+1]).  Each
  * clause's `out` is a DEVICE array of nseg variables; `init` (if any) is the
- * prior value of every segment's variable.  Same device path as
- * accr_batch_reduce.
+ * prior value of every segment's variable.  The offsets are checked on the host
+ * and uploaded; one launch folds segments of at most 4 KiB in groups of lanes
+ * and longer ones, up to the warp-region limit of accr_batch_tiling, a warp
+ * each; longer ones still run as tiles of a batched launch.  A segment's form
+ * depends on its own type and length only.
  *
  *   values    DEVICE array of in_type
  *   offsets   HOST array of nseg+1 non-decreasing element offsets (loop bounds

@@ -596,28 +596,24 @@ struct RegionSource {
     }
 };
 
-// Segments [off[s], off[s+1]) of one array, one variable per segment.
+// Listed segments [off[s], off[s+1]) of one array, one variable per segment (the
+// offsets were checked by the caller).
 struct SegmentSource {
     const void *values;
     const int64_t *off;
+    const int32_t *idx;
     int in_type, nc;
     int64_t eb;
     const ClauseDev *base;  // lowered clauses; out = the arrays' starts
     int ndesc(int64_t) const { return nc > RD_CLAUSES ? 2 : 1; }
-    int fill(int64_t s, RegionDev *out, ClauseMemo &) const {
-        const int64_t lo = off[s], hi = off[s + 1];
-        if (lo < 0 || hi < lo)
-            return set_error(ACCR_EINVAL, "segmented: offsets not non-decreasing at %lld", (long long)s);
-        const void *in = (const char *)values + lo * eb;
-        int rc = check_region_ptr(in, hi - lo, in_type, s);
-        if (rc != ACCR_OK) return rc;
-        if (hi > lo && !values) return set_error(ACCR_EINVAL, "segmented: values is NULL");
+    int fill(int64_t i, RegionDev *out, ClauseMemo &) const {
+        const int64_t s = idx[i], lo = off[s], hi = off[s + 1];
         ClauseDev cl[ACCR_MAX_CLAUSES];
         for (int c = 0; c < nc; ++c) {
             cl[c] = base[c];
             cl[c].out = (char *)base[c].out + s * type_bytes(base[c].acc_type);
         }
-        RegionSource::put(out, in, hi - lo, in_type, cl, nc);
+        RegionSource::put(out, (const char *)values + lo * eb, hi - lo, in_type, cl, nc);
         return ACCR_OK;
     }
 };
@@ -758,17 +754,6 @@ static int plan_from_regions(const accr_region *regs, int64_t R, HostPlan &P) {
     return plan_chunked(src, R, P);
 }
 
-static int plan_from_segments(const void *values, const int64_t *off, int64_t nseg, int in_type,
-                              const accr_clause *clauses, int nc, unsigned flags, HostPlan &P) {
-    if (nseg < 0 || (nseg > 0 && !off)) return set_error(ACCR_EINVAL, "segmented: bad offsets");
-    if (nseg > INT32_MAX / 2) return set_error(ACCR_EINVAL, "segmented: too many segments");
-    ClauseDev base[ACCR_MAX_CLAUSES];
-    int rc = lower_clauses(in_type, clauses, nc, flags & ACCR_COMPENSATED, base);
-    if (rc != ACCR_OK) return rc;
-    SegmentSource src{values, off, in_type, nc, (int64_t)type_bytes(in_type), base};
-    return plan_chunked(src, nseg, P);
-}
-
 static int batch_grid(const HostPlan &P) {
     static std::mutex mu;
     static int cached[64] = {0};
@@ -834,6 +819,74 @@ static StreamBufs *bufs_for(accr_stream_t stream) {
     return b;
 }
 
+// Device memory of at least `bytes` for a plan and `words` counters (zero when no
+// kernel uses them).  Growing synchronises the stream.
+static int grow(StreamBufs *B, size_t bytes, size_t words, cudaStream_t s) {
+    if (B->dev_bytes >= bytes && B->ncounters >= words) return ACCR_OK;
+    if (fault_take(ACCR_FAULT_ALLOC)) return set_error(ACCR_ENOMEM, "batch: injected allocation failure");
+    int rc = cuda_check(cudaStreamSynchronize(s), "batch: grow sync");
+    if (rc != ACCR_OK) return rc;
+    if (B->dev_bytes < bytes) {
+        if (B->dev) cudaFree(B->dev);
+        B->dev = nullptr;
+        B->dev_bytes = 0;
+        const size_t want = std::max(bytes, (size_t)1 << 20);
+        if (cudaMalloc(&B->dev, want) != cudaSuccess) {
+            cudaGetLastError();
+            return set_error(ACCR_ENOMEM, "batch: cudaMalloc of %zu bytes failed", want);
+        }
+        B->dev_bytes = want;
+    }
+    if (B->ncounters < words) {
+        if (B->counters) cudaFree(B->counters);
+        B->counters = nullptr;
+        B->ncounters = 0;
+        const size_t want = std::max(words, (size_t)65536);
+        if (cudaMalloc(&B->counters, want * 4) != cudaSuccess) {
+            cudaGetLastError();
+            return set_error(ACCR_ENOMEM, "batch: cudaMalloc of counters failed");
+        }
+        rc = cuda_check(cudaMemset(B->counters, 0, want * 4), "batch: clear counters");
+        if (rc != ACCR_OK) return rc;
+        B->ncounters = want;
+    }
+    return ACCR_OK;
+}
+
+// The next pinned staging buffer (double-buffered: waits until the copy that last
+// used it is done), of at least `bytes`.
+static int next_stage(StreamBufs *B, size_t bytes, int *slot) {
+    const int i = B->next;
+    B->next ^= 1;
+    if (!B->stage_done[i]) {
+        int rc = cuda_check(cudaEventCreateWithFlags(&B->stage_done[i], cudaEventDisableTiming), "batch: event");
+        if (rc != ACCR_OK) return rc;
+    } else {
+        int rc = cuda_check(cudaEventSynchronize(B->stage_done[i]), "batch: staging wait");
+        if (rc != ACCR_OK) return rc;
+    }
+    if (B->stage_bytes[i] < bytes) {
+        if (B->stage[i]) cudaFreeHost(B->stage[i]);
+        B->stage[i] = nullptr;
+        B->stage_bytes[i] = 0;
+        const size_t want = std::max(bytes, (size_t)1 << 20);
+        if (cudaMallocHost(&B->stage[i], want) != cudaSuccess) {
+            cudaGetLastError();
+            return set_error(ACCR_ENOMEM, "batch: cudaMallocHost of %zu bytes failed", want);
+        }
+        B->stage_bytes[i] = want;
+    }
+    *slot = i;
+    return ACCR_OK;
+}
+
+// Uploads a staging buffer's first `bytes` to the stream's device memory.
+static int send_stage(StreamBufs *B, int i, size_t bytes, cudaStream_t s) {
+    int rc = cuda_check(cudaMemcpyAsync(B->dev, B->stage[i], bytes, cudaMemcpyHostToDevice, s), "batch: plan upload");
+    if (rc != ACCR_OK) return rc;
+    return cuda_check(cudaEventRecord(B->stage_done[i], s), "batch: event record");
+}
+
 static int run_once(HostPlan &P, unsigned flags, accr_stream_t stream) {
     cudaStream_t s = (cudaStream_t)stream;
     const size_t R = P.regions.size();
@@ -842,37 +895,8 @@ static int run_once(HostPlan &P, unsigned flags, accr_stream_t stream) {
             (long long)P.tile_bytes, P.small.size());
     StreamBufs *B = bufs_for(stream);
     std::lock_guard<std::mutex> lk(B->mu);
-    // device plan + partials
-    if ((B->dev_bytes < P.total_bytes || B->ncounters < R + 4) && fault_take(ACCR_FAULT_ALLOC))
-        return set_error(ACCR_ENOMEM, "batch: injected allocation failure");
-    if (B->dev_bytes < P.total_bytes || B->ncounters < R + 4) {
-        int rc = cuda_check(cudaStreamSynchronize(s), "batch: grow sync");
-        if (rc != ACCR_OK) return rc;
-        if (B->dev_bytes < P.total_bytes) {
-            if (B->dev) cudaFree(B->dev);
-            B->dev = nullptr;
-            B->dev_bytes = 0;
-            size_t want = std::max(P.total_bytes, (size_t)1 << 20);
-            if (cudaMalloc(&B->dev, want) != cudaSuccess) {
-                cudaGetLastError();
-                return set_error(ACCR_ENOMEM, "batch: cudaMalloc of %zu bytes failed", want);
-            }
-            B->dev_bytes = want;
-        }
-        if (B->ncounters < R + 4) {
-            if (B->counters) cudaFree(B->counters);
-            B->counters = nullptr;
-            B->ncounters = 0;
-            size_t want = std::max(R + 4, (size_t)65536);
-            if (cudaMalloc(&B->counters, want * 4) != cudaSuccess) {
-                cudaGetLastError();
-                return set_error(ACCR_ENOMEM, "batch: cudaMalloc of counters failed");
-            }
-            rc = cuda_check(cudaMemset(B->counters, 0, want * 4), "batch: clear counters");
-            if (rc != ACCR_OK) return rc;
-            B->ncounters = want;
-        }
-    }
+    int rc = grow(B, P.total_bytes, R + 4, s);  // device plan + partials
+    if (rc != ACCR_OK) return rc;
     if (R <= (size_t)INL_REGIONS && P.tiles.size() <= (size_t)INL_TILES && P.small.size() <= (size_t)INL_SMALL) {
         static BatchArgsInline ai;  // built under B->mu; launched by value
         static std::mutex inl_mu;
@@ -885,7 +909,7 @@ static int run_once(HostPlan &P, unsigned flags, accr_stream_t stream) {
         std::copy(P.regions.begin(), P.regions.end(), ai.regions);
         std::copy(P.tiles.begin(), P.tiles.end(), ai.tiles);
         std::copy(P.small.begin(), P.small.end(), ai.small);
-        int rc = launch_guard("batch_kernel");
+        rc = launch_guard("batch_kernel");
         if (rc != ACCR_OK) return rc;
         batch_kernel_inline<<<batch_grid(P), BB, 0, s>>>(ai);
         rc = launched("batch_kernel");
@@ -893,33 +917,10 @@ static int run_once(HostPlan &P, unsigned flags, accr_stream_t stream) {
         if (flags & ACCR_SYNC) return cuda_check(cudaStreamSynchronize(s), "batch: sync");
         return ACCR_OK;
     }
-    // pinned staging (double-buffered; wait until the copy that last used it is done)
-    const int i = B->next;
-    B->next ^= 1;
-    if (!B->stage_done[i]) {
-        int rc = cuda_check(cudaEventCreateWithFlags(&B->stage_done[i], cudaEventDisableTiming), "batch: event");
-        if (rc != ACCR_OK) return rc;
-    } else {
-        int rc = cuda_check(cudaEventSynchronize(B->stage_done[i]), "batch: staging wait");
-        if (rc != ACCR_OK) return rc;
-    }
-    if (B->stage_bytes[i] < P.plan_bytes) {
-        if (B->stage[i]) cudaFreeHost(B->stage[i]);
-        B->stage[i] = nullptr;
-        B->stage_bytes[i] = 0;
-        size_t want = std::max(P.plan_bytes, (size_t)1 << 20);
-        if (cudaMallocHost(&B->stage[i], want) != cudaSuccess) {
-            cudaGetLastError();
-            return set_error(ACCR_ENOMEM, "batch: cudaMallocHost of %zu bytes failed", want);
-        }
-        B->stage_bytes[i] = want;
-    }
+    int i = 0;
+    if ((rc = next_stage(B, P.plan_bytes, &i)) != ACCR_OK) return rc;
     write_plan(P, B->stage[i]);
-    int rc = cuda_check(cudaMemcpyAsync(B->dev, B->stage[i], P.plan_bytes, cudaMemcpyHostToDevice, s),
-                        "batch: plan upload");
-    if (rc != ACCR_OK) return rc;
-    rc = cuda_check(cudaEventRecord(B->stage_done[i], s), "batch: event record");
-    if (rc != ACCR_OK) return rc;
+    if ((rc = send_stage(B, i, P.plan_bytes, s)) != ACCR_OK) return rc;
     BatchArgs a = args_for(P, B->dev, B->counters);
     if ((rc = launch_guard("batch_kernel")) != ACCR_OK) return rc;
     batch_kernel<<<batch_grid(P), BB, 0, s>>>(a);
@@ -934,6 +935,35 @@ int batch_launch_regions(const accr_region *regions, int64_t nregions, accr_stre
     int rc = plan_from_regions(regions, nregions, P);
     if (rc != ACCR_OK) return rc;
     return run_once(P, 0, stream);
+}
+
+int batch_launch_segments(const void *values, const int64_t *off, const int32_t *idx, int64_t n, int in_type,
+                          const ClauseDev *cl, int nc, accr_stream_t stream) {
+    HostPlan &P = thread_plan(0);
+    SegmentSource src{values, off, idx, in_type, nc, (int64_t)type_bytes(in_type), cl};
+    int rc = plan_chunked(src, n, P);
+    if (rc != ACCR_OK) return rc;
+    return run_once(P, 0, stream);
+}
+
+int64_t batch_small_bytes() { return g_small_bytes.load(); }
+
+int PlanStage::begin(accr_stream_t stream, size_t bytes) {
+    bufs = bufs_for(stream);
+    bufs->mu.lock();
+    int rc = grow(bufs, bytes, 0, (cudaStream_t)stream);
+    if (rc == ACCR_OK) rc = next_stage(bufs, bytes, &slot);
+    if (rc != ACCR_OK) return rc;
+    host = bufs->stage[slot];
+    dev = bufs->dev;
+    return ACCR_OK;
+}
+
+int PlanStage::upload(size_t bytes, cudaStream_t s) { return send_stage(bufs, slot, bytes, s); }
+
+void PlanStage::end() {
+    if (bufs) bufs->mu.unlock();
+    bufs = nullptr;
 }
 
 }  // namespace accr
@@ -983,19 +1013,6 @@ extern "C" ACCR_API int accr_batch_reduce(const accr_region *regions, int64_t nr
     if (flags & ACCR_PLAIN) return run_plain(regions, nregions, flags, stream);
     HostPlan &P = thread_plan(0);
     int rc = plan_from_regions(regions, nregions, P);
-    if (rc != ACCR_OK) return rc;
-    return run_once(P, flags, stream);
-}
-
-extern "C" ACCR_API int accr_segmented_reduce(const void *values, const int64_t *offsets, int64_t nseg,
-                                              int32_t in_type, const accr_clause *clauses, int32_t nclauses,
-                                              uint32_t flags, accr_stream_t stream) {
-    ACCR_TRACE("accr_segmented_reduce");
-    clear_error();
-    if (flags & ~(ACCR_SYNC | ACCR_COMPENSATED))
-        return set_error(ACCR_EINVAL, "accr_segmented_reduce: unsupported flags 0x%x", flags);
-    HostPlan &P = thread_plan(0);
-    int rc = plan_from_segments(values, offsets, nseg, in_type, clauses, nclauses, flags, P);
     if (rc != ACCR_OK) return rc;
     return run_once(P, flags, stream);
 }
