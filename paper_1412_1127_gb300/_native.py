@@ -55,12 +55,12 @@ class Result(ctypes.Structure):
 # Every symbol include/accr.h declares, with its ctypes signature.
 _vp, _i32, _i64, _u32, _u64 = (ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64,
                                ctypes.c_uint32, ctypes.c_uint64)
-_CP = ctypes.POINTER(Clause)
+_CP = _vp  # accr_clause array: packed bytes (the binding's) or a ctypes array of Clause
 SIGNATURES = {
     "accr_reduce": (ctypes.c_int, [_vp, _i64, _i32, _CP, _i32, _u32, _vp]),
     "accr_rowreduce": (ctypes.c_int, [_vp, _i64, _i64, _i64, _i32, _CP, _i32, _u32, _vp]),
     "accr_batch_reduce": (ctypes.c_int, [ctypes.POINTER(Region), _i64, _u32, _vp]),
-    "accr_segmented_reduce": (ctypes.c_int, [_vp, ctypes.POINTER(_i64), _i64, _i32, _CP, _i32, _u32, _vp]),
+    "accr_segmented_reduce": (ctypes.c_int, [_vp, _vp, _i64, _i32, _CP, _i32, _u32, _vp]),
     "accr_batch_create": (ctypes.c_int, [ctypes.POINTER(Region), _i64, _u32, ctypes.POINTER(_vp)]),
     "accr_batch_launch": (ctypes.c_int, [_vp, _vp]),
     "accr_batch_destroy": (ctypes.c_int, [_vp]),
