@@ -875,11 +875,12 @@ __global__ void __launch_bounds__(BFP_THREADS, 1) bfs_persistent_kernel(const ui
 //     d away, so `depth` levels run on the tile's own copy and leave its
 //     interior exact; then the interior goes back to the bitmaps (two copies,
 //     read and written in turn), one grid barrier carries the `||` of "a
-//     frontier is left", and the tiles load again.
+//     frontier is left", and the tiles load again.  (Within those levels the halo's
+//     far rows stop mattering one by one, and their warps only keep the barrier.)
 //
 // With one tile the loop runs to the end without grid barriers.  1024 x 1024
-// cells, 62 % open, about 1,260 levels: 6.2 ms in the cell-wise form, 0.63 ms here
-// (0.33 us a level, and 4 us a step of 28 levels for loading, storing and the
+// cells, 62 % open, about 1,260 levels: 6.2 ms in the cell-wise form, 0.60 ms here
+// (0.31 us a level, and 4 us a step of 28 levels for loading, storing and the
 // barrier; what is left is the chain of a level's instructions and its CTA barrier).
 constexpr int BT_R = 4;                     // rows per thread
 constexpr int BT_THREADS = 512;             // 16 warps: 64 rows a tile
@@ -963,6 +964,8 @@ __global__ void __launch_bounds__(BT_THREADS, 1) bfs_tile_kernel(const __grid_co
                 a[j] = in ? __ldcg(fin + (int64_t)r * p.wpr + word) : 0u;
                 f[j] = in ? __ldcg(rin + (int64_t)r * p.wpr + word) : 0u;
             }
+            const int wr0 = top + warp * BT_R;                   // this warp's first row
+            const bool owns = wr0 < r1 && wr0 + BT_R > r0;       // the same for the warp
             bool more = true;
             int base = L;
             do {
@@ -989,7 +992,10 @@ __global__ void __launch_bounds__(BT_THREADS, 1) bfs_tile_kernel(const __grid_co
                     }
                     uint32_t above = warp > 0 ? edge[d & 1][warp - 1][1][lane] : 0u;
                     const uint32_t below = warp + 1 < NW ? edge[d & 1][warp + 1][0][lane] : 0u;
-                    if (!__any_sync(0xffffffffu, (any | above | below) != 0u)) continue;  // nothing near this warp's rows
+                    // Rows further than the levels left from the interior can no longer
+                    // reach it, and rows with nothing near them do not change.
+                    if (wr0 >= r1 + (run - d) || wr0 + BT_R <= r0 - (run - d)) continue;
+                    if (!__any_sync(0xffffffffu, (any | above | below) != 0u)) continue;
 #pragma unroll
                     for (int j = 0; j < BT_R; ++j) {
                         uint32_t lw = __shfl_up_sync(0xffffffffu, f[j], 1), rw = __shfl_down_sync(0xffffffffu, f[j], 1);
@@ -1003,7 +1009,7 @@ __global__ void __launch_bounds__(BT_THREADS, 1) bfs_tile_kernel(const __grid_co
                     }
 #pragma unroll
                     for (int i = 0; i < 5; ++i) {
-                        if ((d >> i) & 1) {
+                        if (owns && ((d >> i) & 1)) {
 #pragma unroll
                             for (int j = 0; j < BT_R; ++j) pl[i][j] |= f[j];
                         }
