@@ -108,7 +108,6 @@ template <typename T, int NC>
 __device__ __noinline__ void tile_fold(const BatchArgs &p, const RegionDev *d, int r, int64_t k,
                                           Acc (*sh)[BB / 32], int *s_last) {
     constexpr bool E64 = sizeof(T) == 8;
-    constexpr int EPV = 16 / (int)sizeof(T);
     const int64_t TE = p.tile_bytes / (int64_t)sizeof(T);
     const int64_t n = d->n;
     const int64_t tile0 = d->tile0;
@@ -129,38 +128,7 @@ __device__ __noinline__ void tile_fold(const BatchArgs &p, const RegionDev *d, i
         A[c].a = id[c];
         A[c].c = 0.f;
     }
-    const int64_t mis = (int64_t)(((16 - ((uintptr_t)in & 15)) & 15) / sizeof(T));
-    const int64_t head = mis < len ? mis : len;
-    const uint4 *vin = (const uint4 *)(in + head);
-    const int64_t nvec = (len - head) / EPV;
-    const int64_t tail0 = head + nvec * EPV;
-    if (threadIdx.x < head) {
-        T x = in[threadIdx.x];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) fold_one<T>(w[c], A[c], x);
-    }
-    if (tail0 + threadIdx.x < len) {
-        T x = in[tail0 + threadIdx.x];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) fold_one<T>(w[c], A[c], x);
-    }
-    int64_t v = threadIdx.x;
-    for (; v + (BU - 1) * BB < nvec; v += BB * BU) {
-        uint4 b[BU];
-#pragma unroll
-        for (int u = 0; u < BU; ++u) b[u] = ld_batch(vin + v + u * BB);
-#pragma unroll
-        for (int c = 0; c < NC; ++c) fold_vec<T, BU>(w[c], A[c], b);
-    }
-#pragma unroll
-    for (int u = 0; u < BU; ++u) {
-        const int64_t vv = v + u * BB;
-        if (vv < nvec) {
-            uint4 b = ld_batch(vin + vv);
-#pragma unroll
-            for (int c = 0; c < NC; ++c) fold_vec<T, 1>(w[c], A[c], &b);
-        }
-    }
+    stream_fold<T, NC, BU, BB>(in, len, (int)threadIdx.x, w, A, ld_batch);
     cta_merge<NC, BB>(w, id, E64, A, sh);
 
     if (ntiles == 1) {
@@ -218,7 +186,6 @@ __device__ __noinline__ void tile_fold(const BatchArgs &p, const RegionDev *d, i
 template <typename T, int NC>
 __device__ __noinline__ void warp_fold(const RegionDev *d, int lane) {
     constexpr bool E64 = sizeof(T) == 8;
-    constexpr int EPV = 16 / (int)sizeof(T);
     const int64_t n = d->n;
     const T *in = (const T *)d->in;
     int w[NC];
@@ -229,38 +196,7 @@ __device__ __noinline__ void warp_fold(const RegionDev *d, int lane) {
         A[c].a = d->cl[c].ident;
         A[c].c = 0.f;
     }
-    const int64_t mis = (int64_t)(((16 - ((uintptr_t)in & 15)) & 15) / sizeof(T));
-    const int64_t head = mis < n ? mis : n;
-    const uint4 *vin = (const uint4 *)(in + head);
-    const int64_t nvec = (n - head) / EPV;
-    const int64_t tail0 = head + nvec * EPV;
-    if (lane < head) {
-        T x = in[lane];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) fold_one<T>(w[c], A[c], x);
-    }
-    if (tail0 + lane < n) {
-        T x = in[tail0 + lane];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) fold_one<T>(w[c], A[c], x);
-    }
-    int64_t v = lane;
-    for (; v + (SU - 1) * 32 < nvec; v += 32 * SU) {
-        uint4 b[SU];
-#pragma unroll
-        for (int u = 0; u < SU; ++u) b[u] = ld_batch(vin + v + u * 32);
-#pragma unroll
-        for (int c = 0; c < NC; ++c) fold_vec<T, SU>(w[c], A[c], b);
-    }
-#pragma unroll
-    for (int u = 0; u < SU; ++u) {
-        const int64_t vv = v + u * 32;
-        if (vv < nvec) {
-            uint4 b = ld_batch(vin + vv);
-#pragma unroll
-            for (int c = 0; c < NC; ++c) fold_vec<T, 1>(w[c], A[c], &b);
-        }
-    }
+    stream_fold<T, NC, SU, 32>(in, n, lane, w, A, ld_batch);
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
         warp_merge(w[c], E64, A[c]);
@@ -625,7 +561,10 @@ struct SegmentSource {
 // descriptor, then tile).
 template <typename Src>
 static int plan_chunked(const Src &src, int64_t n, HostPlan &P) {
-    const int64_t small_b = g_small_bytes.load(), tile_b = P.tile_override > 0 ? P.tile_override : g_tile_bytes.load();
+    // (a stretch that one warp or CTA folds stays below 64 GiB: 32-bit vector counts)
+    constexpr int64_t most = (int64_t)1 << 35;
+    const int64_t small_b = std::min(g_small_bytes.load(), most);
+    const int64_t tile_b = std::min(P.tile_override > 0 ? P.tile_override : g_tile_bytes.load(), most);
     P.tile_bytes = tile_b;
     const int nch = n >= PAR_MIN_REGIONS ? 2 * plan_pool().threads() : 1;
     std::vector<PlanChunk> ch((size_t)nch);

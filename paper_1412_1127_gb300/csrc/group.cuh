@@ -136,26 +136,4 @@ __device__ __forceinline__ void group_fold(const T *in, int len, bool live, int 
     for (int c = 0; c < NC; ++c) group_merge<PAIR>(w[c], E64, A[c], L);
 }
 
-// The element that leaves a fold under working code w as it is (element bits).
-template <typename T>
-inline uint64_t neutral_element(int w) {
-    constexpr bool e64 = sizeof(T) == 8;
-    switch (w) {
-    case W_MUL32:
-    case W_MUL64:
-    case W_LAND: return 1;
-    case W_MAXI: return e64 ? (uint64_t)INT64_MIN : (uint64_t)(uint32_t)INT32_MIN;
-    case W_MINI: return e64 ? (uint64_t)INT64_MAX : (uint64_t)(uint32_t)INT32_MAX;
-    case W_AND: return ~0ull;
-    case W_ADDF:
-    case W_ADDF_COMP:
-    case W_ADDF_WIDE: return e64 ? d2u(-0.0) : f2u(-0.0f);
-    case W_MULF:
-    case W_MULF_WIDE: return e64 ? d2u(1.0) : f2u(1.0f);
-    case W_MAXF: return e64 ? d2u(-INFINITY) : f2u(-INFINITY);
-    case W_MINF: return e64 ? d2u(INFINITY) : f2u(INFINITY);
-    default: return 0;  // sums, |, ^, ||
-    }
-}
-
 }  // namespace accr

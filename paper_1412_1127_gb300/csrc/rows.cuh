@@ -44,44 +44,12 @@ template <typename T, int NC, bool FIXED>
 __device__ __forceinline__ void fold_stretch(const T *row, int len, const ClauseDev *cl, const int (&w)[NC], int lane,
                                              Acc (&A)[NC]) {
     constexpr bool E64 = sizeof(T) == 8;
-    constexpr int EPV = 16 / (int)sizeof(T);
-    const int mis = (int)(((16 - ((uintptr_t)row & 15)) & 15) / sizeof(T));
-    const int head = mis < len ? mis : len;
-    const uint4 *vr = (const uint4 *)(row + head);
-    const int nvec = (len - head) / EPV;
-    const int tail0 = head + nvec * EPV;
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
         A[c].a = cl[c].ident;
         A[c].c = 0.f;
     }
-    if (lane < head) {
-        T x = row[lane];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) fold_one<T>(w[c], A[c], x);
-    }
-    if (tail0 + lane < len) {
-        T x = row[tail0 + lane];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) fold_one<T>(w[c], A[c], x);
-    }
-    int v = lane;
-    for (; v + (RU2 - 1) * 32 < nvec; v += 32 * RU2) {
-        uint4 b[RU2];
-#pragma unroll
-        for (int u = 0; u < RU2; ++u) b[u] = ld_row(vr + v + u * 32);
-#pragma unroll
-        for (int c = 0; c < NC; ++c) fold_vec<T, RU2>(w[c], A[c], b);
-    }
-#pragma unroll
-    for (int u = 0; u < RU2; ++u) {
-        const int vv = v + u * 32;
-        if (vv < nvec) {
-            uint4 b = ld_row(vr + vv);
-#pragma unroll
-            for (int c = 0; c < NC; ++c) fold_vec<T, 1>(w[c], A[c], &b);
-        }
-    }
+    stream_fold<T, NC, RU2, 32>(row, len, lane, w, A, ld_row);
 #pragma unroll
     for (int c = 0; c < NC; ++c) warp_merge<FIXED>(w[c], E64, A[c]);
 }
