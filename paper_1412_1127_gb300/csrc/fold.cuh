@@ -499,26 +499,6 @@ __device__ __forceinline__ void fold_vec(int w, Acc &A, const uint4 *v) {
     }
 }
 
-// Fold the first `cnt` of NV vectors (a stretch's last, partial round).  A
-// float sum in double takes them as one chunk, the missing ones as -0: vector
-// by vector it would pay the FP64 pipe per element.
-template <typename T, int NV>
-__device__ __forceinline__ void fold_prefix(int w, Acc &A, const uint4 *v, int cnt) {
-    if constexpr (std::is_same<T, float>::value && NV > 1) {
-        if (w == W_ADDF_WIDE) {
-            uint4 f[NV];
-#pragma unroll
-            for (int u = 0; u < NV; ++u)
-                f[u] = u < cnt ? v[u] : make_uint4(0x80000000u, 0x80000000u, 0x80000000u, 0x80000000u);
-            if (cnt > 0) fold_vec<T, NV>(w, A, f);
-            return;
-        }
-    }
-#pragma unroll
-    for (int u = 0; u < NV; ++u)
-        if (u < cnt) fold_vec<T, 1>(w, A, v + u);
-}
-
 // The element that leaves a fold under working code w as it is (element bits).
 template <typename T>
 __host__ __device__ __forceinline__ uint64_t neutral_element(int w) {

@@ -90,45 +90,60 @@ __global__ void __launch_bounds__(RB, 2) reduce_kernel(const __grid_constant__ R
         A[c].c = 0.f;
     }
 
+    // the unaligned head's and the ragged tail's elements (threads of CTA 0): loaded
+    // before the vectors, folded after them
     const int64_t gtid = (int64_t)blockIdx.x * RB + threadIdx.x;
-    if (gtid < head) {
-        T x = in[gtid];
+    T xh = T(), xt = T();
+    if (gtid < head) xh = in[gtid];
+    if (tail0 + gtid < n) xt = in[tail0 + gtid];
+    // Rounds of RB * RU vectors, CTA-contiguous; the last, partial one is loaded like
+    // a full one, missing vectors read as the clause's neutral element (one fold for
+    // both: the generic kernels carry every operator's code).  A region of less than
+    // one round of the grid has only a partial round, its vectors dealt out grid-wide
+    // so that every CTA has some.  (Folding a round in halves, each loaded again as
+    // soon as it is folded, gave the same times.)
+    const int64_t step = (int64_t)gridDim.x * (RB * RU);
+    for (int64_t base = (int64_t)blockIdx.x * (RB * RU); p.spread || base < nvec; base += step) {
+        const bool full = !p.spread && base + RB * RU <= nvec;  // the same for the CTA
+        uint4 b[RU];
+        int cnt = RU;
+        if (full) {
 #pragma unroll
-        for (int c = 0; c < NC; ++c) fold_one<T>(w[c], A[c], x);
+            for (int u = 0; u < RU; ++u) b[u] = ld_stream(vin + base + threadIdx.x + u * RB);
+        } else {
+            const int64_t v = p.spread ? gtid : base + threadIdx.x, us = p.spread ? (int64_t)gridDim.x * RB : RB;
+            const uint4 n0 = neutral_vector<T>(w[0]);
+            cnt = 0;
+#pragma unroll
+            for (int u = 0; u < RU; ++u) {
+                b[u] = n0;
+                if (v + u * us < nvec) {
+                    b[u] = ld_stream(vin + v + u * us);
+                    cnt = u + 1;
+                }
+            }
+        }
+        fold_vec<T, RU>(w[0], A[0], b);
+#pragma unroll
+        for (int c = 1; c < NC; ++c) {
+            if (!full) {
+                const uint4 nn = neutral_vector<T>(w[c]);
+#pragma unroll
+                for (int u = 0; u < RU; ++u)
+                    if (u >= cnt) b[u] = nn;
+            }
+            fold_vec<T, RU>(w[c], A[c], b);
+        }
+        if (!full) break;
+    }
+    if (gtid < head) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) fold_one<T>(w[c], A[c], xh);
     }
     if (tail0 + gtid < n) {
-        T x = in[tail0 + gtid];
 #pragma unroll
-        for (int c = 0; c < NC; ++c) fold_one<T>(w[c], A[c], x);
+        for (int c = 0; c < NC; ++c) fold_one<T>(w[c], A[c], xt);
     }
-
-    // Full rounds: CTA-contiguous chunks of RB * RU vectors.  (Folding a round in
-    // halves, each loaded again as soon as it is folded, gave the same times:
-    // the sum, max and min of 2^28 floats 0.160 ms against 0.159.)
-    uint4 b[RU];
-    int64_t v = (int64_t)blockIdx.x * (RB * RU) + threadIdx.x;
-    const int64_t step = (int64_t)gridDim.x * (RB * RU);
-    for (; !p.spread && v + (RU - 1) * RB < nvec; v += step) {
-#pragma unroll
-        for (int u = 0; u < RU; ++u) b[u] = ld_stream(vin + v + u * RB);
-#pragma unroll
-        for (int c = 0; c < NC; ++c) fold_vec<T, RU>(w[c], A[c], b);
-    }
-    // The last, partial round, loads in flight together.  A region of less than
-    // one round has only this: its vectors are then dealt out grid-wide (us apart),
-    // so that every CTA has some.
-    if (p.spread) v = (int64_t)blockIdx.x * RB + threadIdx.x;
-    const int64_t us = p.spread ? (int64_t)gridDim.x * RB : RB;
-    int cnt = 0;
-#pragma unroll
-    for (int u = 0; u < RU; ++u) {
-        if (v + u * us < nvec) {
-            b[u] = ld_stream(vin + v + u * us);
-            cnt = u + 1;
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < NC; ++c) fold_prefix<T, RU>(w[c], A[c], b, cnt);
 
     cta_merge<NC, RB, (W0 >= 0)>(w, ident, E64, A, sh);
     const int G = gridDim.x;
