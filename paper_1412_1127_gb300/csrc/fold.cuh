@@ -238,59 +238,52 @@ __host__ __device__ __forceinline__ void two_sum_merge(float &s, float &c, float
 }
 
 // Sum of the 2*NV doubles of a chunk.  GB300's FP64 pipe retires about two
-// adds per SM per clock, too few for a double sum at HBM rate, and integer work
-// on the significands about four values a clock, so a chunk of 8 or more values
-// uses both pipes at once: the first DV values are added as doubles, the others
-// in integer block floating point: each significand (with its implicit bit) is
-// aligned to the largest exponent among them with 6 guard bits, the aligned
-// magnitudes are added in an int64 with their signs, and the total is converted
-// and scaled by an exact power of two.
+// adds per SM per clock, too few for a double sum at HBM rate, so chunks of
+// 8 or more values are summed in integer block floating point: each
+// significand (with its implicit bit) is aligned to the chunk's largest
+// exponent with 6 guard bits, the aligned magnitudes are added in an int64
+// with their signs, and the total is converted and scaled by an exact power
+// of two -- two FP64-pipe operations per chunk instead of one per value.
 // Bits shifted out are truncated: at most 2^-6 of the largest value's ulp per
 // element (under 0.25 ulp for a chunk of 16).  Zeros and subnormals shift out
 // whole: chunks whose largest exponent is within 60 of the subnormal range, and
-// short chunks, are added as doubles.  Finite inputs only.
-// Three clauses over 17.3M doubles: 37.5 us, 70 with FP64 adds alone.
+// short chunks, are added as doubles.  Finite inputs only.  (5 of 16 values on the
+// FP64 pipe meanwhile was faster, 2^27 doubles 0.158 ms against 0.160, but
+// rounds a chunk five times instead of once: about 5 % more error.)
 template <int NV>
 __device__ __forceinline__ double chunk_sum_f64(const uint4 *v) {
     constexpr int E = 2 * NV;
-    constexpr int DV = E < 8 ? E : E < 16 ? 3 : 5;
-    double t = u2d(word64(v[0], 0));
+    uint32_t hi[E], lo[E], emax = 0;
 #pragma unroll
-    for (int j = 1; j < DV; ++j) t = __dadd_rn(t, u2d(word64(v[j >> 1], j & 1)));
-    if constexpr (E < 8) {
-        return t;
-    } else {
-        uint32_t hi[E - DV], lo[E - DV], emax = 0;
-#pragma unroll
-        for (int j = DV; j < E; ++j) {
-            lo[j - DV] = (j & 1) ? v[j >> 1].z : v[j >> 1].x;
-            hi[j - DV] = (j & 1) ? v[j >> 1].w : v[j >> 1].y;
-            emax = max(emax, hi[j - DV] & 0x7ff00000u);
-        }
-        if (emax < 61u << 20) {  // tiny values: the scale below would leave the normal range
-#pragma unroll
-            for (int j = DV; j < E; ++j) t = __dadd_rn(t, u2d(word64(v[j >> 1], j & 1)));
-            return t;
-        }
-        // a negative magnitude is added as its complement, and the ones still
-        // missing for two's complement are counted
-        uint64_t S = 0;
-        int32_t negs = 0;
-#pragma unroll
-        for (int j = 0; j < E - DV; ++j) {
-            const uint64_t m = ((uint64_t)((hi[j] & 0x000fffffu) | 0x00100000u) << 32) | lo[j];
-            const uint32_t sh = (emax - (hi[j] & 0x7ff00000u)) >> 20;
-            uint64_t mag;
-            asm("shr.u64 %0, %1, %2;" : "=l"(mag) : "l"(m << 6), "r"(sh));  // 64 and more: 0
-            const int32_t s = (int32_t)hi[j] >> 31;
-            S += mag ^ (uint64_t)(int64_t)s;
-            negs -= s;
-        }
-        S += (uint64_t)(int64_t)negs;
-        // S counts units of 2^(emax - 1075 - 6); that power of two is normal here
-        const double scale = u2d((uint64_t)((emax >> 20) - 1081 + 1023) << 52);
-        return __fma_rn(__ll2double_rn((long long)S), scale, t);
+    for (int j = 0; j < E; ++j) {
+        lo[j] = (j & 1) ? v[j >> 1].z : v[j >> 1].x;
+        hi[j] = (j & 1) ? v[j >> 1].w : v[j >> 1].y;
+        emax = max(emax, hi[j] & 0x7ff00000u);
     }
+    if (E < 8 || emax < 61u << 20) {  // tiny values: the scale below would leave the normal range
+        double t = u2d(word64(v[0], 0));
+#pragma unroll
+        for (int j = 1; j < E; ++j) t = __dadd_rn(t, u2d(word64(v[j >> 1], j & 1)));
+        return t;
+    }
+    // a negative magnitude is added as its complement, and the ones still
+    // missing for two's complement are counted
+    uint64_t S = 0;
+    int32_t negs = 0;
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+        const uint64_t m = ((uint64_t)((hi[j] & 0x000fffffu) | 0x00100000u) << 32) | lo[j];
+        const uint32_t sh = (emax - (hi[j] & 0x7ff00000u)) >> 20;
+        uint64_t mag;
+        asm("shr.u64 %0, %1, %2;" : "=l"(mag) : "l"(m << 6), "r"(sh));  // 64 and more: 0
+        const int32_t s = (int32_t)hi[j] >> 31;
+        S += mag ^ (uint64_t)(int64_t)s;
+        negs -= s;
+    }
+    S += (uint64_t)(int64_t)negs;
+    // S counts units of 2^(emax - 1075 - 6); that power of two is normal here
+    const double scale = u2d((uint64_t)((emax >> 20) - 1081 + 1023) << 52);
+    return __dmul_rn(__ll2double_rn((long long)S), scale);
 }
 
 // a += the sum of the 4*NV floats of a chunk, in double.  Converting and adding

@@ -329,8 +329,11 @@ static int grid_for(int nc, int64_t n) {
     }
     const int64_t nvec = n * (int64_t)sizeof(T) / 16;
     // Two vectors a thread until the chip is full: a small region's time is the
-    // latency of its loads and merges, so it is spread over more SMs first.
-    int64_t want = (nvec + (int64_t)RB * 2 - 1) / ((int64_t)RB * 2);
+    // latency of its loads and merges, so it is spread over more SMs first.  Doubles
+    // get a whole round a thread: a sum rounds once a chunk (chunk_sum_f64) and once
+    // at each level of the merges, so more threads would mean more error.
+    const int64_t per = (int64_t)RB * (std::is_same<T, double>::value ? RU : 2);
+    int64_t want = (nvec + per - 1) / per;
     if (want < 1) want = 1;
     return (int)(want < maxg ? want : maxg);
 }
