@@ -7,11 +7,11 @@
 // reads a and b straight from global memory; Sec. 4.2 (Matrix Mul) notes that
 // the tiled CUDA SDK version, which stages tiles in shared memory and shares
 // them among a block's threads, is much faster.  This kernel is the tiled
-// form: a CTA computes a 128 x 128 block of c, stages 16-wide k slices of a
+// form: a CTA computes a BM x BN block of c, stages 16-wide k slices of a
 // (transposed) and b in double-buffered shared memory, and every thread keeps
-// an 8 x 8 register block (two 4 x 4 quadrants 64 apart, so the 16-byte
-// shared-memory reads of a warp hit distinct banks or broadcast), with its
-// operand fragments double-buffered in registers.
+// a TR x TC register block (a side of 8 is two runs of 4 half a tile apart, so
+// the 16-byte shared-memory reads of a warp hit distinct banks or broadcast),
+// with its operand fragments double-buffered in registers.
 //
 // Every output still sums its l terms in order 0..LEN-1.  Mode SERIAL rounds
 // each product and then each sum (no fused multiply-add), which is exactly
@@ -23,9 +23,7 @@
 
 namespace accr {
 
-constexpr int MT = 128;   // CTA tile (rows and columns of c)
 constexpr int KT = 16;    // k slice per stage
-constexpr int NTH = 256;  // threads per CTA
 
 template <bool SERIAL>
 __device__ __forceinline__ float mac(float acc, float x, float y) {
@@ -33,22 +31,35 @@ __device__ __forceinline__ float mac(float acc, float x, float y) {
     else return __fmaf_rn(x, y, acc);
 }
 
-template <bool SERIAL, bool VEC>
-__global__ void __launch_bounds__(NTH, 2) matmul_simt_kernel(const float *__restrict__ a, const float *__restrict__ b,
-                                                             float *__restrict__ c, int64_t len) {
-    __shared__ __align__(16) float As[2][KT][MT];  // a slice, transposed: As[k][row]
-    __shared__ __align__(16) float Bs[2][KT][MT];  // b slice: Bs[k][col]
+// Row r of a's slice at k sits at column r ^ swz(k): the four k groups that a
+// warp's loader stores at once then fall into different banks (they were a
+// four-way conflict), and four consecutive rows stay together.  (SERIAL's 128 x 128
+// tile has no registers left for it: LEN 4096 4612 us with, 4567 without.)
+template <int SWZ>
+__device__ __forceinline__ int a_col(int r, int k) {
+    return r ^ (((k >> 2) & 3) * SWZ);
+}
+
+template <bool SERIAL, bool VEC, int BM, int BN, int TR, int TC>
+__global__ void __launch_bounds__(BM * BN / (TR * TC), 512 / (BM * BN / (TR * TC)))
+    matmul_simt_kernel(const float *__restrict__ a, const float *__restrict__ b, float *__restrict__ c, int64_t len) {
+    constexpr int NTH = BM * BN / (TR * TC);  // threads
+    constexpr int QR = TR / 4, QC = TC / 4;   // runs of 4 a side
+    constexpr int LA = BM * KT / 4 / NTH, LB = BN * KT / 4 / NTH;  // float4 loads per thread and slice
+    constexpr int SWZ = SERIAL && BM == 128 ? 0 : 8;
+    static_assert(LA * NTH * 4 == BM * KT && LB * NTH * 4 == BN * KT, "loads split evenly");
+    __shared__ __align__(16) float As[2][KT][BM];  // a slice, transposed: As[k][a_col(row, k)]
+    __shared__ __align__(16) float Bs[2][KT][BN];  // b slice: Bs[k][col]
     const int tid = threadIdx.x;
-    const int tx = tid & 15, ty = tid >> 4;
-    const int64_t row0 = (int64_t)blockIdx.y * MT, col0 = (int64_t)blockIdx.x * MT;
+    const int tx = tid % (BN / TC), ty = tid / (BN / TC);
+    const int64_t row0 = (int64_t)blockIdx.y * BM, col0 = (int64_t)blockIdx.x * BN;
 
-    // loaders: a 128x16 slice = 512 float4 (two per thread: rows tid>>2 and 64 + tid>>2,
-    //          k (tid&3)*4); b 16x128 slice = 512 float4 (k tid>>5 and 8 + tid>>5, col (tid&31)*4)
+    // loaders: a slice: four float4 a row (k (tid & 3) * 4), rows tid / 4 and on by NTH / 4;
+    //          b slice: BN / 4 float4 a k row, neighbouring threads along it
     const int a_r = tid >> 2, a_k = (tid & 3) * 4;
-    const int b_k = tid >> 5, b_c = (tid & 31) * 4;
 
-    auto load_a = [&](int64_t k0, int half, float4 &v) {
-        const int64_t r = row0 + a_r + half * 64, k = k0 + a_k;
+    auto load_a = [&](int64_t k0, int h, float4 &v) {
+        const int64_t r = row0 + a_r + h * (NTH / 4), k = k0 + a_k;
         if (VEC && r < len && k + 3 < len) {
             v = __ldg(reinterpret_cast<const float4 *>(a + r * len + k));
         } else {
@@ -58,8 +69,9 @@ __global__ void __launch_bounds__(NTH, 2) matmul_simt_kernel(const float *__rest
             v.w = (r < len && k + 3 < len) ? a[r * len + k + 3] : 0.f;
         }
     };
-    auto load_b = [&](int64_t k0, int half, float4 &v) {
-        const int64_t k = k0 + b_k + half * 8, cc = col0 + b_c;
+    auto load_b = [&](int64_t k0, int h, float4 &v) {
+        const int i = tid + h * NTH;
+        const int64_t k = k0 + i / (BN / 4), cc = col0 + (i % (BN / 4)) * 4;
         if (VEC && k < len && cc + 3 < len) {
             v = __ldg(reinterpret_cast<const float4 *>(b + k * len + cc));
         } else {
@@ -69,29 +81,33 @@ __global__ void __launch_bounds__(NTH, 2) matmul_simt_kernel(const float *__rest
             v.w = (k < len && cc + 3 < len) ? b[k * len + cc + 3] : 0.f;
         }
     };
-    auto store_tiles = [&](int buf, const float4 (&va)[2], const float4 (&vb)[2]) {
+    auto store_tiles = [&](int buf, const float4 (&va)[LA], const float4 (&vb)[LB]) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            As[buf][a_k + 0][a_r + h * 64] = va[h].x;
-            As[buf][a_k + 1][a_r + h * 64] = va[h].y;
-            As[buf][a_k + 2][a_r + h * 64] = va[h].z;
-            As[buf][a_k + 3][a_r + h * 64] = va[h].w;
-            *reinterpret_cast<float4 *>(&Bs[buf][b_k + h * 8][b_c]) = vb[h];
+        for (int h = 0; h < LA; ++h) {
+            const int r = a_col<SWZ>(a_r + h * (NTH / 4), a_k);
+            As[buf][a_k + 0][r] = va[h].x;
+            As[buf][a_k + 1][r] = va[h].y;
+            As[buf][a_k + 2][r] = va[h].z;
+            As[buf][a_k + 3][r] = va[h].w;
+        }
+#pragma unroll
+        for (int h = 0; h < LB; ++h) {
+            const int i = tid + h * NTH;
+            *reinterpret_cast<float4 *>(&Bs[buf][i / (BN / 4)][(i % (BN / 4)) * 4]) = vb[h];
         }
     };
 
-    float acc[8][8];
+    float acc[TR][TC];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < TR; ++i)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+        for (int j = 0; j < TC; ++j) acc[i][j] = 0.f;
 
-    float4 va[2], vb[2];
+    float4 va[LA], vb[LB];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        load_a(0, h, va[h]);
-        load_b(0, h, vb[h]);
-    }
+    for (int h = 0; h < LA; ++h) load_a(0, h, va[h]);
+#pragma unroll
+    for (int h = 0; h < LB; ++h) load_b(0, h, vb[h]);
     store_tiles(0, va, vb);
     __syncthreads();
     const int64_t nk = (len + KT - 1) / KT;
@@ -100,47 +116,48 @@ __global__ void __launch_bounds__(NTH, 2) matmul_simt_kernel(const float *__rest
         const bool more = kt + 1 < nk;
         if (more) {  // fetch the next slice while this one is used
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                load_a((kt + 1) * KT, h, va[h]);
-                load_b((kt + 1) * KT, h, vb[h]);
-            }
+            for (int h = 0; h < LA; ++h) load_a((kt + 1) * KT, h, va[h]);
+#pragma unroll
+            for (int h = 0; h < LB; ++h) load_b((kt + 1) * KT, h, vb[h]);
         }
         // operand fragments double-buffered in registers: k+1 is read from
-        // shared memory while the 64 products of k issue
-        float4 fa[2][2], fb[2][2];
-        fa[0][0] = *reinterpret_cast<const float4 *>(&As[cur][0][ty * 4]);
-        fa[0][1] = *reinterpret_cast<const float4 *>(&As[cur][0][64 + ty * 4]);
-        fb[0][0] = *reinterpret_cast<const float4 *>(&Bs[cur][0][tx * 4]);
-        fb[0][1] = *reinterpret_cast<const float4 *>(&Bs[cur][0][64 + tx * 4]);
+        // shared memory while the products of k issue
+        float4 fa[2][QR], fb[2][QC];
+        auto fetch = [&](int k, float4 (&xa)[QR], float4 (&xb)[QC]) {
+#pragma unroll
+            for (int q = 0; q < QR; ++q)
+                xa[q] = *reinterpret_cast<const float4 *>(&As[cur][k][a_col<SWZ>(q * (BM / QR) + ty * 4, k)]);
+#pragma unroll
+            for (int q = 0; q < QC; ++q) xb[q] = *reinterpret_cast<const float4 *>(&Bs[cur][k][q * (BN / QC) + tx * 4]);
+        };
+        fetch(0, fa[0], fb[0]);
 #pragma unroll
         for (int k = 0; k < KT; ++k) {
             const int p = k & 1;
-            if (k + 1 < KT) {
-                fa[p ^ 1][0] = *reinterpret_cast<const float4 *>(&As[cur][k + 1][ty * 4]);
-                fa[p ^ 1][1] = *reinterpret_cast<const float4 *>(&As[cur][k + 1][64 + ty * 4]);
-                fb[p ^ 1][0] = *reinterpret_cast<const float4 *>(&Bs[cur][k + 1][tx * 4]);
-                fb[p ^ 1][1] = *reinterpret_cast<const float4 *>(&Bs[cur][k + 1][64 + tx * 4]);
-            }
-            const float ar[8] = {fa[p][0].x, fa[p][0].y, fa[p][0].z, fa[p][0].w,
-                                 fa[p][1].x, fa[p][1].y, fa[p][1].z, fa[p][1].w};
-            const float br[8] = {fb[p][0].x, fb[p][0].y, fb[p][0].z, fb[p][0].w,
-                                 fb[p][1].x, fb[p][1].y, fb[p][1].z, fb[p][1].w};
+            if (k + 1 < KT) fetch(k + 1, fa[p ^ 1], fb[p ^ 1]);
+            float ar[TR], br[TC];
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+            for (int q = 0; q < QR; ++q)
+                ar[q * 4 + 0] = fa[p][q].x, ar[q * 4 + 1] = fa[p][q].y, ar[q * 4 + 2] = fa[p][q].z, ar[q * 4 + 3] = fa[p][q].w;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) acc[i][j] = mac<SERIAL>(acc[i][j], ar[i], br[j]);
+            for (int q = 0; q < QC; ++q)
+                br[q * 4 + 0] = fb[p][q].x, br[q * 4 + 1] = fb[p][q].y, br[q * 4 + 2] = fb[p][q].z, br[q * 4 + 3] = fb[p][q].w;
+#pragma unroll
+            for (int i = 0; i < TR; ++i)
+#pragma unroll
+                for (int j = 0; j < TC; ++j) acc[i][j] = mac<SERIAL>(acc[i][j], ar[i], br[j]);
         }
         if (more) store_tiles(cur ^ 1, va, vb);
         __syncthreads();
     }
-    // write the 8 x 8 register block
+    // write the register block
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int64_t r = row0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4));
+    for (int i = 0; i < TR; ++i) {
+        const int64_t r = row0 + (i >> 2) * (BM / QR) + ty * 4 + (i & 3);
         if (r >= len) continue;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int64_t cc = col0 + h * 64 + tx * 4;
+        for (int h = 0; h < QC; ++h) {
+            const int64_t cc = col0 + h * (BN / QC) + tx * 4;
             float4 v = make_float4(acc[i][h * 4 + 0], acc[i][h * 4 + 1], acc[i][h * 4 + 2], acc[i][h * 4 + 3]);
             if (VEC && cc + 3 < len) {
                 *reinterpret_cast<float4 *>(c + r * len + cc) = v;
@@ -207,21 +224,42 @@ __global__ void __launch_bounds__(PROBE_THREADS) fma2_probe_kernel(int64_t round
     sink[(int64_t)blockIdx.x * PROBE_THREADS + threadIdx.x] = s * (1.f / 32.f);
 }
 
+template <bool SERIAL, int BM, int BN, int TR, int TC>
+static void simt_launch(const float *a, const float *b, float *c, int64_t len, bool vec, cudaStream_t s) {
+    const dim3 grid((unsigned)((len + BN - 1) / BN), (unsigned)((len + BM - 1) / BM));
+    constexpr int NTH = BM * BN / (TR * TC);
+    if (vec) matmul_simt_kernel<SERIAL, true, BM, BN, TR, TC><<<grid, NTH, 0, s>>>(a, b, c, len);
+    else matmul_simt_kernel<SERIAL, false, BM, BN, TR, TC><<<grid, NTH, 0, s>>>(a, b, c, len);
+}
+
 int matmul_simt(const float *a, const float *b, float *c, int64_t len, bool serial, cudaStream_t s) {
     if (len == 0) return ACCR_OK;
-    const int64_t tiles = (len + MT - 1) / MT;
+    const int64_t tiles = (len + 127) / 128;
     if (tiles > 65535) return set_error(ACCR_EINVAL, "accr_matmul_nest: len too large for the SIMT grid");
-    dim3 grid((unsigned)tiles, (unsigned)tiles);
     // 16-byte vector access needs 16-byte aligned rows
     int rc = launch_guard("matmul_simt_kernel");
     if (rc != ACCR_OK) return rc;
     const bool vec = (len % 4 == 0) && ((uintptr_t)a % 16 == 0) && ((uintptr_t)b % 16 == 0) && ((uintptr_t)c % 16 == 0);
+    // The tile by how the matrix fills the chip (every form adds an output's terms
+    // in the same order, so they give the same bits).  Measured, us, 128 x 128 /
+    // 64 x 64 / 32 x 32 tiles: LEN 512 60 / 25 / 19, 900 117 / 68 / 64, 1024 115 / 72 / 76,
+    // 1200 150 / 117 / 139, 1448 181 / 179 / 227, 1536 173 / 177 / 228, 2048 411 / 423 / 533.
+    // SERIAL's separate products and sums leave the large tile short of registers:
+    // 1024 205 / 101 / 102, 1448 308 / 262 / 285, 2048 676 / 625, 3000 1996 / 1934.
+    const int64_t sms = device_info().sms;
+    const int64_t t128 = tiles * tiles, t64 = ((len + 63) / 64) * ((len + 63) / 64);
+    // Past one 128 x 128 tile an SM its rounds (one tile an SM) cost 3.8 of the small
+    // tile's: 3072 1997 / 2070 us, 3500 3371 / 2997, 4096 4555 / 4688.
+    const int64_t r128 = (t128 + sms - 1) / sms, r64 = (t64 + sms - 1) / sms;
+    const bool small = t64 * 10 < sms * 16;
     if (serial) {
-        if (vec) matmul_simt_kernel<true, true><<<grid, NTH, 0, s>>>(a, b, c, len);
-        else matmul_simt_kernel<true, false><<<grid, NTH, 0, s>>>(a, b, c, len);
+        if (small) simt_launch<true, 32, 32, 4, 4>(a, b, c, len, vec, s);
+        else if (r128 < 2 || r128 * 38 >= r64 * 10) simt_launch<true, 64, 64, 8, 4>(a, b, c, len, vec, s);
+        else simt_launch<true, 128, 128, 8, 8>(a, b, c, len, vec, s);
     } else {
-        if (vec) matmul_simt_kernel<false, true><<<grid, NTH, 0, s>>>(a, b, c, len);
-        else matmul_simt_kernel<false, false><<<grid, NTH, 0, s>>>(a, b, c, len);
+        if (small) simt_launch<false, 32, 32, 4, 4>(a, b, c, len, vec, s);
+        else if (t128 * 10 < sms * 9) simt_launch<false, 64, 64, 8, 4>(a, b, c, len, vec, s);
+        else simt_launch<false, 128, 128, 8, 8>(a, b, c, len, vec, s);
     }
     return launched("matmul_simt_kernel");
 }
