@@ -35,6 +35,7 @@
 #include "common.cuh"
 #include "debug.cuh"
 #include "fold.cuh"
+#include "overlap.cuh"
 
 namespace accr {
 
@@ -223,6 +224,7 @@ __device__ __forceinline__ void batch_body(const BatchArgs &p, const RegionDev *
     __shared__ Acc sh[RD_CLAUSES][BB / 32];
     __shared__ int s_last;
     __shared__ long long s_q;
+    grid_dependency();
     // tiles of long regions, one CTA per tile, taken from a queue (largest
     // first within each element-type group); the next index is fetched while
     // the current tile is folded
@@ -850,7 +852,7 @@ static int run_once(HostPlan &P, unsigned flags, accr_stream_t stream) {
         std::copy(P.small.begin(), P.small.end(), ai.small);
         rc = launch_guard("batch_kernel");
         if (rc != ACCR_OK) return rc;
-        batch_kernel_inline<<<batch_grid(P), BB, 0, s>>>(ai);
+        launch_overlapped(batch_kernel_inline, dim3((unsigned)batch_grid(P)), BB, 0, s, ai);
         rc = launched("batch_kernel");
         if (rc != ACCR_OK) return rc;
         if (flags & ACCR_SYNC) return cuda_check(cudaStreamSynchronize(s), "batch: sync");
@@ -862,7 +864,7 @@ static int run_once(HostPlan &P, unsigned flags, accr_stream_t stream) {
     if ((rc = send_stage(B, i, P.plan_bytes, s)) != ACCR_OK) return rc;
     BatchArgs a = args_for(P, B->dev, B->counters);
     if ((rc = launch_guard("batch_kernel")) != ACCR_OK) return rc;
-    batch_kernel<<<batch_grid(P), BB, 0, s>>>(a);
+    launch_overlapped(batch_kernel, dim3((unsigned)batch_grid(P)), BB, 0, s, a);
     rc = launched("batch_kernel");
     if (rc != ACCR_OK) return rc;
     if (flags & ACCR_SYNC) return cuda_check(cudaStreamSynchronize(s), "batch: sync");

@@ -20,6 +20,7 @@
 #include <string.h>
 
 #include "common.cuh"
+#include "overlap.cuh"
 
 namespace accr {
 
@@ -48,6 +49,7 @@ __global__ void __launch_bounds__(BM * BN / (TR * TC), 512 / (BM * BN / (TR * TC
     constexpr int LA = BM * KT / 4 / NTH, LB = BN * KT / 4 / NTH;  // float4 loads per thread and slice
     constexpr int SWZ = SERIAL && BM == 128 ? 0 : 8;
     static_assert(LA * NTH * 4 == BM * KT && LB * NTH * 4 == BN * KT, "loads split evenly");
+    grid_dependency();
     __shared__ __align__(16) float As[2][KT][BM];  // a slice, transposed: As[k][a_col(row, k)]
     __shared__ __align__(16) float Bs[2][KT][BN];  // b slice: Bs[k][col]
     const int tid = threadIdx.x;
@@ -228,8 +230,8 @@ template <bool SERIAL, int BM, int BN, int TR, int TC>
 static void simt_launch(const float *a, const float *b, float *c, int64_t len, bool vec, cudaStream_t s) {
     const dim3 grid((unsigned)((len + BN - 1) / BN), (unsigned)((len + BM - 1) / BM));
     constexpr int NTH = BM * BN / (TR * TC);
-    if (vec) matmul_simt_kernel<SERIAL, true, BM, BN, TR, TC><<<grid, NTH, 0, s>>>(a, b, c, len);
-    else matmul_simt_kernel<SERIAL, false, BM, BN, TR, TC><<<grid, NTH, 0, s>>>(a, b, c, len);
+    launch_overlapped(vec ? matmul_simt_kernel<SERIAL, true, BM, BN, TR, TC> : matmul_simt_kernel<SERIAL, false, BM, BN, TR, TC>,
+                      grid, NTH, 0, s, a, b, c, len);
 }
 
 int matmul_simt(const float *a, const float *b, float *c, int64_t len, bool serial, cudaStream_t s) {

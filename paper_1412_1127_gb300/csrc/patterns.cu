@@ -33,6 +33,7 @@
 #include "common.cuh"
 #include "debug.cuh"
 #include "fold.cuh"
+#include "overlap.cuh"
 
 namespace accr {
 
@@ -299,6 +300,7 @@ __device__ __noinline__ void nearest_select(const NearestArgs &p, NearestShared 
 __global__ void __launch_bounds__(NK_THREADS, 2) nearest_kernel(const __grid_constant__ NearestArgs p) {
     __shared__ NearestShared s;
     __shared__ int am_last;
+    grid_dependency();
     const int t = threadIdx.x, lane = t & 31;
     // points are float2; the vector part starts at a 16-byte boundary
     const int64_t head = (((uintptr_t)p.pts & 15) != 0 && p.n > 0) ? 1 : 0;
@@ -417,7 +419,7 @@ static int nearest_launch(const float *pts, int64_t n, float qx, float qy, int k
     a.counter = scr->counters + 1;
     int rc = launch_guard("nearest_kernel");
     if (rc != ACCR_OK) return rc;
-    nearest_kernel<<<grid, NK_THREADS, 0, s>>>(a);
+    launch_overlapped(nearest_kernel, dim3((unsigned)grid), NK_THREADS, 0, s, a);
     return launched("nearest_kernel");
 }
 
@@ -672,6 +674,7 @@ template <bool AL>
 __global__ void __launch_bounds__(SF_THREADS, 1) standardize_fused_kernel(const __grid_constant__ StdArgs p) {
     __shared__ StatPartial sh[SF_THREADS / 32];
     __shared__ float s_mean, s_rstd;
+    grid_dependency();
     const int t = threadIdx.x, G = gridDim.x;
     unsigned gen = (*(volatile unsigned *)&p.bar[1]) >> 1;
     const int64_t nq = p.n / 4, per = (nq + G - 1) / G;
@@ -816,6 +819,7 @@ __global__ void __launch_bounds__(BF_THREADS) bfs_level_kernel(const uint8_t *__
                                                                int64_t rows, int64_t cols, int32_t L, int mode,
                                                                unsigned *more, const unsigned *before,
                                                                unsigned *partial, unsigned *counter) {
+    grid_dependency();
     if (before && *(const volatile unsigned *)before == 0u) {
         if (blockIdx.x == 0 && threadIdx.x == 0) *more = 0u;
         return;
@@ -1271,16 +1275,16 @@ extern "C" ACCR_API int accr_standardize(const float *x, int64_t n, float *y, do
     } else {
         // one cooperative launch: co-residency of every CTA is guaranteed, so
         // the wait at the grid barrier cannot starve a CTA that has to arrive
-        void *args[] = {&a};
         const bool al = (((uintptr_t)x | (uintptr_t)y) & 15) == 0;
-        const void *fn = al ? (const void *)standardize_fused_kernel<true> : (const void *)standardize_fused_kernel<false>;
+        auto fused_kernel = al ? standardize_fused_kernel<true> : standardize_fused_kernel<false>;
         if (grid == 1) {  // one CTA waits for nobody: an ordinary launch
-            rc = cuda_check(cudaLaunchKernel(fn, grid, SF_THREADS, args, 0, s), "accr_standardize: launch");
+            launch_overlapped(fused_kernel, dim3(1), SF_THREADS, 0, s, a);
         } else {
-            rc = cuda_check(cudaLaunchCooperativeKernel(fn, grid, SF_THREADS, args, 0, s),
+            void *args[] = {&a};
+            rc = cuda_check(cudaLaunchCooperativeKernel((void *)fused_kernel, dim3((unsigned)grid), dim3(SF_THREADS), args, 0, s),
                             "accr_standardize: cooperative launch");
+            if (rc != ACCR_OK) return rc;
         }
-        if (rc != ACCR_OK) return rc;
         if ((rc = launched("standardize_kernel (fused)")) != ACCR_OK) return rc;
     }
     if (flags & ACCR_SYNC) {
@@ -1375,9 +1379,9 @@ extern "C" ACCR_API int accr_grid_bfs(const uint8_t *open, int64_t rows, int64_t
         }
         for (int i = 0; i < BFS_GROUP; ++i) {
             if ((rc = launch_guard("bfs_level_kernel")) != ACCR_OK) return rc;
-            bfs_level_kernel<<<grid, BF_THREADS, 0, s>>>(open, dist, rows, cols, (int32_t)(L0 + i),
-                                                         mode == ACCR_BFS_GUARDED ? 1 : 0, more + i,
-                                                         i > 0 ? more + i - 1 : nullptr, partial, counter);
+            launch_overlapped(bfs_level_kernel, dim3((unsigned)grid), BF_THREADS, 0, s, open, dist, rows, cols,
+                              (int32_t)(L0 + i), mode == ACCR_BFS_GUARDED ? 1 : 0, more + i, i > 0 ? more + i - 1 : nullptr,
+                              partial, counter);
             if ((rc = launched("bfs_level_kernel")) != ACCR_OK) return rc;
         }
         rc = cuda_check(cudaMemcpyAsync(hmore, more, BFS_GROUP * sizeof(unsigned), cudaMemcpyDeviceToHost, s),

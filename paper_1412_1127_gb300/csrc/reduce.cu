@@ -20,6 +20,7 @@
 
 #include "common.cuh"
 #include "fold.cuh"
+#include "overlap.cuh"
 
 namespace accr {
 
@@ -70,6 +71,7 @@ __global__ void __launch_bounds__(RB, 2) reduce_kernel(const __grid_constant__ R
     constexpr int EPV = 16 / (int)sizeof(T);
     __shared__ Acc sh[NC][RB / 32];
     __shared__ int am_last;
+    grid_dependency();
 
     const T *in = (const T *)p.in;
     const int64_t n = p.n;
@@ -237,7 +239,7 @@ template <typename T, int NC, int W0 = -1, int W1 = -1, int W2 = -1>
 static int launch_t(ReduceArgs &a, int grid, cudaStream_t s) {
     int rc = launch_guard("reduce_kernel");
     if (rc != ACCR_OK) return rc;
-    reduce_kernel<T, NC, W0, W1, W2><<<grid, RB, 0, s>>>(a);
+    launch_overlapped(reduce_kernel<T, NC, W0, W1, W2>, dim3((unsigned)grid), RB, 0, s, a);
     return launched("reduce_kernel");
 }
 

@@ -14,6 +14,7 @@
 #include "debug.cuh"
 #include "fold.cuh"
 #include "group.cuh"
+#include "overlap.cuh"
 #include "rows.cuh"
 
 namespace accr {
@@ -29,6 +30,7 @@ template <typename T, int NC, int W0, int W1, int GV>
 __global__ void __launch_bounds__(WB) rowgroup_kernel(const __grid_constant__ RowArgs p) {
     constexpr bool E64 = sizeof(T) == 8;
     constexpr int EPV = 16 / (int)sizeof(T);
+    grid_dependency();
     const int lane = threadIdx.x & 31, L = p.lanes;
     const int l = lane & (L - 1);
     const int rpw = 32 / L;  // rows per warp
@@ -59,7 +61,8 @@ struct GroupLaunch {
         static std::atomic<int> cached[64];
         const int maxg = resident_ctas(rowgroup_kernel<T, NC, W0, W1, GV>, WB, cached);
         const int64_t per_cta = (int64_t)(WB / 32) * (32 / a.lanes);
-        rowgroup_kernel<T, NC, W0, W1, GV><<<clamp_grid((a.rows + per_cta - 1) / per_cta, maxg), WB, 0, s>>>(a);
+        const int grid = clamp_grid((a.rows + per_cta - 1) / per_cta, maxg);
+        launch_overlapped(rowgroup_kernel<T, NC, W0, W1, GV>, dim3((unsigned)grid), WB, 0, s, a);
     }
     template <typename T, int NC, int W0, int W1>
     int run(RowArgs &a, cudaStream_t s) const {

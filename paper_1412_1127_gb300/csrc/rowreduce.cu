@@ -43,6 +43,7 @@
 #include "debug.cuh"
 #include "fold.cuh"
 #include "group.cuh"
+#include "overlap.cuh"
 #include "rows.cuh"
 
 namespace accr {
@@ -86,6 +87,7 @@ template <typename T, int NC, int W0 = -1, int W1 = -1, int FORM = ROW_SEG>
 __global__ void __launch_bounds__(row_threads<T, NC, FORM>()) rowreduce_kernel(const __grid_constant__ RowArgs p) {
     constexpr bool E64 = sizeof(T) == 8, FIXED = W0 >= 0;
     constexpr int NTH = row_threads<T, NC, FORM>(), NW = NTH / 32;
+    grid_dependency();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t gw = (int64_t)blockIdx.x * NW + warp;
     const int64_t cols = p.cols;
@@ -242,29 +244,26 @@ template <typename T, int NC, int W0, int W1, int FORM>
 static void row_form(const RowArgs &a, cudaStream_t s) {
     static std::atomic<int> cached[64];
     constexpr int NTH = row_threads<T, NC, FORM>();
+    auto kernel = rowreduce_kernel<T, NC, W0, W1, FORM>;
     if (FORM == ROW_SEG_CTA) {  // a CTA per row, a warp per segment
         const int nt = a.cpr * 32 < NTH ? (int)a.cpr * 32 : NTH;
-        rowreduce_kernel<T, NC, W0, W1, FORM><<<(unsigned)a.rows, nt, 0, s>>>(a);
+        launch_overlapped(kernel, dim3((unsigned)a.rows), nt, 0, s, a);
         return;
     }
-    const int maxg = resident_ctas(rowreduce_kernel<T, NC, W0, W1, FORM>, NTH, cached);
+    const int maxg = resident_ctas(kernel, NTH, cached);
     // chunks of long rows: at most one CTA per chunk, each taking a contiguous
     // run; else a warp per row, rows past the resident grid in later rounds
     const int64_t want = FORM == ROW_SPLIT ? a.rows * a.cpr : (a.rows + NTH / 32 - 1) / (NTH / 32);
-    rowreduce_kernel<T, NC, W0, W1, FORM><<<clamp_grid(want, maxg), NTH, 0, s>>>(a);
+    launch_overlapped(kernel, dim3((unsigned)clamp_grid(want, maxg)), NTH, 0, s, a);
 }
 
 template <typename T, int NC, int W0, int W1>
 static int row_launch_t(RowArgs &a, int form, cudaStream_t s) {
     int rc = launch_guard("rowreduce_kernel");
     if (rc != ACCR_OK) return rc;
-    if (form == ROW_SPLIT) {
-        row_form<T, NC, W0, W1, ROW_SPLIT>(a, s);
-    } else if (form == ROW_SEG) {
-        row_form<T, NC, W0, W1, ROW_SEG>(a, s);
-    } else {
-        row_form<T, NC, W0, W1, ROW_SEG_CTA>(a, s);
-    }
+    if (form == ROW_SPLIT) row_form<T, NC, W0, W1, ROW_SPLIT>(a, s);
+    else if (form == ROW_SEG) row_form<T, NC, W0, W1, ROW_SEG>(a, s);
+    else row_form<T, NC, W0, W1, ROW_SEG_CTA>(a, s);
     return launched("rowreduce_kernel");
 }
 

@@ -26,6 +26,7 @@
 #include "common.cuh"
 #include "fold.cuh"
 #include "group.cuh"
+#include "overlap.cuh"
 #include "rows.cuh"
 
 namespace accr {
@@ -52,6 +53,7 @@ template <typename T, int NC, int W0, int W1>
 __global__ void __launch_bounds__(SB) segment_kernel(const __grid_constant__ SegArgs p) {
     constexpr bool E64 = sizeof(T) == 8;
     constexpr int EPV = 16 / (int)sizeof(T);
+    grid_dependency();
     const int lane = threadIdx.x & 31;
     int w[NC];
 #pragma unroll
@@ -134,7 +136,8 @@ struct SegLaunch {
         for (int c = 0; c < NC; ++c) a.neutral[c] = neutral_element<T>(a.cl[c].wcode);
         const int maxg = resident_ctas(segment_kernel<T, NC, W0, W1>, SB, cached);
         const int64_t items = a.nmid + (a.nseg + SEG_PER_WARP - 1) / SEG_PER_WARP;
-        segment_kernel<T, NC, W0, W1><<<clamp_grid((items + SB / 32 - 1) / (SB / 32), maxg), SB, 0, s>>>(a);
+        const int grid = clamp_grid((items + SB / 32 - 1) / (SB / 32), maxg);
+        launch_overlapped(segment_kernel<T, NC, W0, W1>, dim3((unsigned)grid), SB, 0, s, a);
         return launched("segment_kernel");
     }
 };
