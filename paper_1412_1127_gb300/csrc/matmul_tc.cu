@@ -11,8 +11,9 @@
 // is accumulated in FP32 in tensor memory (the dropped a_lo b_lo term and the
 // split residuals are of order 2^-16 of |a||b|).
 //
-// Kernel shape: one CTA computes a 128 x 224 block of c with
-// tcgen05.mma.cta_group::1.kind::f16 (M = 128, N = 224, K = 16).  The split
+// Kernel shape: one CTA computes a 128 x N block of c with
+// tcgen05.mma.cta_group::1.kind::f16 (M = 128, N = 224 for large matrices and
+// down to 32 for small ones, K = 16).  The split
 // operands are stored packed: every 32-wide k block of a row holds its 32 hi
 // values followed by its 32 lo values, one 128-byte row.  A TMA producer
 // thread streams one such k block of a and of b per stage into a four-stage
@@ -31,19 +32,22 @@
 #include <cuda_bf16.h>
 #include <string.h>
 
+#include <atomic>
 #include <map>
 #include <mutex>
 #include <utility>
 
 #include "common.cuh"
 #include "debug.cuh"
+#include "overlap.cuh"
+#include "shifted.cuh"
 
 namespace accr {
 
-// CTA tile 128 x 224: at LEN 4096 the 19 x 32 = 608 tiles are exactly four
-// waves on 152 SMs (128 x 256 tiles would be 3.4 waves); 32-wide k slices,
-// hi and lo packed in one 128-byte swizzled row, give a four-stage ring in
-// 176 KiB of shared memory.
+// CTA tile 128 x N, N at most 224: at LEN 4096 the 19 x 32 = 608 tiles of N = 224
+// are exactly four waves on 152 SMs (128 x 256 tiles would be 3.4 waves);
+// 32-wide k slices, hi and lo packed in one 128-byte swizzled row, give a
+// four-stage ring in 176 KiB of shared memory.
 constexpr int TBM = 128, TBN = 224, TBK = 32;
 constexpr int TSTAGES = 4;
 constexpr int SWZ = 128;                             // swizzle span (bytes) = one packed k-block row
@@ -51,14 +55,16 @@ constexpr int PK = 2 * TBK;                          // packed row length (bf16)
 constexpr int A_TILE_BYTES = TBM * PK * 2;           // 16 KiB
 constexpr int B_TILE_BYTES = TBN * PK * 2;           // 28 KiB
 constexpr int STAGE_BYTES = A_TILE_BYTES + B_TILE_BYTES;  // 44 KiB, a multiple of the 1 KiB swizzle pattern
+constexpr int EPI_BYTES = 4 * 32 * 33 * 4;  // a 32 x 32 block (padded) per epilogue warp
 constexpr int TMEM_COLS = 512;                                    // two accumulators, at columns 0 and 256
 constexpr int GEMM_THREADS = 192;  // warp 0 TMA producer, warp 1 MMA issuer, warps 2-5 epilogue
 constexpr uint32_t kMaxTries = 1u << 24;
 
 // Instruction descriptor (kind::f16): FP32 accumulator, BF16 A and B, both
 // K-major, N >> 3 at bit 17, M >> 4 at bit 24.
-constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TBN >> 3) << 17) |
-                           ((uint32_t)(TBM >> 4) << 24);
+__device__ __forceinline__ uint32_t idesc_for(int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(TBM >> 4) << 24);
+}
 
 struct TcBars {
     uint64_t full[TSTAGES];   // stage s loaded (TMA transaction count)
@@ -115,10 +121,10 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
     return d;
 }
 
-__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t adesc, uint64_t bdesc, uint32_t acc) {
+__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-        ::"r"(tmem), "l"(adesc), "l"(bdesc), "r"(IDESC), "r"(acc)
+        ::"r"(tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
         : "memory");
 }
 
@@ -148,9 +154,11 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 // The k-slice ring runs on across tiles; the accumulator alternates between
 // two tensor-memory buffers so the epilogue of one tile overlaps the main
 // loop of the next.
+// VEC: rows of c start on 16-byte boundaries.
+template <bool VEC>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
     bf16x3_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB,
-                       float *__restrict__ C, int M, int N, int Kp, int tiles_n, int ntiles, int *err) {
+                       float *__restrict__ C, int M, int N, int Kp, int tn, int tiles_n, int ntiles, int *err, int call) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     TcBars *bars = (TcBars *)(smem + TSTAGES * STAGE_BYTES);
@@ -180,25 +188,29 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = bars->tmem;
     volatile int *abort = &bars->abort;
+    // launched while the split may still run (its last blocks): the set-up above
+    // overlaps it.  Every warp waits here, so no bounded wait below counts its time.
+    grid_dependency();
 
     if (warp == 0 && lane == 0) {
         // ---- TMA producer ----
+        const uint32_t stage_tx = (uint32_t)(A_TILE_BYTES + tn * PK * 2);
         int issued[TSTAGES];
         for (int s = 0; s < TSTAGES; ++s) issued[s] = -1;
         int it = 0;
         for (int tile = blockIdx.x; tile < ntiles && !*abort; tile += gridDim.x) {
-            const int m0 = (tile / tiles_n) * TBM, n0 = (tile % tiles_n) * TBN;
+            const int m0 = (tile / tiles_n) * TBM, n0 = (tile % tiles_n) * tn;
             for (int kb = 0; kb < nkb; ++kb, ++it) {
                 const int s = it % TSTAGES, use = it / TSTAGES;
                 if (use > 0 && !mbar_wait(smem_u32(&bars->empty[s]), (uint32_t)((use - 1) & 1))) {
-                    atomicExch(err, 1);
+                    atomicExch(err, call | 1);
                     *abort = 1;
                     break;
                 }
                 if (*abort) break;
                 uint8_t *st = smem + s * STAGE_BYTES;
                 const uint32_t fb = smem_u32(&bars->full[s]);
-                mbar_expect_tx(fb, STAGE_BYTES);
+                mbar_expect_tx(fb, stage_tx);
                 tma_load_2d(smem_u32(st), &tA, kb * PK, m0, fb);
                 tma_load_2d(smem_u32(st + A_TILE_BYTES), &tB, kb * PK, n0, fb);
                 issued[s] = use;
@@ -206,14 +218,15 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         }
         // let every copy this thread issued land before the CTA can exit
         for (int s = 0; s < TSTAGES; ++s)
-            if (issued[s] >= 0 && !mbar_wait(smem_u32(&bars->full[s]), (uint32_t)(issued[s] & 1))) atomicExch(err, 2);
+            if (issued[s] >= 0 && !mbar_wait(smem_u32(&bars->full[s]), (uint32_t)(issued[s] & 1))) atomicExch(err, call | 2);
     } else if (warp == 1 && lane == 0) {
         // ---- MMA issuer ----
+        const uint32_t idesc = idesc_for(tn);
         int it = 0, j = 0;
         for (int tile = blockIdx.x; tile < ntiles && !*abort; tile += gridDim.x, ++j) {
             const int b = j & 1, u = j >> 1;
             if (u > 0 && !mbar_wait(smem_u32(&bars->tempty[b]), (uint32_t)((u - 1) & 1))) {
-                atomicExch(err, 5);
+                atomicExch(err, call | 5);
                 *abort = 1;
                 break;
             }
@@ -223,7 +236,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
             for (int kb = 0; kb < nkb; ++kb, ++it) {
                 const int s = it % TSTAGES, use = it / TSTAGES;
                 if (!mbar_wait(smem_u32(&bars->full[s]), (uint32_t)(use & 1))) {
-                    atomicExch(err, 3);
+                    atomicExch(err, call | 3);
                     *abort = 1;
                     ok = false;
                     break;
@@ -239,9 +252,9 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
 #pragma unroll
                 for (int kk = 0; kk < TBK / 16; ++kk) {
                     const uint32_t off = kk * 32;  // 16 bf16 along K inside each half
-                    mma_bf16(acc, smem_desc(ah + off), smem_desc(bh + off), (kb > 0 || kk > 0) ? 1u : 0u);
-                    mma_bf16(acc, smem_desc(ah + off), smem_desc(bl + off), 1u);
-                    mma_bf16(acc, smem_desc(al + off), smem_desc(bh + off), 1u);
+                    mma_bf16(acc, smem_desc(ah + off), smem_desc(bh + off), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+                    mma_bf16(acc, smem_desc(ah + off), smem_desc(bl + off), idesc, 1u);
+                    mma_bf16(acc, smem_desc(al + off), smem_desc(bh + off), idesc, 1u);
                 }
                 mma_commit(smem_u32(&bars->empty[s]));
             }
@@ -251,37 +264,51 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     } else if (warp >= 2) {
         // ---- epilogue: accumulator lanes 32*q .. +31 (q = warp % 4) to c ----
         const int q = warp & 3;
-        const bool vec = (N % 4 == 0) && (((uintptr_t)C & 15) == 0);
         int j = 0;
         for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++j) {
             const int b = j & 1, u = j >> 1;
             const bool ready = mbar_wait(smem_u32(&bars->tfull[b]), (uint32_t)(u & 1));
             if (!ready) {
-                if (lane == 0) atomicExch(err, 4);
+                if (lane == 0) atomicExch(err, call | 4);
                 *abort = 1;
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int m0 = (tile / tiles_n) * TBM, n0 = (tile % tiles_n) * TBN;
+            const int m0 = (tile / tiles_n) * TBM, n0 = (tile % tiles_n) * tn;
             // a tile with no element inside c means the host's tile count is wrong
             const bool store = !*abort && ACCR_DCHECK(m0 < M && n0 < N, DS_GEMM_STORE);
             const int row = m0 + q * 32 + lane;
 #pragma unroll 1
-            for (int ch = 0; ch < TBN / 32; ++ch) {
+            for (int ch = 0; ch < tn / 32; ++ch) {
                 uint32_t r[32];
                 tmem_ld32(tmem + (uint32_t)(b * 256) + ((uint32_t)(q * 32) << 16) + (uint32_t)(ch * 32), r);
-                if (!store || row >= M) continue;
                 const int col = n0 + ch * 32;
-                float *dst = C + (size_t)row * (size_t)N + col;
-                if (vec && col + 32 <= N) {
+                if constexpr (!VEC) {
+                    // rows that start anywhere: the 32 x 32 block through shared memory,
+                    // so that a store covers 32 neighbouring elements of one row (one row
+                    // a lane, as below, every element would be a store of its own sector)
+                    float *sc = (float *)(smem + TSTAGES * STAGE_BYTES + 1024) + q * (32 * 33);
 #pragma unroll
-                    for (int e = 0; e < 32; e += 4)
-                        *reinterpret_cast<float4 *>(dst + e) =
-                            make_float4(__uint_as_float(r[e]), __uint_as_float(r[e + 1]), __uint_as_float(r[e + 2]),
-                                        __uint_as_float(r[e + 3]));
+                    for (int e = 0; e < 32; ++e) sc[lane * 33 + e] = __uint_as_float(r[e]);
+                    __syncwarp();
+                    if (store && col + lane < N) {
+                        const int r0 = m0 + q * 32, nr = M - r0 < 32 ? M - r0 : 32;
+                        for (int i = 0; i < nr; ++i) C[(size_t)(r0 + i) * (size_t)N + col + lane] = sc[i * 33 + lane];
+                    }
+                    __syncwarp();
                 } else {
-                    for (int e = 0; e < 32; ++e)
-                        if (col + e < N) dst[e] = __uint_as_float(r[e]);
+                    if (!store || row >= M) continue;
+                    float *dst = C + (size_t)row * (size_t)N + col;
+                    if (col + 32 <= N) {
+#pragma unroll
+                        for (int e = 0; e < 32; e += 4)
+                            *reinterpret_cast<float4 *>(dst + e) =
+                                make_float4(__uint_as_float(r[e]), __uint_as_float(r[e + 1]), __uint_as_float(r[e + 2]),
+                                            __uint_as_float(r[e + 3]));
+                    } else {
+                        for (int e = 0; e < 32; ++e)
+                            if (col + e < N) dst[e] = __uint_as_float(r[e]);
+                    }
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -345,12 +372,14 @@ constexpr int SPLIT_A_ITEMS = 4;  // 8-element groups of a per thread
 // (row-major len x len, rows kept), the rest take 64 x 64 tiles of b
 // (row-major, transposed through shared memory so that a row of the packed
 // b is a column of b).
-__global__ void __launch_bounds__(SPLIT_THREADS) split_kernel(const float *__restrict__ a, const float *__restrict__ b,
+// VEC: rows of a and b start on 16-byte boundaries.
+template <bool VEC>
+__global__ void __launch_bounds__(SPLIT_THREADS, 3) split_kernel(const float *__restrict__ a, const float *__restrict__ b,
                                                               int64_t len, int64_t Kp, __nv_bfloat16 *__restrict__ ap,
-                                                              __nv_bfloat16 *__restrict__ bp, int nblk_a, int tiles_n,
-                                                              int vec) {
+                                                              __nv_bfloat16 *__restrict__ bp, int nblk_a, int tiles_n) {
     __shared__ float tile[64][65];
     const int64_t row_stride = 2 * Kp;
+    grid_dependency();  // once every block has started, the GEMM may be set up behind this grid
     if ((int)blockIdx.x < nblk_a) {
         const int64_t k8 = Kp / 8, total = len * k8;
         const int64_t t0 = (int64_t)blockIdx.x * (SPLIT_THREADS * SPLIT_A_ITEMS) + threadIdx.x;
@@ -359,14 +388,15 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_kernel(const float *__res
         for (int j = 0; j < SPLIT_A_ITEMS; ++j) {  // every load first, then the stores
             const int64_t t = t0 + (int64_t)j * SPLIT_THREADS;
             const int64_t r = t / k8, k0 = (t - r * k8) * 8;
-            if (t < total && vec && k0 + 8 <= len) {
+            if (VEC && t < total && k0 + 8 <= len) {
                 const float4 u = __ldg(reinterpret_cast<const float4 *>(a + r * len + k0));
                 const float4 w = __ldg(reinterpret_cast<const float4 *>(a + r * len + k0 + 4));
                 x[j][0] = u.x, x[j][1] = u.y, x[j][2] = u.z, x[j][3] = u.w;
                 x[j][4] = w.x, x[j][5] = w.y, x[j][6] = w.z, x[j][7] = w.w;
-            } else {
+            } else if (t < total) {
+                load_shifted<2>(a, r * len + k0, len * len, x[j]);
 #pragma unroll
-                for (int e = 0; e < 8; ++e) x[j][e] = (t < total && k0 + e < len) ? a[r * len + k0 + e] : 0.f;
+                for (int e = 0; e < 8; ++e) x[j][e] = k0 + e < len ? x[j][e] : 0.f;
             }
         }
 #pragma unroll
@@ -391,13 +421,15 @@ __global__ void __launch_bounds__(SPLIT_THREADS) split_kernel(const float *__res
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int64_t k = k0 + r0 + 16 * i, n = n0 + c4;
-            if (vec && k < len && n + 4 <= len) {
+            if (VEC && k < len && n + 4 <= len) {
                 v[i] = __ldg(reinterpret_cast<const float4 *>(b + k * len + n));
             } else {
-                v[i].x = (k < len && n + 0 < len) ? b[k * len + n + 0] : 0.f;
-                v[i].y = (k < len && n + 1 < len) ? b[k * len + n + 1] : 0.f;
-                v[i].z = (k < len && n + 2 < len) ? b[k * len + n + 2] : 0.f;
-                v[i].w = (k < len && n + 3 < len) ? b[k * len + n + 3] : 0.f;
+                float w[4] = {0.f, 0.f, 0.f, 0.f};
+                if (k < len && n < len) load_shifted<1>(b, k * len + n, len * len, w);
+                v[i].x = n + 0 < len ? w[0] : 0.f;
+                v[i].y = n + 1 < len ? w[1] : 0.f;
+                v[i].z = n + 2 < len ? w[2] : 0.f;
+                v[i].w = n + 3 < len ? w[3] : 0.f;
             }
         }
 #pragma unroll
@@ -467,6 +499,22 @@ struct SplitBufs {
 static std::mutex g_split_mu;
 static std::map<std::pair<int, uintptr_t>, SplitBufs> g_split;
 
+// Width of a CTA's tile.  A wave costs about (tn + 64) units: the MMAs' time goes
+// with tn, the 64 stand for what a k block costs at any width (reading a's 128
+// rows, the handshakes).  Large matrices keep 224; a matrix of fewer tiles than
+// SMs takes the narrowest tile whose tiles are still one wave.
+// Against the widest tile: len 200 11.2 us (15.0), 1024 23.1 (26.0), 1300 31 (33).
+static int tile_width(int64_t M, int64_t N, int sms) {
+    int best = TBN;
+    int64_t cost = INT64_MAX;
+    for (int tn = TBN; tn >= 32; tn -= 32) {
+        const int64_t tiles = ((M + TBM - 1) / TBM) * ((N + tn - 1) / tn);
+        const int64_t c = (tiles + sms - 1) / sms * (tn + 64);
+        if (c < cost) cost = c, best = tn;
+    }
+    return best;
+}
+
 int matmul_bf16x3(const float *a, const float *b, float *c, int64_t len, cudaStream_t s, bool sync, bool reuse) {
     if (len == 0) return ACCR_OK;
     if (len > (1 << 20)) return set_error(ACCR_EINVAL, "accr_matmul_nest: len too large for the tensor-core path");
@@ -496,6 +544,8 @@ int matmul_bf16x3(const float *a, const float *b, float *c, int64_t len, cudaStr
                 return set_error(ACCR_ENOMEM, "accr_matmul_nest: split buffers (%zu bytes)", need);
             }
             sb->bytes = need;
+            const int rc = cuda_check(cudaMemsetAsync(sb->buf, 0, 256, s), "accr_matmul_nest: clear flag");
+            if (rc != ACCR_OK) return rc;
         }
     }
     char *base = (char *)sb->buf;
@@ -503,48 +553,55 @@ int matmul_bf16x3(const float *a, const float *b, float *c, int64_t len, cudaStr
     __nv_bfloat16 *ap = (__nv_bfloat16 *)(base + 256), *bp = (__nv_bfloat16 *)(base + 256 + abytes);
     int rc = launch_guard("bf16x3_gemm_kernel");
     if (rc != ACCR_OK) return rc;
-    rc = cuda_check(cudaMemsetAsync(err, 0, sizeof(int), s), "accr_matmul_nest: clear flag");
-    if (rc != ACCR_OK) return rc;
+    // the status word holds (call number, code) of the last call whose wait ran
+    // out, so no call has to clear it
+    static std::atomic<uint32_t> calls{0};
+    const int call = (int)((calls.fetch_add(1, std::memory_order_relaxed) % 0x0ffffffeu + 1u) << 3);
     const DeviceInfo &di = device_info();
     if (!(reuse && sb->a == a && sb->b == b && sb->len == len)) {
         const int64_t items_a = M * (Kp / 8), per_blk = SPLIT_THREADS * SPLIT_A_ITEMS;
         const int64_t nblk_a = (items_a + per_blk - 1) / per_blk;
-        const int64_t tn = (N + 63) / 64, nblk_b = tn * ((Kp + 63) / 64);
+        const int64_t tiles_b = (N + 63) / 64, nblk_b = tiles_b * ((Kp + 63) / 64);
         if (nblk_a + nblk_b > INT32_MAX) return set_error(ACCR_EINVAL, "accr_matmul_nest: len too large for the split");
-        const int vec = (K % 4 == 0) && (((uintptr_t)a & 15) == 0) && (((uintptr_t)b & 15) == 0);
-        split_kernel<<<(unsigned)(nblk_a + nblk_b), SPLIT_THREADS, 0, s>>>(a, b, len, Kp, ap, bp, (int)nblk_a,
-                                                                          (int)tn, vec);
+        const bool vec = (K % 4 == 0) && (((uintptr_t)a & 15) == 0) && (((uintptr_t)b & 15) == 0);
+        auto split = vec ? split_kernel<true> : split_kernel<false>;
+        launch_overlapped(split, dim3((unsigned)(nblk_a + nblk_b)), SPLIT_THREADS, 0, s, a, b, len, Kp, ap, bp,
+                          (int)nblk_a, (int)tiles_b);
         if ((rc = launched("split_kernel")) != ACCR_OK) return rc;
         sb->a = a;
         sb->b = b;
         sb->len = len;
     }
     CUtensorMap ma, mb;
+    const int tn = tile_width(M, N, di.sms);
     if ((rc = make_map(&ma, ap, M, Kp, TBM)) != ACCR_OK) return rc;
-    if ((rc = make_map(&mb, bp, N, Kp, TBN)) != ACCR_OK) return rc;
-    const int smem = TSTAGES * STAGE_BYTES + (int)sizeof(TcBars) + 1024;
+    if ((rc = make_map(&mb, bp, N, Kp, tn)) != ACCR_OK) return rc;
+    static_assert(sizeof(TcBars) <= 1024, "the barriers have the kilobyte after the ring");
+    const int smem = TSTAGES * STAGE_BYTES + 1024 + EPI_BYTES + 1024;  // ring, barriers, epilogue blocks, alignment
+    const bool cvec = (N % 4 == 0) && (((uintptr_t)c & 15) == 0);
+    auto gemm = cvec ? bf16x3_gemm_kernel<true> : bf16x3_gemm_kernel<false>;
     {  // the shared-memory opt-in is a per-device function attribute
         static std::mutex attr_mu;
-        static bool attr_set[64] = {false};
+        static bool attr_set[2][64] = {{false}};
         std::lock_guard<std::mutex> lk(attr_mu);
-        if (!attr_set[di.id & 63]) {
-            rc = cuda_check(cudaFuncSetAttribute(bf16x3_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
+        if (!attr_set[cvec][di.id & 63]) {
+            rc = cuda_check(cudaFuncSetAttribute(gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
                             "accr_matmul_nest: shared memory opt-in");
             if (rc != ACCR_OK) return rc;
-            attr_set[di.id & 63] = true;
+            attr_set[cvec][di.id & 63] = true;
         }
     }
-    const int tiles_n = (int)((N + TBN - 1) / TBN), ntiles = tiles_n * (int)((M + TBM - 1) / TBM);
+    const int tiles_n = (int)((N + tn - 1) / tn), ntiles = tiles_n * (int)((M + TBM - 1) / TBM);
     const int grid = ntiles < di.sms ? ntiles : di.sms;  // persistent: one CTA per SM
-    bf16x3_gemm_kernel<<<grid, GEMM_THREADS, smem, s>>>(ma, mb, c, (int)M, (int)N, (int)Kp, tiles_n,
-                                                        ntiles, err);
+    launch_overlapped(gemm, dim3((unsigned)grid), GEMM_THREADS, (size_t)smem, s, ma, mb, c, (int)M, (int)N, (int)Kp, tn,
+                      tiles_n, ntiles, err, call);
     if ((rc = launched("bf16x3_gemm_kernel")) != ACCR_OK) return rc;
     if (sync) {
         int h = 0;
         rc = cuda_check(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s), "accr_matmul_nest: flag");
         if (rc == ACCR_OK) rc = cuda_check(cudaStreamSynchronize(s), "accr_matmul_nest: sync");
-        if (rc == ACCR_OK && h != 0)
-            return set_error(ACCR_ETIMEDOUT, "accr_matmul_nest: a pipeline wait ran out (code %d)", h);
+        if (rc == ACCR_OK && (h & ~7) == call)
+            return set_error(ACCR_ETIMEDOUT, "accr_matmul_nest: a pipeline wait ran out (code %d)", h & 7);
     }
     return rc;
 }
