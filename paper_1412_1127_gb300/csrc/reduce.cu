@@ -321,7 +321,7 @@ static int launch_nc(ReduceArgs &a, int grid, cudaStream_t s) {
 }
 
 template <typename T>
-static int grid_for(int nc, int64_t n) {
+static int grid_for(int nc, int64_t n, bool two_level) {
     int maxg;
     switch (nc) {
     case 1: maxg = occupancy_grid<T, 1>(); break;
@@ -333,8 +333,10 @@ static int grid_for(int nc, int64_t n) {
     // Two vectors a thread until the chip is full: a small region's time is the
     // latency of its loads and merges, so it is spread over more SMs first.  Doubles
     // get a whole round a thread: a sum rounds once a chunk (chunk_sum_f64) and once
-    // at each level of the merges, so more threads would mean more error.
-    const int64_t per = (int64_t)RB * (std::is_same<T, double>::value ? RU : 2);
+    // at each level of the merges, so more threads would mean more error; and so does
+    // the two-level form, whose partials the host takes one by one (2^20 int32: 64
+    // partials 20-22 us, 256 27-28).
+    const int64_t per = (int64_t)RB * (two_level || std::is_same<T, double>::value ? RU : 2);
     int64_t want = (nvec + per - 1) / per;
     if (want < 1) want = 1;
     return (int)(want < maxg ? want : maxg);
@@ -342,14 +344,16 @@ static int grid_for(int nc, int64_t n) {
 
 // Grid used for (type, nclauses, n): depends only on these and the device, so
 // floating-point results are reproducible run to run.
-int reduce_grid(int in_type, int nc, int64_t n) {
+static int grid_of(int in_type, int nc, int64_t n, bool two_level) {
     switch (in_type) {
-    case ACCR_I32: return grid_for<int32_t>(nc, n);
-    case ACCR_I64: return grid_for<int64_t>(nc, n);
-    case ACCR_F32: return grid_for<float>(nc, n);
-    default: return grid_for<double>(nc, n);
+    case ACCR_I32: return grid_for<int32_t>(nc, n, two_level);
+    case ACCR_I64: return grid_for<int64_t>(nc, n, two_level);
+    case ACCR_F32: return grid_for<float>(nc, n, two_level);
+    default: return grid_for<double>(nc, n, two_level);
     }
 }
+
+int reduce_grid(int in_type, int nc, int64_t n) { return grid_of(in_type, nc, n, false); }
 
 // Issues the kernel for a region whose clauses are already lowered.
 int reduce_launch(const void *in, int64_t n, int in_type, const ClauseDev *cl, int nc, int two_level,
@@ -414,7 +418,7 @@ extern "C" ACCR_API int accr_reduce(const void *in, int64_t n, int32_t in_type, 
     if (n > 0 && !in) return set_error(ACCR_EINVAL, "accr_reduce: in is NULL");
     if (((uintptr_t)in % (uintptr_t)type_bytes(in_type)) != 0)
         return set_error(ACCR_EINVAL, "accr_reduce: in is not aligned to its element size");
-    const int grid = reduce_grid(in_type, nclauses, n);
+    const int grid = grid_of(in_type, nclauses, n, (flags & ACCR_TWO_LEVEL_HOST) != 0);
     const size_t pbytes = (size_t)nclauses * (size_t)grid * sizeof(Partial);
     log_msg(2, "accr_reduce: n=%lld type=%d clauses=%d grid=%d%s", (long long)n, in_type, nclauses, grid,
             (flags & ACCR_TWO_LEVEL_HOST) ? " (two-level host merge)" : "");
