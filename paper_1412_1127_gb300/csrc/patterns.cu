@@ -104,7 +104,7 @@ __device__ __forceinline__ int grid_barrier_or(unsigned *bar, unsigned &gen, boo
 //
 // Distances are never negative, so their bits order as unsigned integers, with
 // a NaN above infinity: NK_NONE, one above infinity, is "no point yet", and a
-// point whose distance is NaN never enters.  Ten million points, k = 10: 42 -> 24.7 us,
+// point whose distance is NaN never enters.  Ten million points, k = 10: 42 -> 22.8 us,
 // of which the bytes take 11.8 and the last CTA about 6.
 
 constexpr int NK_THREADS = 512;               // two CTAs per SM
@@ -646,7 +646,7 @@ __global__ void __launch_bounds__(SD_THREADS) standardize_kernel(const __grid_co
 // vectors a thread reads stay in registers (20 MB over 152 SMs: an array up to
 // 5 million floats is read once), and the second pass takes the rest of the
 // slice from its end backwards, so that what the first pass read last is still
-// in L2.  2^22 floats: 24.6 -> 15.7 us; what bounds it now is the chain of load, CTA
+// in L2.  2^22 floats: 24.6 -> 16.1 us; what bounds it now is the chain of load, CTA
 // merge, barrier, merge and store, a few microseconds each.
 constexpr int SF_THREADS = 1024;
 constexpr int SF_KEEP = 8;  // 32 of the 64 registers a thread of such a CTA has
