@@ -89,3 +89,19 @@ def test_offsets_past_32_bits():
     api.accr_segmented_reduce(v, off, [api.clause("add", out.t)])
     want = [int(np.arange(a, b).sum()) for a, b in [(0, 0), (0, 10), (10, 1000), (1000, 1001), (1001, 3995), (0, 0), (3995, 4000)]]
     assert out.check("sums").cpu().tolist() == want
+
+
+@pytest.mark.parametrize("t", ["f32", "f64"])
+def test_a_tiled_segment_changes_no_other(t):
+    """Segments above 64 KiB are cut into tiles by a second launch."""
+    eb = 4 if t == "f32" else 8
+    L = np.array([4096 // eb + 1, 300, 65536 // eb, 7, 20000 // eb, 0, 33333 // eb, 200000 // eb], dtype=np.int64)
+    off = inputs.offsets_from_lengths(L) + 1
+    v = torch.from_numpy(inputs.normal(int(off[-1]), np.float32 if t == "f32" else np.float64)).cuda()
+    got = []
+    for n in (len(L), len(L) - 1):  # with the tiled last one, without
+        s, m = torch.zeros(n, dtype=TD[t], device="cuda"), torch.zeros(n, dtype=TD[t], device="cuda")
+        api.accr_segmented_reduce(v, off[:n + 1], [api.clause("add", s), api.clause("min", m)], flags=api.ACCR_SYNC)
+        got.append((s[:len(L) - 1].cpu(), m[:len(L) - 1].cpu()))
+    for a, b in zip(*got):
+        assert torch.equal(a.view(torch.uint8), b.view(torch.uint8))
