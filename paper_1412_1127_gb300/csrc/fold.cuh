@@ -246,10 +246,11 @@ __host__ __device__ __forceinline__ void two_sum_merge(float &s, float &c, float
 // of two -- two FP64-pipe operations per chunk instead of one per value.
 // Bits shifted out are truncated: at most 2^-6 of the largest value's ulp per
 // element (under 0.25 ulp for a chunk of 16).  Zeros and subnormals shift out
-// whole: chunks whose largest exponent is within 60 of the subnormal range, and
-// short chunks, are added as doubles.  Finite inputs only.  (5 of 16 values on the
-// FP64 pipe meanwhile was faster, 2^27 doubles 0.158 ms against 0.160, but
-// rounds a chunk five times instead of once: about 5 % more error.)
+// whole: chunks whose largest exponent is within 60 of the subnormal range, chunks
+// with an infinity or a NaN (which have no such significand), and short chunks are
+// added as doubles.  (5 of 16 values on the FP64 pipe meanwhile was faster, 2^27
+// doubles 0.158 ms against 0.160, but rounds a chunk five times instead of once:
+// about 5 % more error.)
 template <int NV>
 __device__ __forceinline__ double chunk_sum_f64(const uint4 *v) {
     constexpr int E = 2 * NV;
@@ -260,7 +261,9 @@ __device__ __forceinline__ double chunk_sum_f64(const uint4 *v) {
         hi[j] = (j & 1) ? v[j >> 1].w : v[j >> 1].y;
         emax = max(emax, hi[j] & 0x7ff00000u);
     }
-    if (E < 8 || emax < 61u << 20) {  // tiny values: the scale below would leave the normal range
+    // one unsigned compare for both ends: tiny values, whose scale below would leave
+    // the normal range (the difference wraps), and the exponent of infinity and NaN
+    if (E < 8 || emax - (61u << 20) >= (0x7ffu - 61u) << 20) {
         double t = u2d(word64(v[0], 0));
 #pragma unroll
         for (int j = 1; j < E; ++j) t = __dadd_rn(t, u2d(word64(v[j >> 1], j & 1)));
