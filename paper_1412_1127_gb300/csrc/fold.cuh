@@ -251,9 +251,11 @@ __host__ __device__ __forceinline__ void two_sum_merge(float &s, float &c, float
 // added as doubles.  (5 of 16 values on the FP64 pipe meanwhile was faster, 2^27
 // doubles 0.158 ms against 0.160, but rounds a chunk five times instead of once:
 // about 5 % more error.)
+// 16 values at most: 16 aligned magnitudes below 2^59 stay below 2^63.
 template <int NV>
 __device__ __forceinline__ double chunk_sum_f64(const uint4 *v) {
     constexpr int E = 2 * NV;
+    static_assert(E <= 16, "the int64 sum holds 16 magnitudes");
     uint32_t hi[E], lo[E], emax = 0;
 #pragma unroll
     for (int j = 0; j < E; ++j) {
@@ -353,6 +355,7 @@ __device__ __forceinline__ double add_chunk_wide(double a, const uint4 *v) {
 // Fold NV 16-byte vectors of T into A under working code w (warp-uniform).
 template <typename T, int NV>
 __device__ __forceinline__ void fold_vec(int w, Acc &A, const uint4 *v) {
+    static_assert(NV <= 8 || NV % 8 == 0, "double sums take eight vectors at a time");
     if constexpr (std::is_integral<T>::value) {
         using UT = typename std::make_unsigned<T>::type;
         switch (w) {
@@ -430,7 +433,10 @@ __device__ __forceinline__ void fold_vec(int w, Acc &A, const uint4 *v) {
                 }
                 A.a = f2u((p0 + p1) + (p2 + p3));
             } else {
-                A.a = d2u(__dadd_rn(u2d(A.a), chunk_sum_f64<NV>(v)));
+                double a = u2d(A.a);
+#pragma unroll
+                for (int i = 0; i < NV; i += 8) a = __dadd_rn(a, chunk_sum_f64<(NV < 8 ? NV : 8)>(v + i));
+                A.a = d2u(a);
             }
         } break;
         case W_ADDF_COMP: {
