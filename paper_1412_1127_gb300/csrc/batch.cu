@@ -297,6 +297,10 @@ __global__ void __launch_bounds__(BB, MINB) batch_kernel_inline(const __grid_con
 static std::atomic<int64_t> g_small_bytes{ACCR_SMALL_BYTES};
 static std::atomic<int64_t> g_tile_bytes{ACCR_TILE_BYTES};
 
+// What one warp or CTA folds stays below 64 GiB (stream_fold counts vectors in 32 bits).
+constexpr int64_t MAX_STRETCH_BYTES = (int64_t)1 << 35;
+int64_t batch_small_bytes() { return std::min(g_small_bytes.load(), MAX_STRETCH_BYTES); }
+
 struct HostPlan {
     std::vector<RegionDev> regions;
     std::vector<int2> tiles;      // queue order
@@ -563,10 +567,8 @@ struct SegmentSource {
 // descriptor, then tile).
 template <typename Src>
 static int plan_chunked(const Src &src, int64_t n, HostPlan &P) {
-    // (a stretch that one warp or CTA folds stays below 64 GiB: 32-bit vector counts)
-    constexpr int64_t most = (int64_t)1 << 35;
-    const int64_t small_b = std::min(g_small_bytes.load(), most);
-    const int64_t tile_b = std::min(P.tile_override > 0 ? P.tile_override : g_tile_bytes.load(), most);
+    const int64_t small_b = batch_small_bytes();
+    const int64_t tile_b = std::min(P.tile_override > 0 ? P.tile_override : g_tile_bytes.load(), MAX_STRETCH_BYTES);
     P.tile_bytes = tile_b;
     const int nch = n >= PAR_MIN_REGIONS ? 2 * plan_pool().threads() : 1;
     std::vector<PlanChunk> ch((size_t)nch);
@@ -886,8 +888,6 @@ int batch_launch_segments(const void *values, const int64_t *off, const int32_t 
     if (rc != ACCR_OK) return rc;
     return run_once(P, 0, stream);
 }
-
-int64_t batch_small_bytes() { return g_small_bytes.load(); }
 
 int PlanStage::begin(accr_stream_t stream, size_t bytes) {
     bufs = bufs_for(stream);

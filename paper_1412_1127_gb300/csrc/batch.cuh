@@ -19,7 +19,7 @@ struct ClauseDev;
 int batch_launch_segments(const void *values, const int64_t *off, const int32_t *idx, int64_t n, int in_type,
                           const ClauseDev *cl, int nc, accr_stream_t stream);
 
-// Bytes up to which one warp folds a region (accr_batch_tiling).
+// Bytes up to which one warp folds a region (accr_batch_tiling), below 64 GiB.
 int64_t batch_small_bytes();
 
 // A stream's staging for one call's plan: pinned memory to write it into and the

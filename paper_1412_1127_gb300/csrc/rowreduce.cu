@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(row_threads<T, NC, FORM>()) rowreduce_kernel(c
                 const int64_t lo = s * p.chunk;
                 const int64_t len = (cols - lo) < p.chunk ? (cols - lo) : p.chunk;
                 if (!ACCR_DCHECK(lo + len <= cols && s < 32, DS_ROW_CHUNK)) continue;
-                fold_stretch<T, NC, FIXED>((const T *)p.A + r * p.ld + lo, (int)len, p.cl, w, lane, A);
+                fold_stretch<T, NC, FIXED>((const T *)p.A + r * p.ld + lo, len, p.cl, w, lane, A);
 #pragma unroll
                 for (int c = 0; c < NC; ++c) {
                     if (FORM == ROW_SEG) {
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(row_threads<T, NC, FORM>()) rowreduce_kernel(c
         const int64_t r = k / p.cpr, j = k - r * p.cpr, lo = j * p.chunk;
         const int64_t len = (cols - lo) < p.chunk ? (cols - lo) : p.chunk;
         if (!ACCR_DCHECK(r < p.rows && lo + len <= cols, DS_ROW_CHUNK)) continue;
-        fold_stretch<T, NC, FIXED>((const T *)p.A + r * p.ld + lo, (int)len, p.cl, w, lane, A);
+        fold_stretch<T, NC, FIXED>((const T *)p.A + r * p.ld + lo, len, p.cl, w, lane, A);
         if (lane == 0) {
 #pragma unroll
             for (int c = 0; c < NC; ++c) {

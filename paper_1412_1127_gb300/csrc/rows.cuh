@@ -38,10 +38,10 @@ __device__ __forceinline__ uint4 ld_row(const uint4 *p) {
     return v;
 }
 
-// One stretch of `len` elements (at most 64 KiB), folded by one warp and merged
-// across its lanes.
+// One stretch of `len` elements (below 64 GiB, as stream_fold takes), folded by one
+// warp and merged across its lanes.
 template <typename T, int NC, bool FIXED>
-__device__ __forceinline__ void fold_stretch(const T *row, int len, const ClauseDev *cl, const int (&w)[NC], int lane,
+__device__ __forceinline__ void fold_stretch(const T *row, int64_t len, const ClauseDev *cl, const int (&w)[NC], int lane,
                                              Acc (&A)[NC]) {
     constexpr bool E64 = sizeof(T) == 8;
 #pragma unroll

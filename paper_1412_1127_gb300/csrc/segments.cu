@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(SB) segment_kernel(const __grid_constant__ Seg
         if (it < p.nmid) {
             const int64_t s = __ldg(p.mid + it);
             const int64_t lo = seg_offset(p, s), hi = seg_offset(p, s + 1);
-            fold_stretch<T, NC, (W0 >= 0)>((const T *)p.values + lo, (int)(hi - lo), p.cl, w, lane, A);
+            fold_stretch<T, NC, (W0 >= 0)>((const T *)p.values + lo, hi - lo, p.cl, w, lane, A);
             if (lane == 0) store(s, false);
         } else {
             const int64_t s0 = (it - p.nmid) * SEG_PER_WARP;
