@@ -152,23 +152,26 @@ struct LongSegments {
     }
 };
 
-// Checks the offsets [s0, s1] and writes them to dst, relative to off[0] (`narrow`:
-// 32 bits).  Whole blocks are checked by their smallest and largest length;
-// only a block with a longer segment is looked through one by one.
+// Checks the offsets and writes them to dst, relative to off[0] (which is not
+// negative); returns the first segment that ends before it starts, or -1.  Whole
+// blocks are checked by their smallest and largest length and by their offsets'
+// signs (without a negative offset no length overflows); only a block with a
+// longer segment is looked through one by one.
 template <typename O>
 static int64_t copy_offsets(const int64_t *off, int64_t nseg, O *dst, int64_t max_short, int64_t max_mid, LongSegments &L) {
     constexpr int64_t BLK = 512;
     const int64_t base = off[0];
     for (int64_t b = 0; b < nseg; b += BLK) {
         const int64_t e = std::min(nseg, b + BLK);
-        int64_t lo = INT64_MAX, hi = 0;
+        int64_t lo = INT64_MAX, hi = 0, signs = 0;
         for (int64_t s = b; s < e; ++s) {
-            const int64_t n = off[s + 1] - off[s];
+            const int64_t n = (int64_t)((uint64_t)off[s + 1] - (uint64_t)off[s]);
             lo = n < lo ? n : lo;
             hi = n > hi ? n : hi;
-            dst[s] = (O)(off[s] - base);
+            signs |= off[s + 1];
+            dst[s] = (O)((uint64_t)off[s] - (uint64_t)base);
         }
-        if (lo < 0) {
+        if (lo < 0 || signs < 0) {
             for (int64_t s = b; s < e; ++s)
                 if (off[s + 1] < off[s]) return s;
         }
@@ -180,7 +183,7 @@ static int64_t copy_offsets(const int64_t *off, int64_t nseg, O *dst, int64_t ma
             else L.mid[n > 8 * max_short ? 0 : n > 4 * max_short ? 1 : n > 2 * max_short ? 2 : 3].push_back((int32_t)s);
         }
     }
-    dst[nseg] = (O)(off[nseg] - base);
+    dst[nseg] = (O)((uint64_t)off[nseg] - (uint64_t)base);
     return -1;
 }
 
@@ -207,7 +210,7 @@ extern "C" ACCR_API int accr_segmented_reduce(const void *values, const int64_t 
     if (((uintptr_t)values & (uintptr_t)(eb - 1)) != 0)
         return set_error(ACCR_EINVAL, "region 0: in is not aligned to its element size");
     cudaStream_t s = (cudaStream_t)stream;
-    const int64_t total = offsets[nseg] - offsets[0];
+    const int64_t total = (int64_t)((uint64_t)offsets[nseg] - (uint64_t)offsets[0]);
     // (a total below zero, or above what the narrow form holds, takes the wide one;
     // the check below finds decreasing offsets either way)
     const bool wide = total < 0 || total > (int64_t)UINT32_MAX;
