@@ -54,6 +54,15 @@ __device__ __forceinline__ void st_release(unsigned *p, unsigned v) {
 // (generation << 1) | OR of the flags, published by the last CTA to arrive, so
 // the flag comes back with the release instead of through a word of its own.
 // Returns 0 if the wait ran out, else 1 + the OR of the flags.
+//
+// Whether bar[1] shows generation `gen` or one after it.  CTAs that take part in
+// the following barrier keep the word from moving on before they have seen it; one
+// that does not (it only set up) may look late and find a later generation, which
+// must end its wait too (the flag it then reads is not its barrier's: it has no use
+// for it).
+__host__ __device__ __forceinline__ bool generation_reached(unsigned word, unsigned gen) {
+    return (((word >> 1) - gen) & 0x7fffffffu) < 0x40000000u;
+}
 __device__ __forceinline__ int grid_barrier_or(unsigned *bar, unsigned &gen, bool flag, unsigned ctas) {
     __shared__ int s_res;
     __syncthreads();
@@ -70,11 +79,11 @@ __device__ __forceinline__ int grid_barrier_or(unsigned *bar, unsigned &gen, boo
         } else {
             uint32_t i = 0;
             unsigned v = ld_acquire(&bar[1]);
-            while ((v >> 1) != my && ++i <= kSpinLimit) {
+            while (!generation_reached(v, my) && ++i <= kSpinLimit) {
                 if (i > 256) __nanosleep(64);
                 v = ld_acquire(&bar[1]);
             }
-            if ((v >> 1) == my) res = 1 + (int)(v & 1u);
+            if (generation_reached(v, my)) res = 1 + (int)(v & 1u);
         }
         s_res = res;
     }
