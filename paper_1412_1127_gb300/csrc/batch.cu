@@ -789,7 +789,7 @@ static int grow(StreamBufs *B, size_t bytes, size_t words, cudaStream_t s) {
             cudaGetLastError();
             return set_error(ACCR_ENOMEM, "batch: cudaMalloc of counters failed");
         }
-        rc = cuda_check(cudaMemset(B->counters, 0, want * 4), "batch: clear counters");
+        rc = clear_device(B->counters, want * 4, "batch: clear counters");
         if (rc != ACCR_OK) return rc;
         B->ncounters = want;
     }
@@ -983,9 +983,8 @@ extern "C" ACCR_API int accr_batch_create(const accr_region *regions, int64_t nr
     }
     std::vector<char> host(P.plan_bytes);
     write_plan(P, host.data());
-    if ((rc = cuda_check(cudaMemcpy(b->dev, host.data(), P.plan_bytes, cudaMemcpyHostToDevice), "accr_batch_create: upload")) != ACCR_OK)
-        return fail(rc);
-    if ((rc = cuda_check(cudaMemset(b->counters, 0, R * 4), "accr_batch_create: counters")) != ACCR_OK) return fail(rc);
+    if ((rc = upload_device(b->dev, host.data(), P.plan_bytes, "accr_batch_create: upload")) != ACCR_OK) return fail(rc);
+    if ((rc = clear_device(b->counters, R * 4, "accr_batch_create: counters")) != ACCR_OK) return fail(rc);
     if ((rc = cuda_check(cudaEventCreateWithFlags(&b->done, cudaEventDisableTiming), "accr_batch_create: event")) != ACCR_OK)
         return fail(rc);
     if (P.regions.empty()) {

@@ -73,6 +73,13 @@ void *host_staging_for(accr_stream_t stream, size_t bytes);
 // zero before it exits.  Returns nullptr (and sets the error) on failure.
 unsigned *zeroed_words_for(accr_stream_t stream, size_t n);
 
+// Zeroes device memory / copies host memory to it and waits for that, on a stream of
+// their own: work queued afterwards on any stream finds it done.  (cudaMemset, and
+// cudaMemcpy from pageable memory, run on the legacy default stream, may return before
+// they are done, and are not ordered with non-blocking streams.)
+int clear_device(void *p, size_t bytes, const char *where);
+int upload_device(void *p, const void *host, size_t bytes, const char *where);
+
 // ---- types ----------------------------------------------------------------
 inline int type_bytes(int t) { return (t == ACCR_I32 || t == ACCR_F32) ? 4 : 8; }
 inline bool type_is_int(int t) { return t == ACCR_I32 || t == ACCR_I64; }

@@ -116,6 +116,31 @@ const DeviceInfo &device_info() {
     return ref;
 }
 
+// ---- eager clears and uploads -----------------------------------------------
+static int on_own_stream(const char *where, cudaError_t (*f)(void *, const void *, size_t, cudaStream_t), void *p,
+                         const void *host, size_t bytes) {
+    if (bytes == 0) return ACCR_OK;
+    cudaStream_t s;
+    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return cuda_check(e, where);
+    e = f(p, host, bytes, s);
+    const cudaError_t w = cudaStreamSynchronize(s);
+    cudaStreamDestroy(s);
+    return cuda_check(e != cudaSuccess ? e : w, where);
+}
+
+int clear_device(void *p, size_t bytes, const char *where) {
+    return on_own_stream(
+        where, [](void *d, const void *, size_t n, cudaStream_t s) { return cudaMemsetAsync(d, 0, n, s); }, p, nullptr, bytes);
+}
+
+int upload_device(void *p, const void *host, size_t bytes, const char *where) {
+    return on_own_stream(
+        where,
+        [](void *d, const void *h, size_t n, cudaStream_t s) { return cudaMemcpyAsync(d, h, n, cudaMemcpyHostToDevice, s); },
+        p, host, bytes);
+}
+
 // ---- scratch -----------------------------------------------------------------
 struct ScratchEntry {
     Scratch s{};
@@ -190,7 +215,7 @@ Scratch *scratch_for(accr_stream_t stream, size_t bytes) {
         set_error(ACCR_ENOMEM, "scratch: cudaMalloc of %zu bytes failed", head + want);
         return nullptr;
     }
-    if (cuda_check(cudaMemset(p, 0, head), "scratch clear") != ACCR_OK) {
+    if (clear_device(p, head, "scratch clear") != ACCR_OK) {
         cudaFree(p);
         return nullptr;
     }
