@@ -87,14 +87,6 @@ struct BatchArgs {
     unsigned *queue;             // [3] next tile, next warp region, CTAs done
 };
 
-__device__ __forceinline__ uint4 ld_batch(const uint4 *p) {
-    uint4 v;
-    asm("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4];"
-        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-        : "l"(p));
-    return v;
-}
-
 __device__ __forceinline__ Partial ld_partial_cg(const Partial *p) {
     uint4 v = __ldcg(reinterpret_cast<const uint4 *>(p));
     Partial q;
@@ -129,7 +121,7 @@ __device__ __noinline__ void tile_fold(const BatchArgs &p, const RegionDev *d, i
         A[c].a = id[c];
         A[c].c = 0.f;
     }
-    stream_fold<T, NC, BU, BB>(in, len, (int)threadIdx.x, w, A, ld_batch);
+    stream_fold<T, NC, BU, BB>(in, len, (int)threadIdx.x, w, A, ld_stream);
     cta_merge<NC, BB>(w, id, E64, A, sh);
 
     if (ntiles == 1) {
@@ -197,7 +189,7 @@ __device__ __noinline__ void warp_fold(const RegionDev *d, int lane) {
         A[c].a = d->cl[c].ident;
         A[c].c = 0.f;
     }
-    stream_fold<T, NC, SU, 32>(in, n, lane, w, A, ld_batch);
+    stream_fold<T, NC, SU, 32>(in, n, lane, w, A, ld_stream);
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
         warp_merge(w[c], E64, A[c]);

@@ -97,10 +97,10 @@ __device__ __forceinline__ void group_fold(const T *in, int len, bool live, int 
 #pragma unroll
     for (int u = 0; u < GV; ++u) {
         ok[u] = u < rounds && u * L + l < nvec;
-        if (ok[u]) b[u] = __ldg(vr + u * L);
+        if (ok[u]) b[u] = vr[u * L];
     }
-    if (l < head) h = __ldg(in + l);
-    if (tail0 + l < end) t = __ldg(in + tail0 + l);
+    if (l < head) h = in[l];
+    if (tail0 + l < end) t = in[tail0 + l];
     if constexpr (PAIR) {
         GroupFold<T, W0> F0;
         GroupFold<T, W1> F1;
@@ -116,8 +116,8 @@ __device__ __forceinline__ void group_fold(const T *in, int len, bool live, int 
         if (l < head) F0.one(h), F1.one(h);
         if (tail0 + l < end) F0.one(t), F1.one(t);
         if (L < EPV) {  // fewer lanes than a head or tail may have elements
-            for (int j = L + l; j < head; j += L) F0.one(__ldg(in + j)), F1.one(__ldg(in + j));
-            for (int j = tail0 + L + l; j < end; j += L) F0.one(__ldg(in + j)), F1.one(__ldg(in + j));
+            for (int j = L + l; j < head; j += L) F0.one(in[j]), F1.one(in[j]);
+            for (int j = tail0 + L + l; j < end; j += L) F0.one(in[j]), F1.one(in[j]);
         }
         A[0] = F0.get();
         A[1] = F1.get();
@@ -128,8 +128,8 @@ __device__ __forceinline__ void group_fold(const T *in, int len, bool live, int 
             A[c].c = 0.f;
             if (rounds > GV / 2) fold_filled<T, GV, GV>(w[c], A[c], b, ok, neutral[c]);
             else if (rounds > 0) fold_filled<T, GV / 2, GV>(w[c], A[c], b, ok, neutral[c]);
-            for (int j = l; j < head; j += L) fold_one<T>(w[c], A[c], j == l ? h : __ldg(in + j));
-            for (int j = tail0 + l; j < end; j += L) fold_one<T>(w[c], A[c], j == tail0 + l ? t : __ldg(in + j));
+            for (int j = l; j < head; j += L) fold_one<T>(w[c], A[c], j == l ? h : in[j]);
+            for (int j = tail0 + l; j < end; j += L) fold_one<T>(w[c], A[c], j == tail0 + l ? t : in[j]);
         }
     }
 #pragma unroll

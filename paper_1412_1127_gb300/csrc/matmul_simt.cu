@@ -43,7 +43,7 @@ __device__ __forceinline__ int a_col(int r, int k) {
 
 template <bool SERIAL, bool VEC, int BM, int BN, int TR, int TC>
 __global__ void __launch_bounds__(BM * BN / (TR * TC), 512 / (BM * BN / (TR * TC)))
-    matmul_simt_kernel(const float *__restrict__ a, const float *__restrict__ b, float *__restrict__ c, int64_t len) {
+    matmul_simt_kernel(const float *a, const float *b, float *c, int64_t len) {
     constexpr int NTH = BM * BN / (TR * TC);  // threads
     constexpr int QR = TR / 4, QC = TC / 4;   // runs of 4 a side
     constexpr int LA = BM * KT / 4 / NTH, LB = BN * KT / 4 / NTH;  // float4 loads per thread and slice
@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(BM * BN / (TR * TC), 512 / (BM * BN / (TR * TC
     auto load_a = [&](int64_t k0, int h, float4 &v) {
         const int64_t r = row0 + a_r + h * (NTH / 4), k = k0 + a_k;
         if (VEC && r < len && k + 3 < len) {
-            v = __ldg(reinterpret_cast<const float4 *>(a + r * len + k));
+            v = *reinterpret_cast<const float4 *>(a + r * len + k);
         } else {
             v.x = (r < len && k + 0 < len) ? a[r * len + k + 0] : 0.f;
             v.y = (r < len && k + 1 < len) ? a[r * len + k + 1] : 0.f;
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(BM * BN / (TR * TC), 512 / (BM * BN / (TR * TC
         const int i = tid + h * NTH;
         const int64_t k = k0 + i / (BN / 4), cc = col0 + (i % (BN / 4)) * 4;
         if (VEC && k < len && cc + 3 < len) {
-            v = __ldg(reinterpret_cast<const float4 *>(b + k * len + cc));
+            v = *reinterpret_cast<const float4 *>(b + k * len + cc);
         } else {
             v.x = (k < len && cc + 0 < len) ? b[k * len + cc + 0] : 0.f;
             v.y = (k < len && cc + 1 < len) ? b[k * len + cc + 1] : 0.f;

@@ -158,7 +158,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 template <bool VEC>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
     bf16x3_gemm_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB,
-                       float *__restrict__ C, int M, int N, int Kp, int tn, int tiles_n, int ntiles, int *err, int call) {
+                       float *C, int M, int N, int Kp, int tn, int tiles_n, int ntiles, int *err, int call) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     TcBars *bars = (TcBars *)(smem + TSTAGES * STAGE_BYTES);
@@ -374,9 +374,9 @@ constexpr int SPLIT_A_ITEMS = 4;  // 8-element groups of a per thread
 // b is a column of b).
 // VEC: rows of a and b start on 16-byte boundaries.
 template <bool VEC>
-__global__ void __launch_bounds__(SPLIT_THREADS, 3) split_kernel(const float *__restrict__ a, const float *__restrict__ b,
-                                                              int64_t len, int64_t Kp, __nv_bfloat16 *__restrict__ ap,
-                                                              __nv_bfloat16 *__restrict__ bp, int nblk_a, int tiles_n) {
+__global__ void __launch_bounds__(SPLIT_THREADS, 3) split_kernel(const float *a, const float *b,
+                                                              int64_t len, int64_t Kp, __nv_bfloat16 *ap,
+                                                              __nv_bfloat16 *bp, int nblk_a, int tiles_n) {
     __shared__ float tile[64][65];
     const int64_t row_stride = 2 * Kp;
     grid_dependency();  // once every block has started, the GEMM may be set up behind this grid
@@ -389,8 +389,8 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 3) split_kernel(const float *__
             const int64_t t = t0 + (int64_t)j * SPLIT_THREADS;
             const int64_t r = t / k8, k0 = (t - r * k8) * 8;
             if (VEC && t < total && k0 + 8 <= len) {
-                const float4 u = __ldg(reinterpret_cast<const float4 *>(a + r * len + k0));
-                const float4 w = __ldg(reinterpret_cast<const float4 *>(a + r * len + k0 + 4));
+                const float4 u = *reinterpret_cast<const float4 *>(a + r * len + k0);
+                const float4 w = *reinterpret_cast<const float4 *>(a + r * len + k0 + 4);
                 x[j][0] = u.x, x[j][1] = u.y, x[j][2] = u.z, x[j][3] = u.w;
                 x[j][4] = w.x, x[j][5] = w.y, x[j][6] = w.z, x[j][7] = w.w;
             } else if (t < total) {
@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 3) split_kernel(const float *__
         for (int i = 0; i < 4; ++i) {
             const int64_t k = k0 + r0 + 16 * i, n = n0 + c4;
             if (VEC && k < len && n + 4 <= len) {
-                v[i] = __ldg(reinterpret_cast<const float4 *>(b + k * len + n));
+                v[i] = *reinterpret_cast<const float4 *>(b + k * len + n);
             } else {
                 float w[4] = {0.f, 0.f, 0.f, 0.f};
                 if (k < len && n < len) load_shifted<1>(b, k * len + n, len * len, w);

@@ -23,6 +23,21 @@ __device__ __forceinline__ void grid_dependency() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Inputs are read by ordinary loads, not by the read-only path (ld.global.nc, __ldg,
+// const __restrict__ parameters): PTX defines that for memory nothing writes while
+// the kernel lives, and this kernel's life begins while its predecessor may still be
+// writing.  A streaming 16-byte load (read once: no L1 allocation, 256-byte L2
+// fetch), volatile with a memory clobber so that none moves above the wait.  Its rate
+// is the read-only path's (2^28 floats, sum + max + min: 158.1 us both ways).
+__device__ __forceinline__ uint4 ld_stream(const uint4 *p) {
+    uint4 v;
+    asm volatile("ld.global.L1::no_allocate.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p)
+                 : "memory");
+    return v;
+}
+
 template <typename T>
 struct SameType {
     using type = T;

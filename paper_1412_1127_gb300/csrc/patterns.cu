@@ -135,13 +135,10 @@ __device__ __forceinline__ bool pless(uint32_t da, int64_t ia, uint32_t db, int6
     return da < db || (da == db && ia < ib);
 }
 
-// Streaming 16-byte load of two points (read once: no L1 allocation).
+// Two points.
 __device__ __forceinline__ float4 ld_pts(const float4 *p) {
-    float4 v;
-    asm("ld.global.nc.L1::no_allocate.L2::256B.v4.f32 {%0,%1,%2,%3}, [%4];"
-        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-        : "l"(p));
-    return v;
+    const uint4 v = ld_stream(reinterpret_cast<const uint4 *>(p));
+    return make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
 }
 
 __device__ __forceinline__ uint32_t sqdist(float x, float y, float qx, float qy) {
@@ -779,7 +776,7 @@ __global__ void bfs_init_kernel(int32_t *dist, int64_t total, int64_t src, const
 // One level of the pull formulation over the thread's cells, CU cells at a
 // time with every load of a group issued before any is tested: the level is
 // bound by L2 latency, not bandwidth, at the sizes of the BFS workloads.
-__device__ __forceinline__ bool bfs_level(const uint8_t *__restrict__ open, int32_t *dist, int64_t rows,
+__device__ __forceinline__ bool bfs_level(const uint8_t *open, int32_t *dist, int64_t rows,
                                           int64_t cols, int32_t L) {
     constexpr int CU = 4;
     const int64_t total = rows * cols;  // < 2^31 (checked on the host): 32-bit cell arithmetic
@@ -793,7 +790,7 @@ __device__ __forceinline__ bool bfs_level(const uint8_t *__restrict__ open, int3
         for (int j = 0; j < CU; ++j) {
             const int64_t c = c0 + j * nth;
             d[j] = c < total ? __ldcg(dist + c) : 0;
-            need[j] = c < total && __ldg(open + c) != 0;
+            need[j] = c < total && open[c] != 0;
         }
         int32_t nb[CU][4];
 #pragma unroll
@@ -824,7 +821,7 @@ __device__ __forceinline__ bool bfs_level(const uint8_t *__restrict__ open, int3
 // before in the group: once a level changed nothing, the ones after it return.
 constexpr int BFS_GROUP = 8;
 
-__global__ void __launch_bounds__(BF_THREADS) bfs_level_kernel(const uint8_t *__restrict__ open, int32_t *dist,
+__global__ void __launch_bounds__(BF_THREADS) bfs_level_kernel(const uint8_t *open, int32_t *dist,
                                                                int64_t rows, int64_t cols, int32_t L, int mode,
                                                                unsigned *more, const unsigned *before, unsigned *next,
                                                                unsigned *partial, unsigned *counter) {
@@ -863,7 +860,7 @@ __global__ void __launch_bounds__(BF_THREADS) bfs_level_kernel(const uint8_t *__
 // One CTA of BFP_THREADS per SM (fewer arrivals per grid barrier) and one
 // barrier per level, which also carries the level's `||` flag: every CTA
 // learns whether any cell changed from the barrier's release itself.
-__global__ void __launch_bounds__(BFP_THREADS, 1) bfs_persistent_kernel(const uint8_t *__restrict__ open, int32_t *dist,
+__global__ void __launch_bounds__(BFP_THREADS, 1) bfs_persistent_kernel(const uint8_t *open, int32_t *dist,
                                                                        int64_t rows, int64_t cols,
                                                                        int64_t max_levels, unsigned *bar,
                                                                        int64_t *levels_out, int *err) {

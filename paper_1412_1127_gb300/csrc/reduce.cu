@@ -44,15 +44,6 @@ struct ReduceArgs {
     unsigned *counter;           // zero on entry; zero again on exit
 };
 
-// 16-byte streaming load: read-only path, no L1 allocation, 256-byte L2 fetch.
-__device__ __forceinline__ uint4 ld_stream(const uint4 *p) {
-    uint4 v;
-    asm("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4];"
-        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-        : "l"(p));
-    return v;
-}
-
 __device__ __forceinline__ Partial ld_partial(const Partial *p) {
     uint4 v = __ldcg(reinterpret_cast<const uint4 *>(p));
     Partial q;

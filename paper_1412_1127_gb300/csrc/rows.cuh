@@ -8,6 +8,7 @@
 
 #include "common.cuh"
 #include "fold.cuh"
+#include "overlap.cuh"
 
 namespace accr {
 
@@ -30,13 +31,6 @@ struct RowArgs {
 #define ACCR_ROW_RU 8
 #endif
 constexpr int RU2 = ACCR_ROW_RU;
-__device__ __forceinline__ uint4 ld_row(const uint4 *p) {
-    uint4 v;
-    asm("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0,%1,%2,%3}, [%4];"
-        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-        : "l"(p));
-    return v;
-}
 
 // One stretch of `len` elements (below 64 GiB, as stream_fold takes), folded by one
 // warp and merged across its lanes.
@@ -49,7 +43,7 @@ __device__ __forceinline__ void fold_stretch(const T *row, int64_t len, const Cl
         A[c].a = cl[c].ident;
         A[c].c = 0.f;
     }
-    stream_fold<T, NC, RU2, 32>(row, len, lane, w, A, ld_row);
+    stream_fold<T, NC, RU2, 32>(row, len, lane, w, A, ld_stream);
 #pragma unroll
     for (int c = 0; c < NC; ++c) warp_merge<FIXED>(w[c], E64, A[c]);
 }

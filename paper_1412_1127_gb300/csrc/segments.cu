@@ -46,7 +46,7 @@ struct SegArgs {
 };
 
 __device__ __forceinline__ int64_t seg_offset(const SegArgs &p, int64_t i) {
-    return p.wide_off ? __ldg((const long long *)p.off + i) : (int64_t)__ldg((const uint32_t *)p.off + i);
+    return p.wide_off ? ((const int64_t *)p.off)[i] : (int64_t)((const uint32_t *)p.off)[i];
 }
 
 template <typename T, int NC, int W0, int W1>
@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(SB) segment_kernel(const __grid_constant__ Seg
     while (it < items) {
         if (lane == 0) q = atomicAdd(&p.queue[0], 1u);
         if (it < p.nmid) {
-            const int64_t s = __ldg(p.mid + it);
+            const int64_t s = p.mid[it];
             const int64_t lo = seg_offset(p, s), hi = seg_offset(p, s + 1);
             fold_stretch<T, NC, (W0 >= 0)>((const T *)p.values + lo, hi - lo, p.cl, w, lane, A);
             if (lane == 0) store(s, false);

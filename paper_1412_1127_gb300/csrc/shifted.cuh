@@ -12,7 +12,7 @@ namespace accr {
 // than that of 4096.  Vectors that reach outside x[0, total) go element by element;
 // elements there are not needed by the caller and read as zero.
 template <int NV>
-__device__ __forceinline__ void load_shifted(const float *__restrict__ x, int64_t i, int64_t total, float (&out)[4 * NV]) {
+__device__ __forceinline__ void load_shifted(const float *x, int64_t i, int64_t total, float (&out)[4 * NV]) {
     const int m = (int)(((uintptr_t)(x + i) >> 2) & 3);  // elements before x[i] in its vector
     const int64_t v0 = i - m;
     float w[4 * NV + 4];
@@ -20,11 +20,11 @@ __device__ __forceinline__ void load_shifted(const float *__restrict__ x, int64_
     for (int j = 0; j <= NV; ++j) {
         const int64_t e = v0 + 4 * j;
         if (e >= 0 && e + 4 <= total) {
-            const float4 q = (j < NV || m > 0) ? __ldg(reinterpret_cast<const float4 *>(x + e)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 q = (j < NV || m > 0) ? *reinterpret_cast<const float4 *>(x + e) : make_float4(0.f, 0.f, 0.f, 0.f);
             w[4 * j] = q.x, w[4 * j + 1] = q.y, w[4 * j + 2] = q.z, w[4 * j + 3] = q.w;
         } else {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) w[4 * j + k] = (e + k >= 0 && e + k < total) ? __ldg(x + e + k) : 0.f;
+            for (int k = 0; k < 4; ++k) w[4 * j + k] = (e + k >= 0 && e + k < total) ? x[e + k] : 0.f;
         }
     }
     if (m & 1) {
