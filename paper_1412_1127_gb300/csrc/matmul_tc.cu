@@ -177,6 +177,12 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
         bars->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    // Launched while the predecessor may still run: the set-up above overlaps it.  Every
+    // warp waits here, so no bounded wait below counts its time, and the tensor memory is
+    // taken after the wait: the allocation waits without a limit, and with a reused split
+    // the predecessor may be anybody's kernel, which could need the tensor memory that
+    // this CTA would hold while it waits.
+    grid_dependency();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bars->tmem)),
                      "r"(TMEM_COLS)
@@ -188,9 +194,6 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = bars->tmem;
     volatile int *abort = &bars->abort;
-    // launched while the split may still run (its last blocks): the set-up above
-    // overlaps it.  Every warp waits here, so no bounded wait below counts its time.
-    grid_dependency();
 
     if (warp == 0 && lane == 0) {
         // ---- TMA producer ----

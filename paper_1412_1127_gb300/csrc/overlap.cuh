@@ -14,10 +14,11 @@
 
 namespace accr {
 
-// First statement of a kernel launched with launch_overlapped: waits until the
-// previous kernel of the stream has finished and its writes are visible (nothing
-// of this kernel's inputs, outputs or scratch is touched before), then lets the
-// stream's next kernel be set up in turn.
+// In a kernel launched with launch_overlapped, ahead of everything but a CTA's set-up
+// of its own shared memory: waits until the previous kernel of the stream has finished
+// and its writes are visible, then lets the stream's next kernel be set up in turn.
+// Nothing of this kernel's inputs, outputs or scratch is touched before, and nothing
+// is held that a predecessor could wait for (tensor memory).
 __device__ __forceinline__ void grid_dependency() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -42,3 +42,11 @@ def test_streaming_loads_stay_behind_the_wait():
     for f in glob.glob(os.path.join(build.CSRC, "*.cu*")):
         for m in re.finditer(r"asm( volatile)?\(\s*\"ld\.global[^;]*;\"(.*?)\);", open(f).read(), re.S):
             assert m.group(1) and '"memory"' in m.group(2), (os.path.basename(f), m.group(0)[:80])
+
+
+def test_tensor_memory_is_taken_behind_the_wait():
+    """Its allocation waits without a limit: no CTA holds any while it waits for a
+    predecessor that may want some."""
+    text = re.sub(r"//[^\n]*", "", open(os.path.join(build.CSRC, "matmul_tc.cu")).read())
+    body = text[text.index("bf16x3_gemm_kernel("):text.index("split_kernel(")]
+    assert 0 < body.index("grid_dependency()") < body.index("tcgen05.alloc")
