@@ -111,6 +111,13 @@ __device__ __forceinline__ int grid_barrier_or(unsigned *bar, unsigned &gen, boo
 //   * the candidates are ranked by (distance, index).  If there are ever more
 //     than the array holds, the k best of them stay and the k-th is the new bound.
 //
+// The shares' bound is loose where the points' order keeps the near ones in a few
+// of them (a raster 1,024 wide holds a range of columns in each).  Where many warps
+// are within it, the k-th nearest of all warps' points takes its place, and where many
+// threads are left, the k-th nearest of theirs: k rounds of a minimum over the CTA each.
+// 1024 x 1024 raster points, k = 10: 24 us (445 with the shares alone, 8.6 shuffled),
+// 9766 x 1024 32 (600, 16.5).
+//
 // Distances are never negative, so their bits order as unsigned integers, with
 // a NaN above infinity: NK_NONE, one above infinity, is "no point yet", and a
 // point whose distance is NaN never enters.  Ten million points, k = 10: 42 -> 22.8 us,
@@ -122,6 +129,8 @@ constexpr int NK_U = 8;                       // 16-byte vectors (two points eac
 constexpr uint32_t NK_NONE = 0x7f800001u;
 constexpr int NK_BATCH = 64;                  // warps whose threads are looked at together
 constexpr int NK_CAND = 1536;                 // candidates held: one pass adds at most 64 a warp
+constexpr int NK_LOOSE = 2 * NK_BATCH;        // more warps than this within the bound: it is tightened
+constexpr int NK_PASSES = 8;                  // and so it is before more passes than this
 constexpr int NK_MAX_WARPS = 5120;            // warps of the scan (the grid is bounded accordingly: 320 CTAs)
 
 struct __align__(16) PairSlot {
@@ -173,7 +182,7 @@ struct NearestArgs {
 
 struct NearestShared {
     uint16_t warps[NK_MAX_WARPS];
-    uint32_t units[NK_BATCH * 32];
+    uint32_t units[NK_BATCH * 32], ud[NK_BATCH * 32];  // threads to look at, their smallest distances
     int64_t ci[NK_CAND];
     uint32_t cd[NK_CAND];
     int64_t gi[NK_WARPS];
@@ -202,10 +211,81 @@ __device__ __forceinline__ int nk_rank(const NearestShared &s, int c, int n) {
     return r;
 }
 
+// The k-th smallest of the CTA's (distance, index) pairs, N a thread, all different
+// (NK_NONE: none; there are at least k): k rounds, each the smallest pair past the last.
+template <int N>
+__device__ __forceinline__ void nk_kth(NearestShared &s, const uint32_t (&dv)[N], const int64_t (&iv)[N], int k, uint32_t &kd,
+                                       int64_t &ki) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    kd = 0u, ki = -1;
+    for (int r = 0; r < k; ++r) {
+        uint32_t d = NK_NONE;
+        int64_t i = INT64_MAX;
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+            if (pless(kd, ki, dv[j], iv[j]) && pless(dv[j], iv[j], d, i)) d = dv[j], i = iv[j];
+        warp_min_pair(d, i);
+        if (lane == 0) s.gd[warp] = d, s.gi[warp] = i;
+        __syncthreads();
+        kd = s.gd[lane % NK_WARPS], ki = s.gi[lane % NK_WARPS];
+        warp_min_pair(kd, ki);
+        __syncthreads();
+    }
+}
+
+// A warp's nearest point, as the scan stored it.
+__device__ __forceinline__ void nk_warp_min(const NearestArgs &p, int w, uint32_t &d, int64_t &i) {
+    const int W = (int)gridDim.x * NK_WARPS;
+    const uint4 r = w < W ? __ldcg(reinterpret_cast<const uint4 *>(p.wmin + w)) : make_uint4(~0u, ~0u >> 1, NK_NONE, 0u);
+    d = r.z;
+    i = (int64_t)(((uint64_t)r.y << 32) | r.x);
+}
+
+// The two tightenings, out of line: few calls need them, and their code in the
+// select's own cost every call 0.3 us.
+__device__ __noinline__ void nk_tighten_warps(const NearestArgs &p, NearestShared &s) {
+    constexpr int NW = NK_MAX_WARPS / NK_THREADS;
+    const int t = threadIdx.x;
+    uint32_t wd[NW], d;
+    int64_t wi[NW], i;
+#pragma unroll
+    for (int j = 0; j < NW; ++j) nk_warp_min(p, t + j * NK_THREADS, wd[j], wi[j]);
+    nk_kth(s, wd, wi, p.k, d, i);
+    if (t == 0) s.nwarps = 0, s.bd = d, s.bi = i;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < NW; ++j)
+        if (wd[j] < NK_NONE && !pless(d, i, wd[j], wi[j])) s.warps[atomicAdd(&s.nwarps, 1)] = (uint16_t)(t + j * NK_THREADS);
+    __syncthreads();
+}
+
+__device__ __noinline__ void nk_tighten_units(const NearestArgs &p, NearestShared &s) {
+    constexpr int N = NK_BATCH * 32 / NK_THREADS;
+    const int t = threadIdx.x, nu = s.nunits;
+    uint32_t ud[N], un[N], d;
+    int64_t at[N], i;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        const int c = t + j * NK_THREADS;
+        un[j] = c < nu ? s.units[c] : 0u;
+        ud[j] = c < nu ? s.ud[c] : NK_NONE;
+        at[j] = c < nu ? (int64_t)c : INT64_MAX;
+    }
+    nk_kth(s, ud, at, p.k, d, i);
+    if (t == 0) {
+        s.nunits = 0;
+        if (d < s.bd) s.bd = d, s.bi = INT64_MAX;  // k points within d
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < N; ++j)
+        if (ud[j] < NK_NONE && ud[j] <= s.bd) s.units[atomicAdd(&s.nunits, 1)] = un[j];
+    __syncthreads();
+}
+
 // The last CTA: the k nearest of all points, from the threads' nearest ones.
 __device__ __noinline__ void nearest_select(const NearestArgs &p, NearestShared &s) {
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int W = (int)gridDim.x * NK_WARPS;
     const int64_t head = (((uintptr_t)p.pts & 15) != 0 && p.n > 0) ? 1 : 0;
     const float4 *v4 = (const float4 *)(p.pts + 2 * head);
     const int64_t npairs = (p.n - head) / 2, last = head + 2 * npairs;
@@ -218,12 +298,7 @@ __device__ __noinline__ void nearest_select(const NearestArgs &p, NearestShared 
     uint32_t d = NK_NONE;
     int64_t i = INT64_MAX;
 #pragma unroll
-    for (int j = 0; j < NW; ++j) {
-        const int w = warp + NK_WARPS * lane + j * NK_THREADS;
-        const uint4 r = w < W ? __ldcg(reinterpret_cast<const uint4 *>(p.wmin + w)) : make_uint4(~0u, ~0u >> 1, NK_NONE, 0u);
-        wd[j] = r.z;
-        wi[j] = (int64_t)(((uint64_t)r.y << 32) | r.x);
-    }
+    for (int j = 0; j < NW; ++j) nk_warp_min(p, warp + NK_WARPS * lane + j * NK_THREADS, wd[j], wi[j]);
 #pragma unroll
     for (int j = 0; j < NW; ++j)
         if (pless(wd[j], wi[j], d, i)) d = wd[j], i = wi[j];
@@ -245,6 +320,7 @@ __device__ __noinline__ void nearest_select(const NearestArgs &p, NearestShared 
         if (wd[j] < NK_NONE && !pless(s.bd, s.bi, wd[j], wi[j]))
             s.warps[atomicAdd(&s.nwarps, 1)] = (uint16_t)(warp + NK_WARPS * lane + j * NK_THREADS);
     __syncthreads();
+    if (s.nwarps > NK_LOOSE) nk_tighten_warps(p, s);  // the same for all threads; so many warps with a point are at least k
     const int nwarps = s.nwarps;
     const int64_t rounds = npairs > 0 ? (npairs + rstep - 1) / rstep : 1;
     const int64_t nvec = rounds * NK_U, chunks = (nvec + 31) / 32;  // a thread's vectors, 32 to a pass of a warp
@@ -254,9 +330,14 @@ __device__ __noinline__ void nearest_select(const NearestArgs &p, NearestShared 
         for (int b = b0 + warp; b < nwarps && b < b0 + NK_BATCH; b += NK_WARPS) {
             const uint32_t u = (uint32_t)s.warps[b] * 32u + lane;
             const uint32_t du = __ldcg(p.tmin + u);
-            if (du < NK_NONE && du <= s.bd) s.units[atomicAdd(&s.nunits, 1)] = u;
+            if (du < NK_NONE && du <= s.bd) {
+                const int at = atomicAdd(&s.nunits, 1);
+                s.units[at] = u;
+                s.ud[at] = du;
+            }
         }
         __syncthreads();
+        if (s.nunits > p.k && s.nunits * chunks > NK_PASSES * NK_WARPS) nk_tighten_units(p, s);
         const int64_t tasks = s.nunits * chunks;
         for (int64_t t0 = 0; t0 < tasks; t0 += NK_WARPS) {
             const int n = s.ncand;
