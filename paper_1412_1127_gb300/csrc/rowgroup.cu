@@ -45,7 +45,9 @@ __global__ void __launch_bounds__(WB) rowgroup_kernel(const __grid_constant__ Ro
         const int64_t r = rb + lane / L;
         const bool live = r < p.rows;
         Acc A[NC];
-        group_fold<T, NC, W0, W1, GV>((const T *)p.A + (live ? r : rb) * p.ld, cols, live, l, L, rounds, p.cl, p.neutral, w, A);
+        // rows past GROUP_BYTES / 2 (the launch picks GV so) have a vector in every lane
+        group_fold<T, NC, W0, W1, GV, (GV > GROUP_GV / 2)>((const T *)p.A + (live ? r : rb) * p.ld, cols, live, l, L, rounds,
+                                                           p.cl, p.neutral, w, A);
 #pragma unroll
         for (int c = 0; c < NC; ++c)
             if (live && l == 0 && ACCR_DCHECK(r < p.rows, DS_ROW_VAR))
