@@ -216,7 +216,7 @@ __device__ __forceinline__ void batch_body(const BatchArgs &p, const RegionDev *
     __shared__ Acc sh[RD_CLAUSES][BB / 32];
     __shared__ int s_last;
     __shared__ long long s_q;
-    grid_dependency();
+    grid_wait();
     // tiles of long regions, one CTA per tile, taken from a queue (largest
     // first within each element-type group); the next index is fetched while
     // the current tile is folded
@@ -252,6 +252,7 @@ __device__ __forceinline__ void batch_body(const BatchArgs &p, const RegionDev *
         }
         s = __shfl_sync(0xffffffffu, nx, 0);
     }
+    grid_release();  // a warp of the CTA found the queues empty
     // the last CTA to finish returns the queues to zero for the next launch
     __syncthreads();
     if (threadIdx.x == 0) {

@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     // taken after the wait: the allocation waits without a limit, and with a reused split
     // the predecessor may be anybody's kernel, which could need the tensor memory that
     // this CTA would hold while it waits.
-    grid_dependency();
+    grid_wait();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&bars->tmem)),
                      "r"(TMEM_COLS)
@@ -219,6 +219,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                 issued[s] = use;
             }
         }
+        grid_release();  // the last tile's slices are on their way
         // let every copy this thread issued land before the CTA can exit
         for (int s = 0; s < TSTAGES; ++s)
             if (issued[s] >= 0 && !mbar_wait(smem_u32(&bars->full[s]), (uint32_t)(issued[s] & 1))) atomicExch(err, call | 2);
@@ -382,7 +383,8 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 3) split_kernel(const float *a,
                                                               __nv_bfloat16 *bp, int nblk_a, int tiles_n) {
     __shared__ float tile[64][65];
     const int64_t row_stride = 2 * Kp;
-    grid_dependency();  // once every block has started, the GEMM may be set up behind this grid
+    grid_wait();
+    grid_release();  // once every block has started (each is short), the GEMM may be set up behind this grid
     if ((int)blockIdx.x < nblk_a) {
         const int64_t k8 = Kp / 8, total = len * k8;
         const int64_t t0 = (int64_t)blockIdx.x * (SPLIT_THREADS * SPLIT_A_ITEMS) + threadIdx.x;

@@ -387,7 +387,7 @@ __device__ __noinline__ void nearest_select(const NearestArgs &p, NearestShared 
 __global__ void __launch_bounds__(NK_THREADS, 2) nearest_kernel(const __grid_constant__ NearestArgs p) {
     __shared__ NearestShared s;
     __shared__ int am_last;
-    grid_dependency();
+    grid_wait();
     const int t = threadIdx.x, lane = t & 31;
     // points are float2; the vector part starts at a 16-byte boundary
     const int64_t head = (((uintptr_t)p.pts & 15) != 0 && p.n > 0) ? 1 : 0;
@@ -456,6 +456,7 @@ __global__ void __launch_bounds__(NK_THREADS, 2) nearest_kernel(const __grid_con
         const uint32_t d = sqdist(p.pts[2 * last], p.pts[2 * last + 1], p.qx, p.qy);
         if (d < bd) bd = d, bi = last;
     }
+    grid_release();  // the points are read: minima, and the last CTA's select, are left
     const int gt = (int)blockIdx.x * NK_THREADS + t;
     p.tmin[gt] = bd;
     warp_min_pair(bd, bi);
@@ -761,7 +762,7 @@ template <bool AL>
 __global__ void __launch_bounds__(SF_THREADS, 1) standardize_fused_kernel(const __grid_constant__ StdArgs p) {
     __shared__ StatPartial sh[SF_THREADS / 32];
     __shared__ float s_mean, s_rstd;
-    grid_dependency();
+    grid_wait();  // (one CTA is launched overlapped)
     const int t = threadIdx.x, G = gridDim.x;
     unsigned gen = (*(volatile unsigned *)&p.bar[1]) >> 1;
     const int64_t nq = p.n / 4, per = (nq + G - 1) / G;
@@ -802,6 +803,7 @@ __global__ void __launch_bounds__(SF_THREADS, 1) standardize_fused_kernel(const 
         if (t == 0) atomicExch(p.err, p.gen);
         return;
     }
+    grid_release();
     const StdShared st = merge_stats<SF_THREADS>(p.partials, G, p.n);
     if (t == 0) {
         s_mean = st.mean_f;
@@ -906,12 +908,13 @@ __global__ void __launch_bounds__(BF_THREADS) bfs_level_kernel(const uint8_t *op
                                                                int64_t rows, int64_t cols, int32_t L, int mode,
                                                                unsigned *more, const unsigned *before, unsigned *next,
                                                                unsigned *partial, unsigned *counter) {
-    grid_dependency();
+    grid_wait();
     if (before && *(const volatile unsigned *)before == 0u) {
         if (blockIdx.x == 0 && threadIdx.x == 0) *more = 0u;
         return;
     }
     const bool changed = bfs_level(open, dist, rows, cols, L);
+    grid_release();
     if (mode == 1) {
         if (blockIdx.x == 0 && threadIdx.x == 0) *next = 0u;  // for the level that follows this launch
         if (changed) *more = 1u;

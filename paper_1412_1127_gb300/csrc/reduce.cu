@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(RB, 2) reduce_kernel(const __grid_constant__ R
     constexpr int EPV = 16 / (int)sizeof(T);
     __shared__ Acc sh[NC][RB / 32];
     __shared__ int am_last;
-    grid_dependency();
+    grid_wait();
 
     const T *in = (const T *)p.in;
     const int64_t n = p.n;
@@ -98,6 +98,7 @@ __global__ void __launch_bounds__(RB, 2) reduce_kernel(const __grid_constant__ R
     const int64_t step = (int64_t)gridDim.x * (RB * RU);
     for (int64_t base = (int64_t)blockIdx.x * (RB * RU); p.spread || base < nvec; base += step) {
         const bool full = !p.spread && base + RB * RU <= nvec;  // the same for the CTA
+        if (base >= nvec - RELEASE_BYTES / 16) grid_release();
         uint4 b[RU];
         int cnt = RU;
         if (full) {

@@ -30,7 +30,7 @@ template <typename T, int NC, int W0, int W1, int GV>
 __global__ void __launch_bounds__(WB) rowgroup_kernel(const __grid_constant__ RowArgs p) {
     constexpr bool E64 = sizeof(T) == 8;
     constexpr int EPV = 16 / (int)sizeof(T);
-    grid_dependency();
+    grid_wait();
     const int lane = threadIdx.x & 31, L = p.lanes;
     const int l = lane & (L - 1);
     const int rpw = 32 / L;  // rows per warp
@@ -41,6 +41,9 @@ __global__ void __launch_bounds__(WB) rowgroup_kernel(const __grid_constant__ Ro
     for (int c = 0; c < NC; ++c) w[c] = (c == 0 && W0 >= 0) ? W0 : (c == 1 && W1 >= 0) ? W1 : p.cl[c].wcode;
     const int64_t step = (int64_t)gridDim.x * (WB / 32) * rpw;
     const int64_t first = ((int64_t)blockIdx.x * (WB / 32) + (threadIdx.x >> 5)) * rpw;
+    // (released inside the loop, 400,000 rows of 61 took 22.1 us instead of 19.7; a longer
+    // call's end releases)
+    if (p.release_row <= 0) grid_release();
     for (int64_t rb = first; rb < p.rows; rb += step) {  // uniform across the warp
         const int64_t r = rb + lane / L;
         const bool live = r < p.rows;

@@ -87,7 +87,7 @@ template <typename T, int NC, int W0 = -1, int W1 = -1, int FORM = ROW_SEG>
 __global__ void __launch_bounds__(row_threads<T, NC, FORM>()) rowreduce_kernel(const __grid_constant__ RowArgs p) {
     constexpr bool E64 = sizeof(T) == 8, FIXED = W0 >= 0;
     constexpr int NTH = row_threads<T, NC, FORM>(), NW = NTH / 32;
-    grid_dependency();
+    grid_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t gw = (int64_t)blockIdx.x * NW + warp;
     const int64_t cols = p.cols;
@@ -107,6 +107,7 @@ __global__ void __launch_bounds__(row_threads<T, NC, FORM>()) rowreduce_kernel(c
         for (int c = 0; c < NC; ++c) fw[c] = final_code(w[c]);
         const int64_t step = FORM == ROW_SEG ? (int64_t)gridDim.x * NW : (int64_t)gridDim.x;
         for (int64_t r = FORM == ROW_SEG ? gw : (int64_t)blockIdx.x; r < p.rows; r += step) {
+            if (r >= p.release_row) grid_release();
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
                 P[c].a = final_ident(p.cl[c]);
@@ -151,6 +152,7 @@ __global__ void __launch_bounds__(row_threads<T, NC, FORM>()) rowreduce_kernel(c
     const int64_t total = p.rows * p.cpr;
     const int64_t c0 = total * (int64_t)blockIdx.x / gridDim.x, c1 = total * ((int64_t)blockIdx.x + 1) / gridDim.x;
     for (int64_t k = c0 + warp; k < c1; k += NW) {
+        if ((c1 - k) * gridDim.x <= RELEASE_BYTES / SPLIT_CHUNK_BYTES) grid_release();
         const int64_t r = k / p.cpr, j = k - r * p.cpr, lo = j * p.chunk;
         const int64_t len = (cols - lo) < p.chunk ? (cols - lo) : p.chunk;
         if (!ACCR_DCHECK(r < p.rows && lo + len <= cols, DS_ROW_CHUNK)) continue;
@@ -334,6 +336,7 @@ extern "C" ACCR_API int accr_rowreduce(const void *A, int64_t rows, int64_t cols
     a.cols = cols;
     a.ld = ld;
     a.nc = nclauses;
+    a.release_row = rows - RELEASE_BYTES / (row_bytes > 0 ? row_bytes : 1);
     for (int c = 0; c < nclauses; ++c) a.cl[c] = cl[c];
     rc = a.lanes > 0 ? rowgroup_launch(a, in_type, s) : row_dispatch(a, in_type, RowLaunch{form}, s);
     if (rc != ACCR_OK) return rc;

@@ -18,6 +18,7 @@ struct RowArgs {
     int nc;
     ClauseDev cl[ACCR_MAX_CLAUSES];
     uint64_t neutral[ACCR_MAX_CLAUSES];  // group form: an element that leaves the clause's fold as it is
+    int64_t release_row;  // from this row on a warp (or CTA) lets the next kernel be set up
     int lanes;            // group form: lanes per row
     int64_t chunk;        // split form: elements per chunk; segment form: per segment
     int64_t cpr;          // split form: chunks per row; segment form: segments per row

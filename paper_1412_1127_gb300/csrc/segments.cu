@@ -53,7 +53,7 @@ template <typename T, int NC, int W0, int W1>
 __global__ void __launch_bounds__(SB) segment_kernel(const __grid_constant__ SegArgs p) {
     constexpr bool E64 = sizeof(T) == 8;
     constexpr int EPV = 16 / (int)sizeof(T);
-    grid_dependency();
+    grid_wait();
     const int lane = threadIdx.x & 31;
     int w[NC];
 #pragma unroll
@@ -114,6 +114,7 @@ __global__ void __launch_bounds__(SB) segment_kernel(const __grid_constant__ Seg
         }
         it = __shfl_sync(0xffffffffu, q, 0);
     }
+    grid_release();  // a warp of the CTA found the queue empty
     // the last CTA returns the queue to zero for the next launch
     __syncthreads();
     if (threadIdx.x == 0) {

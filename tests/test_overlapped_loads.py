@@ -49,4 +49,4 @@ def test_tensor_memory_is_taken_behind_the_wait():
     predecessor that may want some."""
     text = re.sub(r"//[^\n]*", "", open(os.path.join(build.CSRC, "matmul_tc.cu")).read())
     body = text[text.index("bf16x3_gemm_kernel("):text.index("split_kernel(")]
-    assert 0 < body.index("grid_dependency()") < body.index("tcgen05.alloc")
+    assert 0 < body.index("grid_wait()") < body.index("tcgen05.alloc")
