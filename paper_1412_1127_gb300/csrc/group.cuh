@@ -4,6 +4,8 @@
 
 #include <math.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "fold.cuh"
 #include "overlap.cuh"
@@ -17,6 +19,8 @@ constexpr int64_t GROUP_BYTES = GROUP_GV * 32 * 16;  // 4 KiB
 // single elements in, an accumulator out.  The primary form keeps the
 // accumulator itself; the float sums and extremes keep their own chains between
 // vectors, which saves the accumulator's packing and the chains' merge per vector.
+// (The generic kernels fold float sums and double ones the same way, so that a sum has
+// the same bits alone and beside any other clause.)
 template <typename T, int W>
 struct GroupFold {
     Acc A;
@@ -64,9 +68,10 @@ struct GroupFold<float, W_MAXF> : GroupExtreme<true> {};
 template <>
 struct GroupFold<float, W_MINF> : GroupExtreme<false> {};
 
-// Folds the loaded vectors of one lane.  A pair kernel folds the vectors the
-// lane holds one by one; a generic one fills the others with the clause's
-// neutral element, so that its operator switch runs once for all of them.
+// Folds the loaded vectors of one lane, the missing ones filled with the clause's
+// neutral element, so that an operator switch runs once for all of them: GV, or half
+// where no lane has more (`rounds`).  Double sums round once a chunk of at least four
+// vectors (chunk_sum_f64), fewer go one by one.
 template <typename T, int NV, int GV>
 __device__ __forceinline__ void fold_filled(int w, Acc &A, const uint4 (&b)[GV], const bool (&ok)[GV], uint64_t neutral) {
     const uint32_t lo = (uint32_t)neutral, hi = sizeof(T) == 8 ? (uint32_t)(neutral >> 32) : lo;
@@ -74,6 +79,19 @@ __device__ __forceinline__ void fold_filled(int w, Acc &A, const uint4 (&b)[GV],
 #pragma unroll
     for (int u = 0; u < NV; ++u) f[u] = ok[u] ? b[u] : make_uint4(lo, hi, lo, hi);
     fold_vec<T, NV>(w, A, f);
+}
+template <typename T, int GV>
+__device__ __forceinline__ void fold_lane(int w, Acc &A, const uint4 (&b)[GV], const bool (&ok)[GV], int rounds,
+                                          uint64_t neutral) {
+    if (rounds > GV / 2) {
+        fold_filled<T, GV, GV>(w, A, b, ok, neutral);
+    } else if (std::is_same<T, double>::value && GV / 2 < 4 && w == W_ADDF) {
+#pragma unroll
+        for (int u = 0; u < GV / 2; ++u)
+            if (ok[u]) fold_vec<T, 1>(W_ADDF, A, &b[u]);
+    } else if (rounds > 0) {
+        fold_filled<T, GV / 2, GV>(w, A, b, ok, neutral);
+    }
 }
 
 // One stretch of `len` elements at `in`, folded by a group of L lanes (this lane is
@@ -108,35 +126,51 @@ __device__ __forceinline__ void group_fold(const T *in, int len, bool live, int 
     }
     if (l < head) h = in[l];
     if (tail0 + l < end) t = in[tail0 + l];
+    // this lane's head and tail elements, in one order for every kernel
+    auto ends = [&](auto &&one) {
+        if (l < head) one(h);
+        if (tail0 + l < end) one(t);
+        if (L < EPV) {  // fewer lanes than a head or tail may have elements
+            for (int j = L + l; j < head; j += L) one(in[j]);
+            for (int j = tail0 + L + l; j < end; j += L) one(in[j]);
+        }
+    };
     if constexpr (PAIR) {
+        constexpr bool CHUNK = E64 && W0 == W_ADDF;
         GroupFold<T, W0> F0;
         GroupFold<T, W1> F1;
         F0.init(cl[0].ident);
         F1.init(cl[1].ident);
+        if constexpr (CHUNK) fold_lane<T, GV>(W0, F0.A, b, ok, rounds, neutral[0]);
 #pragma unroll
         for (int u = 0; u < GV; ++u) {
             if (ok[u]) {
-                F0.vec(b[u]);
+                if constexpr (!CHUNK) F0.vec(b[u]);
                 F1.vec(b[u]);
             }
         }
-        if (l < head) F0.one(h), F1.one(h);
-        if (tail0 + l < end) F0.one(t), F1.one(t);
-        if (L < EPV) {  // fewer lanes than a head or tail may have elements
-            for (int j = L + l; j < head; j += L) F0.one(in[j]), F1.one(in[j]);
-            for (int j = tail0 + L + l; j < end; j += L) F0.one(in[j]), F1.one(in[j]);
-        }
+        ends([&](T x) { F0.one(x), F1.one(x); });
         A[0] = F0.get();
         A[1] = F1.get();
     } else {
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
+            if constexpr (std::is_same<T, float>::value) {
+                if (w[c] == W_ADDF) {
+                    GroupFold<float, W_ADDF> F;
+                    F.init(cl[c].ident);
+#pragma unroll
+                    for (int u = 0; u < GV; ++u)
+                        if (ok[u]) F.vec(b[u]);
+                    ends([&](T x) { F.one(x); });
+                    A[c] = F.get();
+                    continue;
+                }
+            }
             A[c].a = cl[c].ident;
             A[c].c = 0.f;
-            if (rounds > GV / 2) fold_filled<T, GV, GV>(w[c], A[c], b, ok, neutral[c]);
-            else if (rounds > 0) fold_filled<T, GV / 2, GV>(w[c], A[c], b, ok, neutral[c]);
-            for (int j = l; j < head; j += L) fold_one<T>(w[c], A[c], j == l ? h : in[j]);
-            for (int j = tail0 + l; j < end; j += L) fold_one<T>(w[c], A[c], j == tail0 + l ? t : in[j]);
+            fold_lane<T, GV>(w[c], A[c], b, ok, rounds, neutral[c]);
+            ends([&](T x) { fold_one<T>(w[c], A[c], x); });
         }
     }
 #pragma unroll
