@@ -242,8 +242,8 @@ ACCR_API int accr_batch_reduce(const accr_region *regions, int64_t nregions,
  * prior value of every segment's variable.  The offsets are checked on the host
  * and uploaded; one launch folds segments of at most 4 KiB in groups of lanes
  * and longer ones, up to the warp-region limit of accr_batch_tiling, a warp
- * each; longer ones still run as tiles of a batched launch.  A segment's form
- * depends on its own type and length only.
+ * each; longer ones are cut into the batch's tiles, which CTAs of the same launch
+ * fold first.  A segment's form depends on its own type and length only.
  *
  *   values    DEVICE array of in_type
  *   offsets   HOST array of nseg+1 non-decreasing element offsets (loop bounds

@@ -293,6 +293,7 @@ static std::atomic<int64_t> g_tile_bytes{ACCR_TILE_BYTES};
 // What one warp or CTA folds stays below 64 GiB (stream_fold counts vectors in 32 bits).
 constexpr int64_t MAX_STRETCH_BYTES = (int64_t)1 << 35;
 int64_t batch_small_bytes() { return std::min(g_small_bytes.load(), MAX_STRETCH_BYTES); }
+int64_t batch_tile_bytes() { return std::min(g_tile_bytes.load(), MAX_STRETCH_BYTES); }
 
 struct HostPlan {
     std::vector<RegionDev> regions;
@@ -531,28 +532,6 @@ struct RegionSource {
     }
 };
 
-// Listed segments [off[s], off[s+1]) of one array, one variable per segment (the
-// offsets were checked by the caller).
-struct SegmentSource {
-    const void *values;
-    const int64_t *off;
-    const int32_t *idx;
-    int in_type, nc;
-    int64_t eb;
-    const ClauseDev *base;  // lowered clauses; out = the arrays' starts
-    int ndesc(int64_t) const { return nc > RD_CLAUSES ? 2 : 1; }
-    int fill(int64_t i, RegionDev *out, ClauseMemo &) const {
-        const int64_t s = idx[i], lo = off[s], hi = off[s + 1];
-        ClauseDev cl[ACCR_MAX_CLAUSES];
-        for (int c = 0; c < nc; ++c) {
-            cl[c] = base[c];
-            cl[c].out = (char *)base[c].out + s * type_bytes(base[c].acc_type);
-        }
-        RegionSource::put(out, (const char *)values + lo * eb, hi - lo, in_type, cl, nc);
-        return ACCR_OK;
-    }
-};
-
 // Builds the plan of n source items: each descriptor goes to the warp list
 // or to tiles by its own type and length, and both queues are ordered by key
 // (a counting sort).  Large plans run in chunks on the planner threads; the
@@ -561,7 +540,7 @@ struct SegmentSource {
 template <typename Src>
 static int plan_chunked(const Src &src, int64_t n, HostPlan &P) {
     const int64_t small_b = batch_small_bytes();
-    const int64_t tile_b = std::min(P.tile_override > 0 ? P.tile_override : g_tile_bytes.load(), MAX_STRETCH_BYTES);
+    const int64_t tile_b = std::min(P.tile_override > 0 ? P.tile_override : batch_tile_bytes(), MAX_STRETCH_BYTES);
     P.tile_bytes = tile_b;
     const int nch = n >= PAR_MIN_REGIONS ? 2 * plan_pool().threads() : 1;
     std::vector<PlanChunk> ch((size_t)nch);
@@ -873,15 +852,6 @@ int batch_launch_regions(const accr_region *regions, int64_t nregions, accr_stre
     return run_once(P, 0, stream);
 }
 
-int batch_launch_segments(const void *values, const int64_t *off, const int32_t *idx, int64_t n, int in_type,
-                          const ClauseDev *cl, int nc, accr_stream_t stream) {
-    HostPlan &P = thread_plan(0);
-    SegmentSource src{values, off, idx, in_type, nc, (int64_t)type_bytes(in_type), cl};
-    int rc = plan_chunked(src, n, P);
-    if (rc != ACCR_OK) return rc;
-    return run_once(P, 0, stream);
-}
-
 int PlanStage::begin(accr_stream_t stream, size_t bytes) {
     bufs = bufs_for(stream);
     bufs->mu.lock();
@@ -891,6 +861,13 @@ int PlanStage::begin(accr_stream_t stream, size_t bytes) {
     host = bufs->stage[slot];
     dev = bufs->dev;
     return ACCR_OK;
+}
+
+int PlanStage::reserve(size_t bytes, size_t words, cudaStream_t s) {
+    const int rc = grow(bufs, bytes, words + 4, s);  // (words 0-3 are the batch's queues)
+    dev = bufs->dev;
+    counters = rc == ACCR_OK ? bufs->counters + 4 : nullptr;
+    return rc;
 }
 
 int PlanStage::upload(size_t bytes, cudaStream_t s) { return send_stage(bufs, slot, bytes, s); }

@@ -12,15 +12,10 @@ namespace accr {
 // depends only on its own type and length.
 int batch_launch_regions(const accr_region *regions, int64_t nregions, accr_stream_t stream, int64_t tile_bytes = 0);
 
-// The same for the listed segments values[off[s] .. off[s + 1]), s = idx[0 .. n),
-// whose offsets the caller has checked; `cl`: lowered clauses, whose outputs are
-// the starts of the variables' arrays.
-struct ClauseDev;
-int batch_launch_segments(const void *values, const int64_t *off, const int32_t *idx, int64_t n, int in_type,
-                          const ClauseDev *cl, int nc, accr_stream_t stream);
-
 // Bytes up to which one warp folds a region (accr_batch_tiling), below 64 GiB.
 int64_t batch_small_bytes();
+// Bytes of a longer region's tiles, below 64 GiB.
+int64_t batch_tile_bytes();
 
 // A stream's staging for one call's plan: pinned memory to write it into and the
 // device memory it is uploaded to.  Held (the stream's plans are made one at a
@@ -28,7 +23,10 @@ int64_t batch_small_bytes();
 struct StreamBufs;
 struct PlanStage {
     char *host = nullptr, *dev = nullptr;
+    unsigned *counters = nullptr;  // reserve()'s words: zero, and left zero by the kernel
     int begin(accr_stream_t stream, size_t bytes);
+    // More device memory (before upload(); `dev` may change), and counter words.
+    int reserve(size_t bytes, size_t words, cudaStream_t s);
     int upload(size_t bytes, cudaStream_t s);
     void end();
     PlanStage() = default;
