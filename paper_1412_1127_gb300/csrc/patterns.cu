@@ -1197,20 +1197,14 @@ __global__ void __launch_bounds__(BT_THREADS, 1) bfs_tile_kernel(const __grid_co
 
 // ---- host side ---------------------------------------------------------------------
 
-// The tiled form.  Tiles are sized so that there is about one per SM (its
-// interior then small and its halo, and so the levels between two barriers,
-// large); the interior is at most 32 rows and at least 4.
-static int bfs_tiled(const uint8_t *open, int64_t rows, int64_t cols, int64_t src, int32_t *dist, int64_t *levels,
-                     cudaStream_t s) {
+// The grid's tiles.  They are sized so that there is about one per SM (its interior
+// then small and its halo, and so the levels between two barriers, large); the
+// interior is at most 32 rows and at least 4.
+static void bfs_shape(BfsTiles &a, int64_t rows, int64_t cols) {
     const DeviceInfo &di = device_info();
-    BfsTiles a;
-    memset(&a, 0, sizeof a);
-    a.open = open;
-    a.dist = dist;
     a.rows = (int)rows;
     a.cols = (int)cols;
     a.wpr = (int)((cols + 31) / 32);
-    a.src = (src >= 0 && src < rows * cols) ? src : -1;
     a.int_words = a.wpr <= 32 ? 32 : 30;
     a.tiles_c = a.wpr <= 32 ? 1 : (a.wpr + 29) / 30;
     if (rows <= BT_ROWS) {
@@ -1222,6 +1216,26 @@ static int bfs_tiled(const uint8_t *open, int64_t rows, int64_t cols, int64_t sr
         a.depth = std::min((BT_ROWS - a.int_rows) / 2, BT_MAX_DEPTH);
     }
     a.tiles_r = (int)((rows + a.int_rows - 1) / a.int_rows);
+}
+
+// Whether the tiles are the faster form.  A step of `depth` levels takes about 5.4 us
+// for each tile an SM has to go through, however few of a tile's 32 words a row fills;
+// a level of the cell-wise form 2.25 us a million cells, and 4 us at least.  Tall grids of
+// fewer than about 30 columns are the ones to lose by tiles, us a level, tiles / cells:
+// 100,000 x 1 7.4 / 3.3, 100,000 x 8 7.4 / 4.7, 1,000,000 x 1 70 / 4.7, 1,000,000 x 8 70 / 19;
+// but 1,000,000 x 40 70 / 91, 16,384 x 4,096 6.7 / 150.
+static bool bfs_tiles_pay(const BfsTiles &a, int64_t cells, int sms) {
+    if (a.depth == 0) return true;
+    const int64_t rounds = ((int64_t)a.tiles_r * a.tiles_c + sms - 1) / sms;
+    return rounds * 5400 / a.depth <= std::max<int64_t>(4000, cells * 9 / 4000);  // ns a level
+}
+
+static int bfs_tiled(BfsTiles &a, const uint8_t *open, int64_t src, int32_t *dist, int64_t *levels, cudaStream_t s) {
+    const DeviceInfo &di = device_info();
+    const int64_t rows = a.rows, cols = a.cols;
+    a.open = open;
+    a.dist = dist;
+    a.src = (src >= 0 && src < rows * cols) ? src : -1;
     const int64_t ntiles = (int64_t)a.tiles_r * a.tiles_c, nwords = rows * a.wpr;
     a.tile_ctas = (unsigned)std::min<int64_t>(ntiles, di.sms);
     // set-up takes 64 words a CTA and step
@@ -1406,8 +1420,12 @@ extern "C" ACCR_API int accr_grid_bfs(const uint8_t *open, int64_t rows, int64_t
     if (total == 0) return ACCR_OK;
     cudaStream_t s = (cudaStream_t)stream;
     const DeviceInfo &di = device_info();
-    if (mode == ACCR_BFS_PERSISTENT && total <= BT_MAX_CELLS && (int64_t)rows * ((cols + 31) / 32) <= BT_MAX_CELLS / 8)
-        return bfs_tiled(open, rows, cols, src, dist, levels, s);
+    if (mode == ACCR_BFS_PERSISTENT && total <= BT_MAX_CELLS && (int64_t)rows * ((cols + 31) / 32) <= BT_MAX_CELLS / 8) {
+        BfsTiles a;
+        memset(&a, 0, sizeof a);
+        bfs_shape(a, rows, cols);
+        if (bfs_tiles_pay(a, total, di.sms)) return bfs_tiled(a, open, src, dist, levels, s);
+    }
     int rc;
     if ((rc = launch_guard("bfs_init_kernel")) != ACCR_OK) return rc;
     bfs_init_kernel<<<di.sms * 4, 256, 0, s>>>(dist, total, (src >= 0 && src < total) ? src : -1, open);
