@@ -484,7 +484,7 @@ ACCR_API int32_t accr_version(void);
 
 /* Bounds checks of debug builds (a substitute for a memory checker; no
  * counterpart in the paper).  A library built with ACCR_DEBUG
- * (libaccr_debug.so) checks the index of every global store of the row,
+ * (libaccr_debug.so) checks the index of every global store of the row, segment,
  * batched-region, k-nearest and tensor-core kernels against its bound; a
  * failed check does not trap: it counts a violation, records the first
  * failing site and skips the access.  This call (after the work has finished:

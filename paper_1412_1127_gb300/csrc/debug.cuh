@@ -1,7 +1,7 @@
 // debug.cuh -- bounds checks of ACCR_DEBUG builds.
 //
 // A debug build (`build(debug=True)`: libaccr_debug.so, -DACCR_DEBUG) checks
-// the index of every global store of the row, batched-region, k-nearest and
+// the index of every global store of the row, segment, batched-region, k-nearest and
 // tensor-core kernels (and the chunk bounds of the split rows) against the
 // bound the host computed.  A failed check does not trap: it counts the
 // violation in a status word of its translation unit, records the first
@@ -22,9 +22,11 @@ enum DebugSite : unsigned {
     DS_BATCH_TILE = 5,     // batch: tile of a region < the region's tiles
     DS_BATCH_SLOT = 6,     // batch: partial slot < all tiles' slots
     DS_BATCH_REGION = 7,   // batch: region index < descriptors
-    DS_NEAREST_SLOT = 8,   // k-nearest: candidate slot < candidates held
+    DS_NEAREST_SLOT = 8,   // k-nearest: thread's and warp's slots of the scan, listed warps, threads and candidates
     DS_NEAREST_OUT = 9,    // k-nearest: k within the candidates' lists
     DS_GEMM_STORE = 10,    // BF16x3 epilogue: row < M and columns < N
+    DS_SEGMENT_VAR = 11,   // segments: variable index < segments
+    DS_SEGMENT_TILE = 12,  // segments: tile < tiles, its segment within the list, tile within the segment
 };
 
 // Host side (runtime.cu): each translation unit with checks registers a

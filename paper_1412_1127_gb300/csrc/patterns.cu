@@ -178,6 +178,7 @@ struct NearestArgs {
     uint32_t *tmin;     // [threads] each thread's smallest distance
     PairSlot *wmin;     // [warps] each warp's nearest point
     unsigned *counter;  // zero on entry and exit
+    int threads;        // of the scan: slots of tmin, 32 for each of wmin
 };
 
 struct NearestShared {
@@ -332,8 +333,7 @@ __device__ __noinline__ void nearest_select(const NearestArgs &p, NearestShared 
             const uint32_t du = __ldcg(p.tmin + u);
             if (du < NK_NONE && du <= s.bd) {
                 const int at = atomicAdd(&s.nunits, 1);
-                s.units[at] = u;
-                s.ud[at] = du;
+                if (ACCR_DCHECK(at < NK_BATCH * 32, DS_NEAREST_SLOT)) s.units[at] = u, s.ud[at] = du;
             }
         }
         __syncthreads();
@@ -458,14 +458,14 @@ __global__ void __launch_bounds__(NK_THREADS, 2) nearest_kernel(const __grid_con
     }
     grid_release();  // the points are read: minima, and the last CTA's select, are left
     const int gt = (int)blockIdx.x * NK_THREADS + t;
-    p.tmin[gt] = bd;
+    if (ACCR_DCHECK(gt < p.threads, DS_NEAREST_SLOT)) p.tmin[gt] = bd;
     warp_min_pair(bd, bi);
     if (lane == 0) {
         PairSlot w;
         w.i = bi;
         w.d = bd;
         w.pad = 0;
-        p.wmin[gt >> 5] = w;
+        if (ACCR_DCHECK(gt < p.threads, DS_NEAREST_SLOT)) p.wmin[gt >> 5] = w;
     }
     __syncthreads();
     if (t == 0) {
@@ -505,6 +505,7 @@ static int nearest_launch(const float *pts, int64_t n, float qx, float qy, int k
     a.tmin = (uint32_t *)scr->buf;
     a.wmin = (PairSlot *)((char *)scr->buf + tbytes);
     a.counter = scr->counters + 1;
+    a.threads = grid * NK_THREADS;
     int rc = launch_guard("nearest_kernel");
     if (rc != ACCR_OK) return rc;
     launch_overlapped(nearest_kernel, dim3((unsigned)grid), NK_THREADS, 0, s, a);

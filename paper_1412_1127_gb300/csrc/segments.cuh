@@ -51,6 +51,8 @@ __device__ __forceinline__ void segment_tile(const SegArgs &p, int q, const int 
     }
     const int64_t s = p.tiled[i], base = seg_offset(p, s), n = seg_offset(p, s + 1) - base;
     const int t0 = p.tile0[i], nt = p.tile0[i + 1] - t0;
+    // the same for the whole CTA
+    if (!ACCR_DCHECK(i < p.ntiled && q >= t0 && q - t0 < nt && s >= 0 && s < p.nseg, DS_SEGMENT_TILE)) return;
     const int64_t lo = (int64_t)(q - t0) * p.tile_elems, len = n - lo < p.tile_elems ? n - lo : p.tile_elems;
     Acc A[NC];
     uint64_t id[NC];
@@ -76,7 +78,7 @@ __device__ __forceinline__ void segment_tile(const SegArgs &p, int q, const int 
             x.a = A[c].a;
             x.c = A[c].c;
             x.pad = 0;
-            p.partials[(int64_t)q * NC + c] = x;
+            if (ACCR_DCHECK(q >= 0 && q < p.ntiles, DS_SEGMENT_TILE)) p.partials[(int64_t)q * NC + c] = x;
         }
         __threadfence();
         *s_last = atomicAdd(&p.tiles_done[i], 1u) == (unsigned)(nt - 1);
@@ -120,6 +122,7 @@ __global__ void __launch_bounds__(SB, TILES ? 2 : 0) segment_kernel(const __grid
     for (int c = 0; c < NC; ++c) w[c] = (c == 0 && W0 >= 0) ? W0 : (c == 1 && W1 >= 0) ? W1 : p.cl[c].wcode;
     Acc A[NC];
     auto store = [&](int64_t s, bool empty) {
+        if (!ACCR_DCHECK(s >= 0 && s < p.nseg, DS_SEGMENT_VAR)) return;
 #pragma unroll
         for (int c = 0; c < NC; ++c) store_var(p.cl[c], s, finish(p.cl[c], E64, empty, to_final(w[c], A[c])));
     };
