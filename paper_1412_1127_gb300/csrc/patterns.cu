@@ -907,7 +907,7 @@ constexpr int BFS_GROUP = 8;
 
 __global__ void __launch_bounds__(BF_THREADS) bfs_level_kernel(const uint8_t *open, int32_t *dist,
                                                                int64_t rows, int64_t cols, int32_t L, int mode,
-                                                               unsigned *more, const unsigned *before, unsigned *next,
+                                                               unsigned *more, const unsigned *before,
                                                                unsigned *partial, unsigned *counter) {
     grid_wait();
     if (before && *(const volatile unsigned *)before == 0u) {
@@ -917,7 +917,6 @@ __global__ void __launch_bounds__(BF_THREADS) bfs_level_kernel(const uint8_t *op
     const bool changed = bfs_level(open, dist, rows, cols, L);
     grid_release();
     if (mode == 1) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) *next = 0u;  // for the level that follows this launch
         if (changed) *more = 1u;
         return;
     }
@@ -1449,7 +1448,7 @@ extern "C" ACCR_API int accr_grid_bfs(const uint8_t *open, int64_t rows, int64_t
     const int grid = (int)std::min<int64_t>(want, (int64_t)per_sm * di.sms);
     Scratch *scr = scratch_for(stream, sizeof(unsigned) * (size_t)grid + 512);
     if (!scr) return ACCR_ENOMEM;
-    unsigned *flags = scr->counters + 32;    // 2 x BFS_GROUP words, the groups alternate
+    unsigned *more = scr->counters + 32;     // BFS_GROUP words
     unsigned *counter = scr->counters + 9;
     unsigned *bar = scr->counters + 12;      // arrivals, generation
     int *err = (int *)(scr->counters + 14);
@@ -1482,20 +1481,18 @@ extern "C" ACCR_API int accr_grid_bfs(const uint8_t *open, int64_t rows, int64_t
         return ACCR_OK;
     }
     // host-driven levels: one launch per level, the flags of a group read back together
-    // (guarded writes need a cleared flag: each level clears the next one's, as a memset
-    // before every group cost 2.4 us a level: 23.9 -> 21.5 at 1024 x 1024)
-    if (mode == ACCR_BFS_GUARDED) {
-        rc = cuda_check(cudaMemsetAsync(flags, 0, sizeof(unsigned), s), "accr_grid_bfs: clear flags");
-        if (rc != ACCR_OK) return rc;
-    }
+    // (guarded writes need cleared flags; each level clearing the next one's instead of a
+    // memset a group took the same 23.4 us a level at 1024 x 1024, 4.2 at 145 x 190)
     for (int64_t L0 = 0; L0 <= total; L0 += BFS_GROUP) {
-        const int g = (int)(L0 / BFS_GROUP & 1);
-        unsigned *more = flags + g * BFS_GROUP, *other = flags + (g ^ 1) * BFS_GROUP;
+        if (mode == ACCR_BFS_GUARDED) {
+            rc = cuda_check(cudaMemsetAsync(more, 0, BFS_GROUP * sizeof(unsigned), s), "accr_grid_bfs: clear flags");
+            if (rc != ACCR_OK) return rc;
+        }
         for (int i = 0; i < BFS_GROUP; ++i) {
             if ((rc = launch_guard("bfs_level_kernel")) != ACCR_OK) return rc;
             launch_overlapped(bfs_level_kernel, dim3((unsigned)grid), BF_THREADS, 0, s, open, dist, rows, cols,
                               (int32_t)(L0 + i), mode == ACCR_BFS_GUARDED ? 1 : 0, more + i, i > 0 ? more + i - 1 : nullptr,
-                              i + 1 < BFS_GROUP ? more + i + 1 : other, partial, counter);
+                              partial, counter);
             if ((rc = launched("bfs_level_kernel")) != ACCR_OK) return rc;
         }
         rc = cuda_check(cudaMemcpyAsync(hmore, more, BFS_GROUP * sizeof(unsigned), cudaMemcpyDeviceToHost, s),
