@@ -5,6 +5,7 @@ raises, so no result can silently come from anywhere but the CUDA kernels.
 """
 import ctypes
 import os
+import sys
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 # The library: the in-tree release build, or another build of it named by
@@ -55,12 +56,47 @@ class Result(ctypes.Structure):
 # Every symbol include/accr.h declares, with its ctypes signature.
 _vp, _i32, _i64, _u32, _u64 = (ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64,
                                ctypes.c_uint32, ctypes.c_uint64)
-_CP = _vp  # accr_clause array: packed bytes (the binding's) or a ctypes array of Clause
+
+
+class _ClauseArray:
+    """Argument type of an ``accr_clause`` array: a ctypes array of or pointer to Clause,
+    or the binding's packed bytes of one or more whole clauses; anything else is refused."""
+    _pointer = ctypes.POINTER(Clause)
+    _size = ctypes.sizeof(Clause)
+
+    @classmethod
+    def from_param(cls, v):
+        if type(v) is bytes:
+            if v and len(v) % cls._size == 0:
+                return v
+            raise TypeError("%d bytes are no array of clauses" % len(v))
+        return cls._pointer.from_param(v)
+
+
+_INT64 = "<i8" if sys.byteorder == "little" else ">i8"
+
+
+class _OffsetArray:
+    """Argument type of an int64 array: a contiguous numpy array of that type, or a ctypes
+    array of or pointer to int64; anything else is refused."""
+    _pointer = ctypes.POINTER(_i64)
+
+    @classmethod
+    def from_param(cls, v):
+        a = getattr(v, "__array_interface__", None)
+        if a is None:
+            return cls._pointer.from_param(v)
+        if a["typestr"] != _INT64 or not v.flags.c_contiguous:
+            raise TypeError("offsets are a contiguous int64 array")
+        return _vp(a["data"][0])
+
+
+_CP = _ClauseArray
 SIGNATURES = {
     "accr_reduce": (ctypes.c_int, [_vp, _i64, _i32, _CP, _i32, _u32, _vp]),
     "accr_rowreduce": (ctypes.c_int, [_vp, _i64, _i64, _i64, _i32, _CP, _i32, _u32, _vp]),
     "accr_batch_reduce": (ctypes.c_int, [ctypes.POINTER(Region), _i64, _u32, _vp]),
-    "accr_segmented_reduce": (ctypes.c_int, [_vp, _vp, _i64, _i32, _CP, _i32, _u32, _vp]),
+    "accr_segmented_reduce": (ctypes.c_int, [_vp, _OffsetArray, _i64, _i32, _CP, _i32, _u32, _vp]),
     "accr_batch_create": (ctypes.c_int, [ctypes.POINTER(Region), _i64, _u32, ctypes.POINTER(_vp)]),
     "accr_batch_launch": (ctypes.c_int, [_vp, _vp]),
     "accr_batch_destroy": (ctypes.c_int, [_vp]),

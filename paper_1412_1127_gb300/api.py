@@ -209,7 +209,7 @@ def accr_segmented_reduce(values, offsets, clauses, flags=0, stream=None):
     arr, keep = _clauses(clauses)
     return check(lib().accr_segmented_reduce(
         values.data_ptr() if values.numel() else None,
-        off.__array_interface__["data"][0], nseg, type_of(values.dtype), arr,
+        off, nseg, type_of(values.dtype), arr,
         len(clauses), flags, _stream(stream)))
 
 
