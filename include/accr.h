@@ -324,7 +324,8 @@ ACCR_API int accr_standardize(const float *x, int64_t n, float *y,
 #define ACCR_BFS_REDUCE 0     /* levels driven by the host; || reduction of the flag */
 #define ACCR_BFS_GUARDED 1    /* levels driven by the host; flag cleared, threads write only 1 */
 #define ACCR_BFS_PERSISTENT 2 /* all levels in one cooperative launch; grids of at most
-                                 2^28 cells on bitmaps, several levels between barriers */
+                                 2^28 cells, but for tall ones of a few columns, on
+                                 bitmaps, several levels between barriers */
 
 /*
  * accr_grid_bfs -- BFS's convergence loop: level-synchronous search on a
@@ -334,7 +335,10 @@ ACCR_API int accr_standardize(const float *x, int64_t n, float *y,
  * the source is closed).  Synchronous.
  *
  *   open      DEVICE uint8[rows*cols]; dist DEVICE int32[rows*cols]
- *   mode      ACCR_BFS_REDUCE | ACCR_BFS_GUARDED | ACCR_BFS_PERSISTENT
+ *   mode      ACCR_BFS_REDUCE | ACCR_BFS_GUARDED | ACCR_BFS_PERSISTENT (whose bitmaps
+ *             are library scratch, kept per stream: 16 bytes for every 32 cells of a
+ *             row, 134 MB at 2^28 cells; where they cannot be allocated, grids above
+ *             1 MiB of them run cell by cell)
  */
 ACCR_API int accr_grid_bfs(const uint8_t *open, int64_t rows, int64_t cols,
                            int64_t src, int32_t *dist, int32_t mode,

@@ -1230,6 +1230,10 @@ static bool bfs_tiles_pay(const BfsTiles &a, int64_t cells, int sms) {
     return rounds * 5400 / a.depth <= std::max<int64_t>(4000, cells * 9 / 4000);  // ns a level
 }
 
+// One of the four bitmaps.
+static size_t bfs_bitmap_each(const BfsTiles &a) { return ((size_t)a.rows * (size_t)a.wpr * 4 + 255) & ~(size_t)255; }
+static size_t bfs_bitmap_bytes(const BfsTiles &a) { return 4 * bfs_bitmap_each(a); }
+
 static int bfs_tiled(BfsTiles &a, const uint8_t *open, int64_t src, int32_t *dist, int64_t *levels, cudaStream_t s) {
     const DeviceInfo &di = device_info();
     const int64_t rows = a.rows, cols = a.cols;
@@ -1241,8 +1245,8 @@ static int bfs_tiled(BfsTiles &a, const uint8_t *open, int64_t src, int32_t *dis
     // set-up takes 64 words a CTA and step
     const int64_t setup = (nwords + 63) / 64;
     const int grid = (int)std::min<int64_t>(std::max<int64_t>(setup, a.tile_ctas), di.sms);
-    const size_t wbytes = ((size_t)nwords * 4 + 255) & ~(size_t)255;
-    Scratch *scr = scratch_for((accr_stream_t)s, 4 * wbytes);
+    const size_t wbytes = bfs_bitmap_each(a);
+    Scratch *scr = scratch_for((accr_stream_t)s, bfs_bitmap_bytes(a));
     if (!scr) return ACCR_ENOMEM;
     int64_t *res = (int64_t *)host_staging_for((accr_stream_t)s, 64);
     if (!res) return ACCR_ENOMEM;
@@ -1424,7 +1428,12 @@ extern "C" ACCR_API int accr_grid_bfs(const uint8_t *open, int64_t rows, int64_t
         BfsTiles a;
         memset(&a, 0, sizeof a);
         bfs_shape(a, rows, cols);
-        if (bfs_tiles_pay(a, total, di.sms)) return bfs_tiled(a, open, src, dist, levels, s);
+        if (bfs_tiles_pay(a, total, di.sms)) {
+            const int rc = bfs_tiled(a, open, src, dist, levels, s);
+            // no room for large bitmaps: cell by cell, which keeps next to nothing
+            if (rc != ACCR_ENOMEM || bfs_bitmap_bytes(a) <= ((size_t)1 << 20)) return rc;
+            clear_error();
+        }
     }
     int rc;
     if ((rc = launch_guard("bfs_init_kernel")) != ACCR_OK) return rc;
