@@ -89,8 +89,9 @@ typedef enum {
 
 /* Flags. */
 #define ACCR_COMPENSATED 0x1u   /* float + into a float variable: compensated
-                                   (Neumaier) sums per thread, pairwise TwoSum
-                                   combine, double-precision cross-gang merge */
+                                   sums per thread (each addition's error added up
+                                   beside it), pairwise TwoSum combine,
+                                   double-precision cross-gang merge */
 #define ACCR_SYNC 0x2u          /* return only after the result is written */
 #define ACCR_TWO_LEVEL_HOST 0x4u /* the paper's two-level form (SRAD in Sec. 4.2):
                                    block partials on the GPU, copied to the
@@ -421,7 +422,7 @@ ACCR_API int accr_server_replay(accr_server *server, const accr_region *regions,
  * ACCR_NOALLOC_SCRATCH_BYTES (+256) bytes compiled into the library, which
  * every GPU that loads the library holds until the process exits.  A region
  * whose nclauses x blocks x 16 bytes exceeds that size is rejected with
- * ACCR_EINVAL (on a 152-SM GB300 the largest need is about 40 KB).
+ * ACCR_EINVAL (on a 152-SM GB300 the largest need is about 20 KB).
  *
  *   flags     ACCR_COMPENSATED | ACCR_SYNC (ACCR_TWO_LEVEL_HOST needs a pinned
  *             host buffer and is rejected with ACCR_EINVAL)

@@ -6,9 +6,10 @@
 // "working code": the per-element operation in the narrowest exact width.
 // Integer max/min/&/|/^/&&/|| work in the element's width and are widened at
 // the end (sign extension commutes with them); + and * work in the variable's
-// width.  Floating-point max/min work on order-preserving integer keys, which
-// order -0 below +0 and are exact.  Float + may be compensated (Neumaier per
-// thread, TwoSum when merging, double for the cross-gang merge).
+// width.  Floating-point max/min order -0 below +0 and are exact: floats fold on the
+// hardware's max/min, doubles as order-preserving integer keys, and both merge as
+// keys.  Float + may be compensated (each addition's error kept by TwoSum, per thread
+// and when merging; double for the cross-gang merge).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -220,7 +221,7 @@ __device__ __forceinline__ float fmin3(float a, float b, float c) {
 // Knuth's TwoSum: the same exact error as Neumaier's ordered form, in six
 // additions for the FMA pipe instead of three plus a compare and two selects
 // for the half-rate ALU pipe, which is what bounded compensated sums.
-__device__ __forceinline__ void neumaier(float &s, float &c, float x) {
+__device__ __forceinline__ void add_compensated(float &s, float &c, float x) {
     const float t = __fadd_rn(s, x);
     const float xp = __fsub_rn(t, s);
     const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, xp)), __fsub_rn(x, xp));
@@ -442,7 +443,7 @@ __device__ __forceinline__ void fold_vec(int w, Acc &A, const uint4 *v) {
         case W_ADDF_COMP: {
             if constexpr (F32) {
                 float s = u2f((uint32_t)A.a), c = A.c;
-                for_each_elem<T, NV>(v, [&](T x) { neumaier(s, c, x); });
+                for_each_elem<T, NV>(v, [&](T x) { add_compensated(s, c, x); });
                 A.a = f2u(s);
                 A.c = c;
             }
@@ -559,7 +560,7 @@ __device__ __forceinline__ void fold_one(int w, Acc &A, T x) {
         case W_ADDF_COMP:
             if constexpr (F32) {
                 float s = u2f((uint32_t)A.a), c = A.c;
-                neumaier(s, c, (float)x);
+                add_compensated(s, c, (float)x);
                 A.a = f2u(s);
                 A.c = c;
             }

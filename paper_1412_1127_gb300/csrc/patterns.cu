@@ -583,14 +583,12 @@ struct StdArgs {
     unsigned gen;
 };
 
-__device__ __forceinline__ void neumaier2(float &s, float &c, float x) { neumaier(s, c, x); }
-
 // x^2 added exactly: p = fl(x*x) through the compensated sum, and the product's
 // rounding error e = x*x - p (exact by fused multiply-add) into the compensation.
 __device__ __forceinline__ void add_square(float &s, float &c, float x) {
     const float p = __fmul_rn(x, x);
     const float e = __fmaf_rn(x, x, -p);
-    neumaier(s, c, p);
+    add_compensated(s, c, p);
     c = __fadd_rn(c, e);
 }
 
@@ -686,24 +684,24 @@ __global__ void __launch_bounds__(SD_THREADS) standardize_kernel(const __grid_co
         const float4 *x4 = (const float4 *)p.x;
         for (int64_t v = gtid; v < nv; v += nth) {
             const float4 a = __ldg(x4 + v);
-            neumaier2(s1, c1, a.x);
+            add_compensated(s1, c1, a.x);
             add_square(s2, c2, a.x);
-            neumaier2(s1, c1, a.y);
+            add_compensated(s1, c1, a.y);
             add_square(s2, c2, a.y);
-            neumaier2(s1, c1, a.z);
+            add_compensated(s1, c1, a.z);
             add_square(s2, c2, a.z);
-            neumaier2(s1, c1, a.w);
+            add_compensated(s1, c1, a.w);
             add_square(s2, c2, a.w);
         }
         for (int64_t i = 4 * nv + gtid; i < p.n; i += nth) {
             const float a = p.x[i];
-            neumaier2(s1, c1, a);
+            add_compensated(s1, c1, a);
             add_square(s2, c2, a);
         }
     } else {
         for (int64_t i = gtid; i < p.n; i += nth) {
             const float a = p.x[i];
-            neumaier2(s1, c1, a);
+            add_compensated(s1, c1, a);
             add_square(s2, c2, a);
         }
     }
@@ -771,7 +769,7 @@ __global__ void __launch_bounds__(SF_THREADS, 1) standardize_fused_kernel(const 
     const int64_t k0 = max(q0, q1 - (int64_t)SF_KEEP * SF_THREADS);  // the kept part: [k0, q1)
     float s1 = -0.f, c1 = 0.f, s2 = -0.f, c2 = 0.f;
     auto add = [&](float a) {
-        neumaier(s1, c1, a);
+        add_compensated(s1, c1, a);
         add_square(s2, c2, a);
     };
     auto add4 = [&](const float4 &v) { add(v.x), add(v.y), add(v.z), add(v.w); };
