@@ -100,7 +100,7 @@ __device__ __forceinline__ Partial ld_partial_cg(const Partial *p) {
 template <typename T, int NC>
 __device__ __noinline__ void tile_fold(const BatchArgs &p, const RegionDev *d, int r, int64_t k,
                                           Acc (*sh)[BB / 32], int *s_last) {
-    constexpr bool E64 = sizeof(T) == 8;
+    constexpr bool E64 = sizeof(T) == 8, HALF = std::is_same<T, double>::value;
     const int64_t TE = p.tile_bytes / (int64_t)sizeof(T);
     const int64_t n = d->n;
     const int64_t tile0 = d->tile0;
@@ -121,7 +121,7 @@ __device__ __noinline__ void tile_fold(const BatchArgs &p, const RegionDev *d, i
         A[c].a = id[c];
         A[c].c = 0.f;
     }
-    stream_fold<T, NC, BU, BB>(in, len, (int)threadIdx.x, w, A, ld_stream);
+    stream_fold<T, NC, BU, BB, HALF>(in, len, (int)threadIdx.x, w, A, ld_stream);
     cta_merge<NC, BB>(w, id, E64, A, sh);
 
     if (ntiles == 1) {
@@ -178,7 +178,7 @@ __device__ __noinline__ void tile_fold(const BatchArgs &p, const RegionDev *d, i
 // A whole short region folded by one warp.
 template <typename T, int NC>
 __device__ __noinline__ void warp_fold(const RegionDev *d, int lane) {
-    constexpr bool E64 = sizeof(T) == 8;
+    constexpr bool E64 = sizeof(T) == 8, HALF = std::is_same<T, double>::value;
     const int64_t n = d->n;
     const T *in = (const T *)d->in;
     int w[NC];
@@ -189,7 +189,7 @@ __device__ __noinline__ void warp_fold(const RegionDev *d, int lane) {
         A[c].a = d->cl[c].ident;
         A[c].c = 0.f;
     }
-    stream_fold<T, NC, SU, 32>(in, n, lane, w, A, ld_stream);
+    stream_fold<T, NC, SU, 32, HALF>(in, n, lane, w, A, ld_stream);
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
         warp_merge(w[c], E64, A[c]);

@@ -44,7 +44,7 @@ __device__ __forceinline__ void fold_stretch(const T *row, int64_t len, const Cl
         A[c].a = cl[c].ident;
         A[c].c = 0.f;
     }
-    stream_fold<T, NC, RU2, 32>(row, len, lane, w, A, ld_stream);
+    stream_fold<T, NC, RU2, 32, true>(row, len, lane, w, A, ld_stream);
 #pragma unroll
     for (int c = 0; c < NC; ++c) warp_merge<FIXED>(w[c], E64, A[c]);
 }

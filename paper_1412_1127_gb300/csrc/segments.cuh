@@ -62,7 +62,7 @@ __device__ __forceinline__ void segment_tile(const SegArgs &p, int q, const int 
         A[c].a = id[c];
         A[c].c = 0.f;
     }
-    stream_fold<T, NC, RU2, SB>((const T *)p.values + base + lo, len, (int)threadIdx.x, w, A, ld_stream);
+    stream_fold<T, NC, RU2, SB, true>((const T *)p.values + base + lo, len, (int)threadIdx.x, w, A, ld_stream);
     cta_merge<NC, SB>(w, id, E64, A, sh);
     if (nt == 1) {
         if (threadIdx.x == 0) {
