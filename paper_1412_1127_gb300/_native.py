@@ -86,7 +86,7 @@ class _OffsetArray:
         a = getattr(v, "__array_interface__", None)
         if a is None:
             return cls._pointer.from_param(v)
-        if a["typestr"] != _INT64 or not v.flags.c_contiguous:
+        if a["typestr"] != _INT64 or a["strides"] is not None:  # None: C-contiguous
             raise TypeError("offsets are a contiguous int64 array")
         return _vp(a["data"][0])
 

@@ -42,24 +42,23 @@ struct LongSegments {
 
 // Checks the offsets and writes them to dst, relative to off[0] (which is not
 // negative); returns the first segment that ends before it starts, or -1.  Whole
-// blocks are checked by their smallest and largest length and by their offsets'
-// signs (without a negative offset no length overflows); only a block with a
-// longer segment is looked through one by one.
+// blocks are checked by their smallest and largest length; a block that starts or has a
+// length beyond any array, where a length may overflow, by its offsets; and only a
+// block with a longer segment is looked through one by one.
 template <typename O>
 static int64_t copy_offsets(const int64_t *off, int64_t nseg, O *dst, int64_t max_short, int64_t max_mid, LongSegments &L) {
-    constexpr int64_t BLK = 512;
+    constexpr int64_t BLK = 512, FAR = (int64_t)1 << 52;  // FAR + BLK * FAR still fits
     const int64_t base = off[0];
     for (int64_t b = 0; b < nseg; b += BLK) {
         const int64_t e = std::min(nseg, b + BLK);
-        int64_t lo = INT64_MAX, hi = 0, signs = 0;
+        int64_t lo = INT64_MAX, hi = 0;
         for (int64_t s = b; s < e; ++s) {
             const int64_t n = (int64_t)((uint64_t)off[s + 1] - (uint64_t)off[s]);
             lo = n < lo ? n : lo;
             hi = n > hi ? n : hi;
-            signs |= off[s + 1];
             dst[s] = (O)((uint64_t)off[s] - (uint64_t)base);
         }
-        if (lo < 0 || signs < 0) {
+        if (lo < 0 || hi > FAR || off[b] > FAR) {
             for (int64_t s = b; s < e; ++s)
                 if (off[s + 1] < off[s]) return s;
         }

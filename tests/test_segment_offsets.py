@@ -26,7 +26,8 @@ def check(tmp_path_factory):
                 "    LongSegments L;\n"
                 "    const int64_t bad = wide ? copy_offsets(off, nseg, (int64_t *)dst, 1024, 16384, L)\n"
                 "                             : copy_offsets(off, nseg, (uint32_t *)dst, 1024, 16384, L);\n"
-                "    *longer = (int64_t)L.tiled.size();\n    for (auto &v : L.mid) *longer += (int64_t)v.size();\n"
+                "    *longer = 0;\n    for (auto &v : L.mid) *longer += (int64_t)v.size();\n"
+                "    for (auto &v : L.tiled) *longer += (int64_t)v.size();\n"
                 "    return bad;\n}\n")
     subprocess.run(["g++", "-O2", "-std=c++17", "-fwrapv", "-shared", "-fPIC", cpp, "-o", lib], check=True)
     L = ctypes.CDLL(lib)
@@ -62,3 +63,15 @@ def test_offsets_come_out_relative_to_the_first(check, wide):
     bad, dst, longer = check(off, wide)
     assert bad == -1 and np.array_equal(dst.astype(np.int64), off - 3)
     assert longer == int((np.diff(off) > 1024).sum())
+
+
+@pytest.mark.parametrize("far", [1 << 52, (1 << 52) + 1, 1 << 62, I64.max - 4000])
+def test_offsets_beyond_any_array(check, far):
+    """Large offsets that do not decrease pass; a decrease behind them is found."""
+    off = np.arange(1502, dtype=np.int64) + 5
+    off[700:] += far - 2000
+    assert check(off, True)[0] == -1
+    for at in (3, 698, 699, 1400):
+        bad = off.copy()
+        bad[at + 1] = bad[at] - 1
+        assert check(bad, True)[0] == at
