@@ -36,7 +36,7 @@ __device__ __forceinline__ int64_t seg_offset(const SegArgs &p, int64_t i) {
 
 // Tile `q` of the long segments, folded by the whole CTA; the last tile of a segment of
 // several to finish merges their partials in tile order.
-template <typename T, int NC>
+template <typename T, int NC, bool FIXED>
 __device__ __forceinline__ void segment_tile(const SegArgs &p, int q, const int (&w)[NC], Acc (*sh)[SB / 32], int *s_last) {
     constexpr bool E64 = sizeof(T) == 8;
     int i = q;  // its place in the list: every segment one tile, or by search
@@ -63,7 +63,7 @@ __device__ __forceinline__ void segment_tile(const SegArgs &p, int q, const int 
         A[c].c = 0.f;
     }
     stream_fold<T, NC, RU2, SB, true>((const T *)p.values + base + lo, len, (int)threadIdx.x, w, A, ld_stream);
-    cta_merge<NC, SB>(w, id, E64, A, sh);
+    cta_merge<NC, SB, FIXED>(w, id, E64, A, sh);
     if (nt == 1) {
         if (threadIdx.x == 0) {
 #pragma unroll
@@ -103,7 +103,7 @@ __device__ __forceinline__ void segment_tile(const SegArgs &p, int q, const int 
             merge(fw[c], E64, A[c], to_final(w[c], Q));
         }
     }
-    cta_merge<NC, SB>(fw, id, E64, A, sh);
+    cta_merge<NC, SB, FIXED>(fw, id, E64, A, sh);
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int c = 0; c < NC; ++c) store_var(p.cl[c], s, finish(p.cl[c], E64, false, A[c]));
@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(SB, TILES ? 2 : 0) segment_kernel(const __grid
         __syncthreads();
         while (q < p.ntiles) {
             if (threadIdx.x == 0) s_q = (int)atomicAdd(&p.queue[2], 1u);
-            segment_tile<T, NC>(p, q, w, sh, &s_last);
+            segment_tile<T, NC, (W0 >= 0)>(p, q, w, sh, &s_last);
             __syncthreads();
             q = s_q;
             __syncthreads();
@@ -224,6 +224,7 @@ struct SegLaunch {
     }
 };
 
-int segments_launch_tiled(SegArgs &a, int in_type, cudaStream_t s);  // segtiles.cu
+int segments_launch_tiled(SegArgs &a, int in_type, cudaStream_t s);    // segtiles.cu
+int segments_launch_tiled64(SegArgs &a, int in_type, cudaStream_t s);  // segtiles64.cu
 
 }  // namespace accr

@@ -101,3 +101,29 @@ def test_a_batch_in_between():
         assert np.array_equal(s.cpu().numpy(), want)
     for i in range(40):
         assert b[i].item() == int(v[i * 1000:i * 1000 + (3 * te if i % 3 == 0 else 50)].astype(np.int64).sum())
+
+
+def micros(fn, n=30):
+    for _ in range(5):
+        fn()
+    best = float("inf")
+    for _ in range(5):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        for _ in range(n):
+            fn()
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b) * 1e3 / n)
+    return best
+
+
+def test_a_second_clause_costs_little():
+    """A sum and a maximum of segments with some long ones, against the sum alone."""
+    g = np.random.default_rng(5)
+    off = np.concatenate([[0], np.cumsum(np.exp(g.uniform(0, np.log(31853), 1060)).astype(np.int64))])
+    v = torch.randn(int(off[-1]), device="cuda")
+    s, m = torch.zeros(1060, device="cuda"), torch.zeros(1060, device="cuda")
+    one = micros(lambda: api.accr_segmented_reduce(v, off, [api.clause("add", s)]))
+    two = micros(lambda: api.accr_segmented_reduce(v, off, [api.clause("add", s), api.clause("max", m)]))
+    assert two <= 1.25 * one, (two, one)
