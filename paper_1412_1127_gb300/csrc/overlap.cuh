@@ -4,7 +4,7 @@
 // Back-to-back kernels of a stream start about 2 us apart however short they are
 // (an empty grid measured 4.1 us a call, ordinary launches' times come in steps of
 // 2.05 us): draining one grid and setting up the next are serial.  With the next
-// grid's CTAs set up while this one runs, a region of no elements takes 2.2 us
+// grid's CTAs set up while this one runs, a region of no elements takes 2.6 us
 // (4.1 before), 2^16 int32 5.2 (8.2), 2^20 6.2 (8.2), 2^24 8.9 (12.3).
 // Cooperative launches and kernels behind copies keep the ordinary order.
 #pragma once
@@ -29,7 +29,7 @@ __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;
 // so), beside LEN 2048 nests 414 (33, 40-43).  The set-up takes about 2 us; CTAs
 // run apart by some rounds, so streaming kernels release with about RELEASE_BYTES left
 // in the grid, 15 us at HBM's rate (at the last round alone 2^28 floats took 159.0
-// instead of 158.2 us, 400,000 rows of 61 21.4 instead of 19.2).  (No memory clobber:
+// instead of 158.2 us, 400,000 rows of 61 21.4 instead of 19.7).  (No memory clobber:
 // the next grid waits for this one's end whatever stands on either side.)
 constexpr int64_t RELEASE_BYTES = (int64_t)96 << 20;
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;"); }
